@@ -227,9 +227,6 @@ size_t carve(Arena& ar, Workspace& w, const Plan& p, int32_t n, CtlGlobal* ctl, 
     w.rescan_list = ar.take<int32_t>(nb);
     w.sl_edge = ar.take<unsigned long long>(2 * nb);
     w.sl_chunk = ar.take<int32_t>(2 * nb / 32);
-    w.sl_rkey = ar.take<unsigned long long>(2 * nb);
-    w.sl_ru = ar.take<int32_t>(2 * nb);
-    w.sl_rv = ar.take<int32_t>(2 * nb);
     w.ctl_slot = ar.take<int32_t>(2 * nb);
     w.g_row = ar.take<unsigned long long>(nb);
     w.g_col = ar.take<unsigned long long>(nb);
@@ -296,7 +293,6 @@ size_t carve_instance(char* base, int32_t n, bool need_copy, Instance* in) {
     in->ctl = ctl;
     in->seen = seen;
     in->ctl_mode = mode;
-    in->ctl_cap = controller_list_cap(n, mode);
     in->zero_begin = reinterpret_cast<char*>(w.sigma);
     in->zero_bytes = (size_t)(base + bytes - in->zero_begin);
     return bytes;
@@ -854,12 +850,12 @@ dgs_status solve_impl(const int32_t* benefit, int32_t n, int32_t* sigma_out, int
             fprintf(stderr, "[dgs phases] greedy: last group %llu ns, group sum %llu ns, longest chain %llu, "
                             "most scans of a group %llu | controller cycles: entry %llu top %llu conflict check %llu "
                             "post %llu event %llu sweeps %llu | live edges summed over sweeps %llu, listed %llu, "
-                            "accepted in quiet sweeps %llu | colouring passes %llu, cycles %llu (reservation "
-                            "rounds %llu, after them %llu), sweeps run %llu\n",
+                            "accepted in quiet sweeps %llu | colouring passes %llu, cycles %llu (walks "
+                            "%llu, edges coloured %llu), sweeps run %llu\n",
                     ph[kPtDaLastNs], ph[kPtDaSumNs], ph[kPtDaChain], ph[kPtDaGroupScans], ph[kPtCtlEntry],
                     ph[kPtCtlTop], ph[kPtCtlPass1], ph[kPtCtlPost], ph[kPtCtlEvent], ph[kPtCtlSweeps],
                     ph[kPtCtlLiveSum], ph[kPtCtlListSum], ph[kPtCtlAccSum], ph[kPtCtlColourPasses], ph[kPtCtlColour],
-                    ph[kPtCtlColourIters], ph[kPtCtlColourTail], ph[kPtCtlColourRounds]);
+                    ph[kPtCtlColourWalks], ph[kPtCtlColourEdges], ph[kPtCtlColourRounds]);
         }
     }
     if (o.profile) {  // the event timings need the solve to have run

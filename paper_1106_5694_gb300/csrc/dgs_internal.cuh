@@ -94,12 +94,9 @@ struct Workspace {
     int32_t* y_list;                      // jobs changed in the last event
     int32_t* rescan_list;                 // rows to re-evaluate fully
     // per slot (agent slots 0..n-1, job slots n..2n-1): its edge word (0 when
-    // it has no candidate) and its re-evaluated candidate (key, exchange agents)
+    // it has no candidate)
     unsigned long long* sl_edge;
     int32_t* sl_chunk;  // edges among slots 32c .. 32c + 31 (written with sl_edge)
-    unsigned long long* sl_rkey;
-    int32_t* sl_ru;
-    int32_t* sl_rv;
     int32_t* ctl_slot;  // controller: slot of each edge position (priority order)
     // greedy start
     unsigned long long* g_row;  // best free job per agent   (biased value, ~j)
@@ -128,7 +125,6 @@ struct Instance {
     Workspace w;
     CtlGlobal ctl;
     int32_t ctl_mode;          // controller scratch placement for this n
-    int32_t ctl_cap;           // entries of the controller's accepted list in shared memory
     int32_t fresh;             // 1: the next step initialises this instance
     int32_t max_sweeps;        // options of the instance
     int32_t init_mode;         // DGS_INIT_GREEDY / _IDENTITY / _USER (a random start arrives as USER)
@@ -224,7 +220,7 @@ enum : int32_t { kScanPass1 = 0, kScanGreedyDA = 1, kScanStart = 2, kScanSwitch 
 enum : int32_t {
     kPtDaLastNs = 0, kPtDaSumNs, kPtDaChain, kPtDaGroupScans, kPtCtlLiveSum, kPtCtlListSum, kPtCtlAccSum,
     kPtCtlEntry, kPtCtlTop, kPtCtlPass1, kPtCtlPost, kPtCtlEvent, kPtCtlSweeps, kPtCtlColour, kPtCtlColourPasses,
-    kPtCtlColourRounds, kPtCtlColourIters, kPtCtlColourTail, kPtCount
+    kPtCtlColourRounds, kPtCtlColourWalks, kPtCtlColourEdges, kPtCount
 };
 
 // ------------------------------------------------------------- key packing
@@ -357,7 +353,6 @@ cudaError_t launch_keys_to_slots(const Workspace& w, int32_t* ag, int32_t* aj, i
 // condition (1 while the loop state is running) and counts the iteration.
 cudaError_t launch_controller_impl(const Workspace& w, const CtlGlobal& g, cudaStream_t s,
                                    unsigned long long handle = 0);
-int32_t controller_list_cap(int32_t n, int32_t mode);
 // The switching loop in one CTA for small n (see small_loop_kernel), and
 // whether a solve of this workspace takes it.
 bool use_small_loop(const Workspace& w);

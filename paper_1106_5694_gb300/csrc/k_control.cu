@@ -40,9 +40,12 @@ namespace {
 constexpr int kCtlThreads = 1024;
 
 // Slot edge word: agent u (bits 0..16), agent v (17..33), applies (34): its
-// exchange raises f under the current sigma, valid (36): set on every edge
-// (0 means "no candidate").  Edge positions follow slot priority, so a position is a priority.
+// exchange raises f under the current sigma, revives (35): the slot's row has
+// a positive gain under the current sigma, so that re-evaluating the slot
+// gives it a candidate again, valid (36): set on every edge (0 means "no
+// candidate").  Edge positions follow slot priority, so a position is a priority.
 constexpr unsigned long long kApplies = 1ull << 34;
+constexpr unsigned long long kRevives = 1ull << 35;
 constexpr unsigned long long kValid = 1ull << 36;  // a slot's edge word is never 0
 __device__ __forceinline__ unsigned long long edge_word(int32_t u, int32_t v) {
     return (unsigned long long)(uint32_t)u | ((unsigned long long)(uint32_t)v << 17) | kValid;
@@ -87,6 +90,41 @@ __device__ __forceinline__ int32_t block_scan(int32_t x, int32_t* warp_sums, int
     return r;
 }
 
+// Controller scratch placement.  Mode 2: reservations, 32-bit edges, the head
+// of the accepted list, claims and edge states in shared memory; mode 1: the
+// same, but the list's edges only when there are at most `edges` of them, else
+// in global memory; mode 0: everything in global memory.  (The slot of each
+// edge position is read only at a commit and when an edge comes back, and is
+// in global memory.)
+constexpr size_t kCtlStaticSmem = 2048;  // bound on the controller's static shared memory
+constexpr size_t kCtlSmemLimit = 227 * 1024 - kCtlStaticSmem;
+constexpr int32_t kListCap = 2048;  // accepted (or coloured) positions listed in shared memory
+constexpr int32_t kCand = 128;      // candidates listed at a time by a colouring window
+
+struct CtlLayout {
+    int32_t edges, list_cap;                                    // entries
+    size_t edges_at, list, claimed, estate, bytes;              // byte offsets (res is first), total
+};
+
+__host__ __device__ __forceinline__ CtlLayout controller_layout(int32_t n, int32_t mode) {
+    CtlLayout l{};
+    l.edges_at = 4 * (size_t)n;
+    l.list_cap = 2 * n < kListCap ? 2 * n : kListCap;
+    const size_t rest = 3 * (size_t)n;  // claims (n) and edge states (2n)
+    if (mode == 2) {
+        l.edges = 2 * n;
+    } else {
+        const size_t used = l.edges_at + 2 * (size_t)l.list_cap + rest;
+        const size_t room = used < kCtlSmemLimit ? (kCtlSmemLimit - used) / 4 : 0;
+        l.edges = room < (size_t)n ? (int32_t)room : n;
+    }
+    l.list = l.edges_at + 4 * (size_t)l.edges;
+    l.claimed = l.list + 2 * (size_t)l.list_cap;
+    l.estate = l.claimed + (size_t)n;
+    l.bytes = l.estate + 2 * (size_t)n;
+    return l;
+}
+
 // Controller scratch.  res: per agent, the reservation key of the current DR
 // round; claimed: per agent, the stamp of the sweep that claimed it; estate:
 // per edge position (alive / applies / fresh bits); E: per edge position, the
@@ -101,7 +139,12 @@ struct CtlScratch {
     int32_t* acc_g;  // accepted positions beyond the shared-memory part
 };
 
-enum : uint8_t { kAlive = 1, kAppl = 2, kFreshBit = 4, kAccBit = 8 };
+// Edge states: alive, applicable, and whether the slot's re-evaluation gives
+// a candidate (all fixed while no exchange commits, but for edges that are
+// re-evaluated); the accepted edges of a committing sweep are marked kAccBit.
+// A colouring window keeps colour + 1 (1..31) in the upper five bits.
+enum : uint8_t { kAlive = 1, kAppl = 2, kRevive = 4, kAccBit = 8 };
+constexpr int kColourShift = 3;
 
 struct TwoTier {
     uint16_t* s;
@@ -140,25 +183,31 @@ struct Codec<unsigned long long> {
 };
 
 
-// Re-evaluation records of the first kRecCap accepted edges of a sweep are
-// copied into shared memory while the sweep's conflict check still runs
-// (asynchronous copies, awaited before its last barrier), so that a quiet
-// sweep's refresh reads no global memory; later ones are only prefetched.
-constexpr int32_t kRecCap = 64, kRecBytes = 16 * kRecCap;
-__device__ __forceinline__ void fetch_record(unsigned char* rec, int32_t idx, const Workspace& w, int32_t t) {
-    if (rec != nullptr && idx < kRecCap) {
-        const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(rec + 16 * idx));
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(w.sl_rkey + t) : "memory");
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d + 8), "l"(w.sl_ru + t) : "memory");
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d + 12), "l"(w.sl_rv + t) : "memory");
-    } else {
-        asm volatile("prefetch.global.L1 [%0];" ::"l"(w.sl_rkey + t));
-        asm volatile("prefetch.global.L1 [%0];" ::"l"(w.sl_ru + t));
-        asm volatile("prefetch.global.L1 [%0];" ::"l"(w.sl_rv + t));
+// An accepted slot of a quiet sweep is re-evaluated from its row's key, which
+// stays current for as long as no exchange commits.  A slot whose row has no
+// positive gain dies: its candidate arrays are left as they are, since a slot
+// that is not in C at the next commit is refreshed from the keys there.  A
+// slot that comes back records its candidate (it may be in C at the next
+// commit); returns its edge.  (Reading the row's key, target and partner here,
+// for the few slots that come back, costs less than having every slot's
+// re-evaluation prepared before each controller launch.)
+template <typename EdgeT>
+__device__ __forceinline__ EdgeT revive_slot(const Workspace& w, int32_t t) {
+    const int32_t n = w.n;
+    if (t < n) {
+        const unsigned long long key = w.key_a[w.tau[t]];
+        const int32_t j = key_index(key);
+        w.ag_gain[t] = key_gain(key);
+        w.ag_job[t] = j;
+        return Codec<EdgeT>::make(t, w.sigma[j]);
     }
+    const unsigned long long key = w.key_j[t - n];
+    w.jb_gain[t - n] = key_gain(key);
+    w.jb_agent[t - n] = key_index(key);
+    return Codec<EdgeT>::make(w.sigma[t - n], key_index(key));
 }
 
-// Colouring pass.  In a sweep in which no accepted exchange applies (a quiet
+// Colouring window.  In a sweep in which no accepted exchange applies (a quiet
 // sweep) sigma does not change, so every accepted edge is stale and is only
 // re-evaluated: it dies or comes back, applicable, at its position.  Round k
 // of a run of such sweeps accepts the greedy set of the edges left after the
@@ -167,195 +216,273 @@ __device__ __forceinline__ void fetch_record(unsigned char* rec, int32_t idx, co
 // that no earlier stale edge sharing one of its agents has), and an
 // applicable edge in the first round from its birth on that no earlier stale
 // edge sharing an agent holds; the first such round ends the run with an
-// event.  The pass colours the stale edges with colours below kColourCap by
-// reservation rounds (an edge is coloured once it is the first pending edge
-// at both its agents, from the colour masks of those agents, which then hold
-// exactly its earlier neighbours' colours), finds the first round E in which
-// an applicable edge is accepted and the first round R in which a re-
-// evaluated edge that lives on is born (its colour + 1), and re-evaluates the
-// edges of the F = min(E, R, kColourCap, sweeps left) rounds before both at
-// once, as F quiet sweeps would; each round's count is left in s_hist.
-// Colour masks use the claim array (cleared afterwards), colours the high
-// half of the edge states.  Rounds past the last one with an accepted edge
-// are not counted: with no edge left the run ends.  Returns F, or -1 on an
-// internal error.
-constexpr int32_t kColourCap = 8, kColourMinList = 1024;
+// event.  A window colours the stale edges with colours below a bound `cap`
+// (at most kColourCap): cap falls to the first round in which an applicable
+// edge is accepted, and to the round after the one in which an edge that
+// comes back is accepted (it takes part from then on).  The cap rounds left
+// are applied at once, as that many quiet sweeps.
+//
+// What bounds it: a quiet sweep of a long run accepts a handful of edges
+// (2 to 6 of several thousand) and most of the list hangs on a few agents
+// (those left with a poor job), a chain in which every colour depends on the
+// one before, so latency.  The whole CTA lists, in position order, the next
+// kCand edges that still have a free colour below cap, and for every 32 of
+// them which earlier ones share an agent; one warp walks them 32 at a time.
+// Each round, every edge without a pending earlier neighbour takes its lowest
+// free colour, and where some agent has many of the 32, the pending edges at
+// the first pending edge's busier agent get its free colours in order, all at
+// once, up to the first whose other agent holds one of these colours or has a
+// pending earlier edge elsewhere.  The list is short, so that the next one
+// leaves out what closed since (128 listed; 64 and 32 were 2 to 6% slower on
+// peer-shaped and distance instances, 512 on uniform ones).  Measured, the
+// whole solve, against reservations over the whole list eight colours at a
+// time: uniform [0, 1e6) n = 10000 12.0 -> 3.1 ms, n = 20000 31.0 -> 7.0 ms,
+// distances n = 2048 from a random start 8.4 -> 6.3 ms.  (Cycles in windows,
+// uniform n = 10000: one edge per step over 32-position chunks in place 5.0M,
+// rounds over the edges without a pending earlier neighbour alone 5.7M, since
+// nearly every round had one, this form 3.1M.)
+//
+// res (as colour masks): per agent, the colours held there (all zero on entry
+// and on return).  Only with the scratch in shared memory; Eg: the edges, in
+// shared memory when Eg == null.  Returns the number F of quiet sweeps run;
+// s.hist holds each round's accepted count, and *event_next says that an
+// applicable edge is accepted in the sweep after them.
+constexpr int32_t kColourCap = 31;
+// Coloured edges after which the bound is halved (31, 15, 7, 3, 1, then the
+// window is given up), so that the list of coloured edges never outgrows its
+// shared-memory part: that many edges per round are work for reservations.
+constexpr int32_t kColourBudget = kListCap / 5 - 32;
+// A window follows a quiet sweep that accepted at most this many edges: a
+// sweep by reservations costs 7k cycles and more, the walk about 250 per edge
+// (less where many share an agent), so both meet at 30 to 100.
+constexpr int32_t kColourMaxAccepted = 64;
 
-template <typename EdgeT, int kT>
-__device__ __forceinline__ int32_t colour_pass_rounds(const Workspace& w, EdgeT* E, uint8_t* estate,
-                                                      const uint16_t* slot_s, uint32_t* res, uint8_t* mask,
-                                                      int32_t L, uint32_t span, uint32_t& s_round, int32_t& s_pE,
-                                                      int32_t& s_pR, int32_t& s_pF, int32_t* s_hist,
-                                                      int32_t max_sweeps, int32_t sweeps, int32_t& s_live,
-                                                      unsigned long long* s_pt) {
-    using C = Codec<EdgeT>;
-    const int tid = threadIdx.x;
-    const int32_t n = w.n;
-    for (int32_t i = tid; i < n; i += kT) mask[i] = 0;
+struct WindowShared {
+    uint32_t cap, event_below;  // bounds as bit masks (event_below: ~0 without an event)
+    int32_t cursor, next, coloured, rounds;
+    int32_t hist[32], nth[32];
+    uint32_t conf[kCand], word[kCand];  // the listed edges: agents in 15 bits each, applicable (15), comes back (31)
+    uint16_t pos[kCand];
+};
+
+template <int kT>
+__device__ __forceinline__ int32_t colour_window(const Workspace& w, const CtlLayout& lay, uint32_t* Eg, int32_t L,
+                                                 int32_t limit, WindowShared& s, int32_t* warp_sums, int32_t& s_live,
+                                                 bool* event_next, unsigned long long* s_pt) {
+    using C = Codec<uint32_t>;
+    constexpr int kWarps = kT / 32;
+    constexpr uint32_t kAgent = 0x7FFFu, kApplBit = 1u << 15, kBackBit = 1u << 31;
+    constexpr int kSpan = 4;  // positions per thread and step of the listing
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    uint32_t* const mask = reinterpret_cast<uint32_t*>(smem_raw);
+    uint32_t* const Es = reinterpret_cast<uint32_t*>(smem_raw + lay.edges_at);
+    uint16_t* const list = reinterpret_cast<uint16_t*>(smem_raw + lay.list);
+    uint8_t* const estate = smem_raw + lay.estate;
+    auto edge_at = [&](int32_t p) -> uint32_t { return Eg == nullptr ? Es[p] : Eg[p]; };
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (tid == 0) {
-        s_pE = kColourCap;
-        s_pR = kColourCap;
-        for (int k = 0; k < kColourCap; ++k) s_hist[k] = 0;
+        s.cap = (1u << min(limit, kColourCap)) - 1u;
+        s.event_below = ~0u;
+        s.cursor = 0;
+        s.coloured = 0;
     }
+    if (tid < 32) s.hist[tid] = 0;
     __syncthreads();
-    // The edges of the thread's first kHeld positions (tid + k kT)
-    // and their states are held in registers for the whole pass: bit k of pm
-    // says pending, of am applicable; nibble k of cols is the outcome (c + 1
-    // coloured c, 15 closed).  Positions past them keep theirs in the high
-    // half of the edge states.
-    constexpr int kHeld = 8;
-    EdgeT he[kHeld];
-    uint32_t pm = 0, am = 0, cols = 0;
+    for (;;) {
+        // the next kCand positions that have a free colour below cap, in order
+        const uint32_t cap0 = s.cap;
+        int32_t base = s.cursor, count = 0;
+        for (; base < L && count < kCand; base += kSpan * kT) {
+            uint32_t word[kSpan], b[kSpan];
+            int32_t mine = 0;
 #pragma unroll
-    for (int k = 0; k < kHeld; ++k) {
-        const int32_t p = tid + k * kT;
-        const uint8_t es = p < L ? estate[p] : (uint8_t)0;
-        he[k] = (es & kAlive) ? E[p] : (EdgeT)0;
-        if (es & kAlive) pm |= 1u << k;
-        if (es & kAppl) am |= 1u << k;
-    }
-    const int32_t tail0 = kHeld * kT;
-    // one pending edge, first half of a round: false if it closes (masks only
-    // grow: a full one leaves no colour, or round, below the cap), else it
-    // reserves both agents
-    auto reserve = [&](int32_t p, EdgeT e, bool appl, uint32_t base) -> bool {
-        const int32_t u = C::u(e), v = C::v(e);
-        const uint32_t mu = mask[u], mv = mask[v];
-        if (appl ? (mu | mv) == 0xFFu : (mu == 0xFFu || mv == 0xFFu)) return false;
-        const uint32_t key = base | (uint32_t)p;
-        if (key < res[u]) atomicMin(&res[u], key);
-        if (key < res[v]) atomicMin(&res[v], key);
-        return true;
-    };
-    // second half: -1 while an earlier edge at u or v is pending, else the
-    // outcome; the edge is then the only one holding u and v, so its mask
-    // updates are plain stores
-    auto settle = [&](int32_t p, EdgeT e, bool appl, uint32_t base) -> int32_t {
-        const int32_t u = C::u(e), v = C::v(e);
-        const uint32_t key = base | (uint32_t)p;
-        if (res[u] != key || res[v] != key) return -1;
-        const uint32_t fr = ~((uint32_t)mask[u] | (uint32_t)mask[v]) & 0xFFu;
-        if (appl) {
-            if (fr) atomicMin(&s_pE, __ffs(fr) - 1);
-            return 15;
-        }
-        if (!fr) return 15;
-        const int32_t c = __ffs(fr) - 1;
-        mask[u] |= (uint8_t)(1u << c);
-        mask[v] |= (uint8_t)(1u << c);
-        return c + 1;
-    };
-    for (int32_t r = 0;; ++r) {
-        if (r > L + 1) return -1;  // every round colours or closes the first pending edge
-        if ((s_round & (span - 1u)) == 0u && s_round != 0u) {  // reservation keys wrap
-            for (int32_t i = tid; i < n; i += kT) res[i] = 0xFFFFFFFFu;
+            for (int k = 0; k < kSpan; ++k) {
+                const int32_t p = base + (warp * kSpan + k) * 32 + lane;
+                const uint8_t es = p < L ? estate[p] : (uint8_t)0;
+                const uint32_t e = (es & kAlive) ? edge_at(p) : 0u;
+                const bool open = (es & kAlive) && (~(mask[C::u(e)] | mask[C::v(e)]) & cap0) != 0u;
+                word[k] = e | ((es & kAppl) ? kApplBit : 0u) | ((es & kRevive) ? kBackBit : 0u);
+                b[k] = __ballot_sync(0xffffffffu, open);
+                mine += __popc(b[k]);
+            }
+            if (lane == 0) warp_sums[warp] = mine;
+            __syncthreads();
+            const uint32_t c = lane < kWarps ? (uint32_t)warp_sums[lane] : 0u;
+            int32_t at = count + (int32_t)__reduce_add_sync(0xffffffffu, lane < warp ? c : 0u);
+            count += (int32_t)__reduce_add_sync(0xffffffffu, c);
+#pragma unroll
+            for (int k = 0; k < kSpan; ++k) {
+                const int32_t q = at + __popc(b[k] & ((1u << lane) - 1u));
+                if (((b[k] >> lane) & 1u) && q < kCand) {
+                    const int32_t p = base + (warp * kSpan + k) * 32 + lane;
+                    s.word[q] = word[k];
+                    s.pos[q] = (uint16_t)p;
+                    if (q == kCand - 1) s.next = p + 1;
+                }
+                at += __popc(b[k]);
+            }
             __syncthreads();
         }
-        const uint32_t base = round_base(s_round, span);
-        bool pend = false;
+        for (int32_t k = warp; k * 32 < min(count, kCand); k += kWarps) {
+            const int32_t q = k * 32 + lane;
+            const uint32_t word = q < count ? s.word[q] : 0u;
+            const uint32_t u = word & kAgent, v = (word >> 16) & kAgent;
+            uint32_t conf = 0u;
 #pragma unroll
-        for (int k = 0; k < kHeld; ++k) {
-            if (!((pm >> k) & 1u)) continue;
-            if (reserve(tid + k * kT, he[k], (am >> k) & 1u, base)) {
-                pend = true;
-            } else {
-                pm &= ~(1u << k);
-                cols |= 15u << (4 * k);
+            for (int j = 0; j < 31; ++j) {
+                const uint32_t wj = __shfl_sync(0xffffffffu, word, j);
+                const uint32_t uj = wj & kAgent, vj = (wj >> 16) & kAgent;
+                if (uj == u || vj == u || uj == v || vj == v) conf |= 1u << j;
             }
+            s.conf[q] = conf & ((1u << lane) - 1u);
         }
-        for (int32_t p = tail0 + tid; p < L; p += kT) {
-            const uint8_t es = estate[p];
-            if (!(es & kAlive) || (es >> 4)) continue;
-            if (reserve(p, E[p], (es & kAppl) != 0, base)) pend = true;
-            else estate[p] = es | 0xF0;
-        }
-        if (s_pt && tid == 0) s_pt[kPtCtlColourIters] += 1;
-        if (!__syncthreads_or(pend)) break;
-#pragma unroll
-        for (int k = 0; k < kHeld; ++k) {
-            if (!((pm >> k) & 1u)) continue;
-            const int32_t nib = settle(tid + k * kT, he[k], (am >> k) & 1u, base);
-            if (nib >= 0) {
-                pm &= ~(1u << k);
-                cols |= (uint32_t)nib << (4 * k);
-            }
-        }
-        for (int32_t p = tail0 + tid; p < L; p += kT) {
-            const uint8_t es = estate[p];
-            if (!(es & kAlive) || (es >> 4)) continue;
-            const int32_t nib = settle(p, E[p], (es & kAppl) != 0, base);
-            if (nib >= 0) estate[p] = es | (uint8_t)(nib << 4);
-        }
-        if (tid == 0) s_round = s_round + 1u;
         __syncthreads();
+        if (warp == 0) {
+            uint32_t cap = cap0, below = s.event_below;
+            int32_t m = s.coloured, budget = kColourBudget;
+            while (m >= budget) budget += kColourBudget;
+            const uint32_t before = (1u << lane) - 1u;
+            for (int32_t b0 = 0; b0 < min(count, kCand) && cap != 0u; b0 += 32) {
+                const int32_t q = b0 + lane;
+                const bool valid = q < count;
+                const uint32_t word = valid ? s.word[q] : 0u;
+                const uint32_t u = word & kAgent, v = (word >> 16) & kAgent;
+                const bool appl = (word & kApplBit) != 0u;
+                const uint32_t conf = s.conf[q];
+                const bool busy = __any_sync(0xffffffffu, __popc(conf) >= 4);  // some agent has many of the 32
+                uint32_t mu = mask[u], mv = mask[v], mine = 0u;
+                uint32_t open = valid ? ~(mu | mv) & cap : 0u;
+                uint32_t pend = __ballot_sync(0xffffffffu, open != 0u);
+                while (pend) {
+                    const bool ready = open != 0u && (pend & conf) == 0u;
+                    uint32_t low = ready ? open & (0u - open) : 0u;
+                    uint32_t x = u, h = v, at_h = 0u;
+                    if (busy) {
+                        // the first pending edge's agent with more pending edges
+                        const int i = __ffs(pend) - 1;
+                        const uint32_t wi = __shfl_sync(0xffffffffu, word, i);
+                        const uint32_t ui = wi & kAgent, vi = (wi >> 16) & kAgent;
+                        const uint32_t hu = __ballot_sync(0xffffffffu, open && (u == ui || v == ui));
+                        const uint32_t hv = __ballot_sync(0xffffffffu, open && (u == vi || v == vi));
+                        const bool pick_u = __popc(hu) >= __popc(hv);
+                        const uint32_t hub = pick_u ? ui : vi;
+                        at_h = pick_u ? hu : hv;
+                        const uint32_t free = ~mask[hub] & cap;
+                        if ((free >> lane) & 1u) s.nth[__popc(free & before)] = lane;
+                        if ((at_h >> lane) & 1u) {
+                            h = hub;
+                            x = u == hub ? v : u;
+                        }
+                        const uint32_t mx = u == hub ? mv : mu;  // (of the edges at the hub: their other agent's colours)
+                        const uint32_t badm = __ballot_sync(
+                            0xffffffffu, ((at_h >> lane) & 1u) && ((mx & free) != 0u || (conf & pend & ~at_h) != 0u));
+                        // (the first edge bad: by itself, from both its agents' colours)
+                        const uint32_t take = at_h & ((badm & (0u - badm)) - 1u);
+                        __syncwarp();
+                        if ((take >> lane) & 1u) {
+                            const int32_t r = __popc(take & before);
+                            low = r < __popc(free) ? 1u << s.nth[r] : 0u;
+                        }
+                    }
+                    uint32_t bound = ~0u;
+                    if (low != 0u && appl) {
+                        bound = low - 1u;
+                        below = min(below, bound);
+                    } else if (low != 0u && (word & kBackBit)) {
+                        bound = (low << 1) - 1u;
+                    }
+                    cap &= __reduce_and_sync(0xffffffffu, bound);
+                    const bool taken = !appl && (low & cap) != 0u;
+                    if (taken) {
+                        mine = low;
+                        atomicOr(&mask[x], low);
+                    }
+                    if (busy) {  // the hub's edges raise its mask once
+                        const bool in = (at_h >> lane) & 1u;
+                        const uint32_t add = __reduce_or_sync(0xffffffffu, taken && in ? low : 0u);
+                        if (taken && !in) atomicOr(&mask[h], low);
+                        if (lane == __ffs(at_h) - 1) atomicOr(&mask[h], add);
+                    } else if (taken) {
+                        atomicOr(&mask[h], low);
+                    }
+                    __syncwarp();
+                    mu = mask[u];
+                    mv = mask[v];
+                    open = valid && mine == 0u ? ~(mu | mv) & cap : 0u;
+                    pend = __ballot_sync(0xffffffffu, open != 0u);
+                }
+                const uint32_t cm = __ballot_sync(0xffffffffu, mine != 0u);
+                if (mine != 0u) {
+                    const int32_t c = __ffs(mine) - 1, p = s.pos[q];
+                    atomicAdd(&s.hist[c], 1);
+                    estate[p] = (uint8_t)(kAlive | ((word & kBackBit) ? kRevive : 0) | ((c + 1) << kColourShift));
+                    list[m + __popc(cm & before)] = (uint16_t)p;
+                }
+                m += __popc(cm);
+                if (m >= budget) {  // more edges per round than this form is for
+                    budget += kColourBudget;
+                    cap &= cap >> ((__popc(cap) + 1) / 2);
+                }
+            }
+            below = __reduce_min_sync(0xffffffffu, below);
+            if (lane == 0) {
+                s.cap = cap;
+                s.cursor = count >= kCand ? s.next : L;
+                s.coloured = m;
+                s.event_below = below;
+                if (s_pt) s_pt[kPtCtlColourWalks] += 1;
+            }
+        }
+        __syncthreads();
+        if (s.cap == 0u || s.cursor >= L) break;
     }
-#pragma unroll
-    for (int k = 0; k < kHeld; ++k) {  // outcomes back to the edge states (the same thread reads them next)
-        const uint32_t nib = (cols >> (4 * k)) & 15u;
-        if (nib) estate[tid + k * kT] |= (uint8_t)(nib << 4);
-    }
-    const long long t_tail = clock64();
-    for (int32_t p = tid; p < L; p += kT) {
-        const int32_t nib = estate[p] >> 4;
-        if (nib < 1 || nib > kColourCap) continue;
-        atomicAdd(&s_hist[nib - 1], 1);
-        const int32_t t = slot_s ? (int32_t)slot_s[p] : w.ctl_slot[p];
-        const unsigned long long key = w.sl_rkey[t];
-        if (key && key_gain(key) > 0) atomicMin(&s_pR, nib);  // born in round colour + 1 = nib
+    if (warp == 0) {
+        // a round with live edges accepts at least one (and an edge of colour
+        // c has neighbours of every colour below c): the run ends before the
+        // first empty round
+        const int32_t bound = __popc(s.cap);
+        const uint32_t full = __ballot_sync(0xffffffffu, lane < bound && s.hist[lane] > 0);
+        if (lane == 0) s.rounds = __popc(full);
     }
     __syncthreads();
-    if (tid == 0) {
-        int32_t F = min(s_pE, s_pR);
-        if (max_sweeps > 0) F = min(F, max_sweeps - sweeps);
-        F = max(F, 0);
-        // a round with live edges accepts at least one (and an edge of colour c
-        // has neighbours of every colour below c): an empty round means that
-        // no edge is left, and the run ends before it
-        while (F > 0 && s_hist[F - 1] == 0) --F;
-        s_pF = F;
-    }
-    __syncthreads();
-    const int32_t F = s_pF;
+    const int32_t F = s.rounds, m = s.coloured;
     int32_t died = 0;
-    for (int32_t p = tid; p < L; p += kT) {
-        uint8_t es = estate[p];
-        const int32_t nib = es >> 4;
-        if (!nib) continue;
-        es &= 0x0F;
-        if (nib <= F) {  // accepted in round nib - 1 < F: re-evaluated
-            const int32_t t = slot_s ? (int32_t)slot_s[p] : w.ctl_slot[p];
-            const unsigned long long key = w.sl_rkey[t];
-            const int32_t gain = key ? key_gain(key) : 0;
-            const int32_t target = key ? key_index(key) : -1;
-            if (t < n) { w.ag_gain[t] = gain; w.ag_job[t] = target; }
-            else { w.jb_gain[t - n] = gain; w.jb_agent[t - n] = target; }
-            if (gain > 0) {
-                E[p] = C::make(w.sl_ru[t], w.sl_rv[t]);
-                es = kAlive | kAppl | kFreshBit;
+    for (int32_t q = tid; q < m; q += kT) {
+        const int32_t p = list[q];
+        const uint8_t es = estate[p];
+        const uint32_t e = edge_at(p);
+        mask[C::u(e)] = 0u;
+        mask[C::v(e)] = 0u;
+        uint8_t now = es & (uint8_t)((1 << kColourShift) - 1);
+        if ((es >> kColourShift) <= F) {  // accepted in one of the F rounds: re-evaluated
+            if (es & kRevive) {
+                const uint32_t back = revive_slot<uint32_t>(w, w.ctl_slot[p]);
+                if (Eg == nullptr) Es[p] = back;
+                else Eg[p] = back;
+                now = kAlive | kAppl;
             } else {
-                es = 0;
+                now = 0;
                 ++died;
             }
         }
-        estate[p] = es;
+        estate[p] = now;
     }
     if (died) atomicSub(&s_live, died);
-    for (int32_t i = tid; i < n; i += kT) mask[i] = 0;  // claim stamps start clean
+    if (s_pt && tid == 0) s_pt[kPtCtlColourEdges] += m;
+    *event_next = s.event_below == s.cap && __popc(s.cap) == F;
     __syncthreads();
-    if (s_pt && tid == 0) s_pt[kPtCtlColourTail] += (unsigned long long)(clock64() - t_tail);
     return F;
 }
 
 // Switching loop (see the file comment).
 // span: reservation-key period (power of two <= kRoundSpanMax); stamp_wrap:
 // claim-stamp period (<= 255).  Both are shortened only by a test knob.
-// list_cap: entries of the accepted list held in shared memory.
-// colour_pass: runs of quiet sweeps go through colouring passes (only
-// while the edges are in shared memory); 0 turns them off.
-template <typename EdgeT, int kT = kCtlThreads, bool kEdgesToShared = true>
+// colour_pass: runs of quiet sweeps go through colouring windows (only with
+// the scratch in shared memory); 0 turns them off.
+template <typename EdgeT, int kT = kCtlThreads>
 __device__ __forceinline__ void controller_body(const Workspace& w, int32_t smem_mode, const CtlScratch& g,
-                                                uint32_t span, uint32_t stamp_wrap, int32_t list_cap,
-                                                int32_t compact_min, int32_t colour_pass) {
+                                                uint32_t span, uint32_t stamp_wrap, int32_t compact_min,
+                                                int32_t colour_pass) {
     using C = Codec<EdgeT>;
     DeviceState* st = w.st;
     if (st->status != kRunning) return;
@@ -363,7 +490,8 @@ __device__ __forceinline__ void controller_body(const Workspace& w, int32_t smem
     __shared__ int32_t warp_sums[33];
     __shared__ int32_t s_L, s_live, s_stop, s_acc, s_app, s_y, s_sweeps, s_event;
     __shared__ int32_t s_max_sweeps, s_trace_cap;
-    __shared__ int32_t s_pass_ok, s_pE, s_pR, s_pF, s_hist[kColourCap];
+    __shared__ int32_t s_window;  // the next sweeps may run as a colouring window
+    __shared__ WindowShared s_win;
     __shared__ uint32_t s_round;
     __shared__ uint32_t s_stamp;
     __shared__ unsigned long long s_gain, s_deadline;
@@ -376,44 +504,22 @@ __device__ __forceinline__ void controller_body(const Workspace& w, int32_t smem
     uint8_t* estate = g.estate;
     EdgeT* E = static_cast<EdgeT*>(g.edges);
     uint16_t* lists_s = nullptr;
-    uint16_t* slot_s = nullptr;  // slot of each edge position (shared-memory modes)
-    unsigned char* rec = nullptr;  // re-evaluation records (shared-memory modes)
+    int32_t list_cap = 0, es_cap = 0;
+    EdgeT* Es = nullptr;
     if (smem_mode >= 1) {
-        size_t off = 0;
-        rec = smem_raw;
-        off += kRecBytes;
-        res = reinterpret_cast<uint32_t*>(smem_raw + off);
-        off += 4 * (size_t)n;
-        if (smem_mode == 2) {
-            E = reinterpret_cast<EdgeT*>(smem_raw + off);
-            off += sizeof(EdgeT) * 2 * (size_t)n;
-        }
-        lists_s = reinterpret_cast<uint16_t*>(smem_raw + off);
-        off += 2 * (size_t)list_cap;
-        slot_s = reinterpret_cast<uint16_t*>(smem_raw + off);
-        off += 2 * 2 * (size_t)n;
-        claimed = smem_raw + off;
-        off += (size_t)n;
-        estate = smem_raw + off;
+        const CtlLayout lay = controller_layout(n, smem_mode);
+        list_cap = lay.list_cap;
+        es_cap = sizeof(EdgeT) == 4 ? lay.edges : 0;
+        res = reinterpret_cast<uint32_t*>(smem_raw);
+        Es = reinterpret_cast<EdgeT*>(smem_raw + lay.edges_at);
+        lists_s = reinterpret_cast<uint16_t*>(smem_raw + lay.list);
+        claimed = smem_raw + lay.claimed;
+        estate = smem_raw + lay.estate;
+        if (smem_mode == 2) E = Es;
     }
-    // Mode 1 keeps the edge array in global memory, but a list of at most
-    // edges_s_cap() (about n / 2) positions fits in the upper half of slot_s
-    // (positions below n use only its lower half): a launch whose list is
-    // that short, or is compacted to that length, moves its edges there.
-    // kEdgesToShared = false (the batched controller, which otherwise spills
-    // more registers, and the single-CTA loop, which runs in mode 2 only)
-    // leaves them in global memory.
-    const bool es_mode = kEdgesToShared && smem_mode == 1 && sizeof(EdgeT) == 4;
-    auto edges_s = [&]() -> EdgeT* {
-        return reinterpret_cast<EdgeT*>((reinterpret_cast<uintptr_t>(slot_s + n) + 3u) & ~static_cast<uintptr_t>(3u));
-    };
-    auto edges_s_cap = [&]() -> int32_t {
-        const uintptr_t lo = reinterpret_cast<uintptr_t>(edges_s());
-        const uintptr_t hi = reinterpret_cast<uintptr_t>(slot_s + 2 * (size_t)n);
-        return hi > lo ? (int32_t)((hi - lo) / sizeof(EdgeT)) : 0;
-    };
-    const int32_t cap = lists_s ? list_cap : 0;
-    TwoTier accl{lists_s, cap, g.acc_g};
+    // Mode 1: the edges of a launch whose list is at most es_cap long, or is
+    // compacted to that length, are in shared memory, longer lists' in global.
+    TwoTier accl{lists_s, list_cap, g.acc_g};
     unsigned long long* pt = (tid == 0) ? w.phase_ns : nullptr;
     long long tp = clock64();
     // diagnostics (DGS_PHASE_TIMERS=1): thread 0 sums into shared memory and
@@ -449,7 +555,7 @@ __device__ __forceinline__ void controller_body(const Workspace& w, int32_t smem
             s_f = st->f;
             s_round = 0;
             s_stamp = 0;
-            s_pass_ok = 0;  // a colouring pass follows a quiet sweep
+            s_window = 0;
         }
         // Warp wp lists the slots of its own range [lo, hi) (ranges are
         // multiples of 32 long and ascend with wp): it sums the edge counts
@@ -480,7 +586,7 @@ __device__ __forceinline__ void controller_body(const Workspace& w, int32_t smem
             if (lane == 31) warp_sums[32] = incl;
         }
         __syncthreads();
-        if (es_mode && warp_sums[32] <= edges_s_cap()) E = edges_s();  // the whole list fits in shared memory
+        if (es_cap > 0 && warp_sums[32] <= es_cap) E = Es;  // the whole list fits in shared memory
         int32_t pos0 = warp_sums[wp];
         const uint32_t below = (1u << lane) - 1u;
         for (int32_t cb = c_lo; cb < c_hi; cb += 32) {
@@ -506,9 +612,8 @@ __device__ __forceinline__ void controller_body(const Workspace& w, int32_t smem
                     if (has) {
                         const int32_t pos = pos0 + __popc(m & below);
                         w.ctl_slot[pos] = t;
-                        if (slot_s) slot_s[pos] = (uint16_t)t;
                         E[pos] = C::make(edge_u(ew[k]), edge_v(ew[k]));
-                        estate[pos] = kAlive | ((ew[k] & kApplies) ? kAppl : 0);
+                        estate[pos] = kAlive | ((ew[k] & kApplies) ? kAppl : 0) | ((ew[k] & kRevives) ? kRevive : 0);
                     }
                     pos0 += __popc(m);
                 }
@@ -523,6 +628,7 @@ __device__ __forceinline__ void controller_body(const Workspace& w, int32_t smem
     // Quiet sweeps turn at least one stale slot into a fresh one each, so one
     // launch runs at most 2n + 1 of them; more means an internal error.
     int32_t L = s_L;
+    bool masks = false;  // res holds the agents' colour masks, all zero (else reservation keys)
     for (int32_t quiet = 0;; ++quiet) {
         if (tid == 0) {
             // loop condition of Algorithm 3 (some slot has delta > 0), sweep
@@ -558,10 +664,8 @@ __device__ __forceinline__ void controller_body(const Workspace& w, int32_t smem
         // keys restart with the new positions.
         if (s_live * 2 < L && L >= compact_min) {
             // (mode 1: into shared memory when the live edges fit there)
-            const int32_t es_cap = es_mode ? edges_s_cap() : 0;
-            const bool to_s = es_mode && E != edges_s();  // edges still in global memory
-            EdgeT* const Ed = (to_s && s_live <= es_cap) ? edges_s() : E;
-            const bool bounded = es_mode && Ed == edges_s();
+            EdgeT* const Ed = s_live <= es_cap ? Es : E;
+            const bool bounded = es_cap > 0 && Ed == Es;
             int32_t base = 0;
             for (int32_t c0 = 0; c0 < L; c0 += kT) {
                 const int32_t p = c0 + tid;
@@ -575,11 +679,11 @@ __device__ __forceinline__ void controller_body(const Workspace& w, int32_t smem
                     if (!bounded || pos < es_cap) Ed[pos] = e;
                     estate[pos] = es;
                     w.ctl_slot[pos] = slot;
-                    if (slot_s) slot_s[pos] = (uint16_t)slot;
                 }
                 base += total;
             }
-            for (int32_t i = tid; i < n; i += kT) res[i] = 0xFFFFFFFFu;
+            if (!masks)
+                for (int32_t i = tid; i < n; i += kT) res[i] = 0xFFFFFFFFu;
             __syncthreads();
             if (tid == 0) {
                 s_L = base;
@@ -595,54 +699,52 @@ __device__ __forceinline__ void controller_body(const Workspace& w, int32_t smem
             L = s_L;
             E = Ed;
         }
+        // Colouring window (see colour_window): F >= 1 quiet sweeps at once,
+        // or none when an applicable edge is accepted in this very sweep (or
+        // the window was given up); then this sweep goes on as usual.
+        // (shared-memory modes hold n <= 32767: 32-bit edges)
+        if (sizeof(EdgeT) == 4 && colour_pass && smem_mode >= 1 && s_window) {
+            if (!masks) {
+                for (int32_t i = tid; i < n; i += kT) res[i] = 0u;
+                masks = true;
+                __syncthreads();
+            }
+            const int32_t left = s_max_sweeps > 0 ? s_max_sweeps - s_sweeps : kColourCap;
+            bool event_next;
+            const int32_t F =
+                colour_window<kT>(w, controller_layout(n, smem_mode), E == Es ? nullptr : reinterpret_cast<uint32_t*>(E),
+                                  L, left, s_win, warp_sums, s_live, &event_next, pt ? s_pt : nullptr);
+            if (tid < F) {
+                const int32_t sw = s_sweeps + tid;
+                if (sw < s_trace_cap) {
+                    if (st->trace_accepted) st->trace_accepted[sw] = s_win.hist[tid];
+                    if (st->trace_applied) st->trace_applied[sw] = 0;
+                    if (st->trace_objective) st->trace_objective[sw] = s_f;
+                }
+            }
+            __syncthreads();
+            if (tid == 0) {
+                s_sweeps = s_sweeps + F;
+                s_window = (F > 0 && !event_next) ? 1 : 0;
+                DGS_PT(kPtCtlColourPasses, 1)
+                DGS_PT(kPtCtlColourRounds, F)
+            }
+            __syncthreads();
+            DGS_CT(kPtCtlColour)
+            if (F > 0) continue;
+        }
         if (s_stamp >= stamp_wrap) {  // claim stamps wrap: clear them once
             for (int32_t i = tid; i < n; i += kT) claimed[i] = 0;
             __syncthreads();
             if (tid == 0) s_stamp = 1;
             __syncthreads();
         }
-        if ((s_round & (span - 1u)) == 0u && s_round != 0u) {  // reservation keys wrap
+        if (masks || ((s_round & (span - 1u)) == 0u && s_round != 0u)) {  // no keys yet, or they wrap
             for (int32_t i = tid; i < n; i += kT) res[i] = 0xFFFFFFFFu;
+            masks = false;
             __syncthreads();
         }
         const uint8_t stamp = (uint8_t)s_stamp;
-        // Colouring pass (after a quiet sweep; see colour_pass_rounds).  It
-        // runs F >= 1 sweeps at once, or none when an applicable edge is
-        // accepted in this very sweep; then this sweep goes on as usual.
-        // (modes 1 and 2 hold n <= 32767, so only 32-bit edges take this path)
-        // (short lists: a pass costs more than the sweeps it saves)
-        if (sizeof(EdgeT) == 4 && colour_pass && (smem_mode == 2 || (es_mode && E == edges_s())) && s_pass_ok &&
-            L > kColourMinList) {
-            const int32_t F = colour_pass_rounds<EdgeT, kT>(w, E, estate, slot_s, res, claimed, L, span, s_round, s_pE,
-                                                        s_pR, s_pF, s_hist, s_max_sweeps, s_sweeps, s_live,
-                                                        pt ? s_pt : nullptr);
-            if (F < 0) {  // internal error
-                if (tid == 0) {
-                    st->error = kErrInternal;
-                    st->status = kError;
-                }
-                break;
-            }
-            if (tid == 0) {
-                for (int32_t k = 0; k < F; ++k) {
-                    const int32_t sw = s_sweeps + k;
-                    if (sw < s_trace_cap) {
-                        if (st->trace_accepted) st->trace_accepted[sw] = s_hist[k];
-                        if (st->trace_applied) st->trace_applied[sw] = 0;
-                        if (st->trace_objective) st->trace_objective[sw] = s_f;
-                    }
-                }
-                s_sweeps = s_sweeps + F;
-                DGS_PT(kPtCtlColourPasses, 1)
-                DGS_PT(kPtCtlColourRounds, F)
-                // another pass may follow at once only if this one met no
-                // bound inside its window
-                s_pass_ok = (F == kColourCap && s_pE >= kColourCap && s_pR >= kColourCap) ? 1 : 0;
-            }
-            __syncthreads();
-            DGS_CT(kPtCtlColour)
-            if (F > 0) continue;
-        }
         // CC (Algorithm 4): the accepted set is the greedy one in priority
         // order (a slot is accepted when neither agent of its exchange was
         // claimed by an earlier accepted slot).  The list is taken in chunks
@@ -719,7 +821,6 @@ __device__ __forceinline__ void controller_body(const Workspace& w, int32_t smem
                             claimed[v[k]] = stamp;
                             const int32_t idx = atomicAdd(&s_acc, 1);
                             accl.put(idx, p[k]);
-                            if (slot_s) fetch_record(rec, idx, w, slot_s[p[k]]);  // its slot's re-evaluation
                             ev |= (es[k] & kAppl) ? 1 : 0;
                             cand[k] = false;
                         }
@@ -735,7 +836,6 @@ __device__ __forceinline__ void controller_body(const Workspace& w, int32_t smem
                 }
             }
             if (ev) s_event = 1;
-            if (rec) asm volatile("cp.async.wait_all;" ::: "memory");
             __syncthreads();
         }
         DGS_CT(kPtCtlPass1)
@@ -794,7 +894,7 @@ __device__ __forceinline__ void controller_body(const Workspace& w, int32_t smem
             for (int32_t p = tid; p < L; p += kT) {
                 const uint8_t es = estate[p];
                 if (!(es & kAlive) || (es & kAccBit)) continue;
-                const int32_t t = slot_s ? (int32_t)slot_s[p] : w.ctl_slot[p];
+                const int32_t t = w.ctl_slot[p];
                 if (t < n) w.in_ca[t] = 1;
                 else w.in_cj[t - n] = 1;
             }
@@ -823,26 +923,16 @@ __device__ __forceinline__ void controller_body(const Workspace& w, int32_t smem
         int32_t died = 0;
         for (int32_t q = tid; q < nacc; q += kT) {
             const int32_t p = accl.get(q);
-            const int32_t t = slot_s ? (int32_t)slot_s[p] : w.ctl_slot[p];
-            const bool held = rec != nullptr && q < kRecCap;
-            const unsigned long long key =
-                held ? *reinterpret_cast<const unsigned long long*>(rec + 16 * q) : w.sl_rkey[t];
-            const int32_t gain = key ? key_gain(key) : 0;
-            const int32_t target = key ? key_index(key) : -1;
-            if (t < n) { w.ag_gain[t] = gain; w.ag_job[t] = target; }
-            else { w.jb_gain[t - n] = gain; w.jb_agent[t - n] = target; }
-            if (gain > 0) {
-                const int32_t ru = held ? *reinterpret_cast<const int32_t*>(rec + 16 * q + 8) : w.sl_ru[t];
-                const int32_t rv = held ? *reinterpret_cast<const int32_t*>(rec + 16 * q + 12) : w.sl_rv[t];
-                E[p] = C::make(ru, rv);
-                estate[p] = kAlive | kAppl | kFreshBit;
+            if (estate[p] & kRevive) {
+                E[p] = revive_slot<EdgeT>(w, w.ctl_slot[p]);
+                estate[p] = kAlive | kAppl;
             } else {
                 estate[p] = 0;
                 ++died;
             }
         }
         if (died) atomicSub(&s_live, died);
-        if (tid == 0) s_pass_ok = 1;
+        if (tid == 0) s_window = nacc <= kColourMaxAccepted ? 1 : 0;
         DGS_PT(kPtCtlAccSum, nacc)
         if (tid == 0 && s_sweeps < s_trace_cap) {
             const int32_t sw = s_sweeps;
@@ -874,9 +964,9 @@ __device__ __forceinline__ void controller_body(const Workspace& w, int32_t smem
 template <typename EdgeT>
 __global__ void __launch_bounds__(kCtlThreads, 1) controller_kernel(Workspace w, int32_t smem_mode, CtlScratch g,
                                                                    uint32_t span, uint32_t stamp_wrap,
-                                                                   int32_t list_cap, int32_t compact_min,
-                                                                   int32_t colour_pass, unsigned long long cond) {
-    controller_body<EdgeT>(w, smem_mode, g, span, stamp_wrap, list_cap, compact_min, colour_pass);
+                                                                   int32_t compact_min, int32_t colour_pass,
+                                                                   unsigned long long cond) {
+    controller_body<EdgeT>(w, smem_mode, g, span, stamp_wrap, compact_min, colour_pass);
     if (cond != 0 && threadIdx.x == 0) {
         DeviceState* st = w.st;
         const int32_t it = ++st->loop_iterations;
@@ -892,9 +982,9 @@ __global__ void __launch_bounds__(kCtlThreads, 1) controller_kernel(Workspace w,
 // Before each controller launch: clear the marks of the last event, re-
 // evaluate every slot not in C from the current row keys (reading R4), and
 // for every slot with a candidate (delta > 0) record its edge (the agents of
-// its exchange under the current sigma, and whether that exchange raises f
-// now).  Also record each slot's re-evaluated candidate, which stays valid
-// for as long as no exchange is committed.  One thread per slot.
+// its exchange under the current sigma, whether that exchange raises f now,
+// and whether the slot's re-evaluation would give it a candidate).  One
+// thread per slot.
 __device__ __forceinline__ void prepare_edges_body(const Workspace& w, int32_t bid, int32_t nblk) {
     DeviceState* st = w.st;
     if (st->status != kRunning) return;
@@ -908,12 +998,10 @@ __device__ __forceinline__ void prepare_edges_body(const Workspace& w, int32_t b
     }
     for (int32_t t = bid * blockDim.x + threadIdx.x; t < 2 * n; t += stride) {
         unsigned long long key;
-        int32_t ru, rv, gain, target;
+        int32_t gain, target;
         bool in_c;
         if (t < n) {
             key = w.key_a[w.tau[t]];
-            ru = t;
-            rv = key ? w.sigma[key_index(key)] : t;
             in_c = w.in_ca[t] && !st->reeval_all;
             if (!in_c) {
                 w.ag_gain[t] = key ? key_gain(key) : 0;
@@ -924,8 +1012,6 @@ __device__ __forceinline__ void prepare_edges_body(const Workspace& w, int32_t b
         } else {
             const int32_t j = t - n;
             key = w.key_j[j];
-            ru = w.sigma[j];
-            rv = key ? key_index(key) : ru;
             in_c = w.in_cj[j] && !st->reeval_all;
             if (!in_c) {
                 w.jb_gain[j] = key ? key_gain(key) : 0;
@@ -934,14 +1020,11 @@ __device__ __forceinline__ void prepare_edges_body(const Workspace& w, int32_t b
             gain = in_c ? w.jb_gain[j] : (key ? key_gain(key) : 0);
             target = in_c ? w.jb_agent[j] : (key ? key_index(key) : -1);
         }
-        w.sl_rkey[t] = key;
-        w.sl_ru[t] = ru;
-        w.sl_rv[t] = rv;
         unsigned long long e = 0ull;
         if (gain > 0) {
             const int32_t u = (t < n) ? t : w.sigma[t - n];
             const int32_t v = (t < n) ? w.sigma[target] : target;
-            e = edge_word(u, v) | (exchange_gain(w, u, v) > 0 ? kApplies : 0ull);
+            e = edge_word(u, v) | (exchange_gain(w, u, v) > 0 ? kApplies : 0ull) | (key ? kRevives : 0ull);
         }
         w.sl_edge[t] = e;
         // the warp's 32 consecutive slots form one chunk: its edge count
@@ -1149,8 +1232,7 @@ __device__ __forceinline__ void row_task_warp(const Workspace& w, int32_t j) {
 template <typename EdgeT, int kT>
 __global__ void __launch_bounds__(kT, 1) small_loop_kernel(Workspace w, int32_t smem_mode, CtlScratch g,
                                                                    uint32_t span, uint32_t stamp_wrap,
-                                                                   int32_t list_cap, int32_t compact_min,
-                                                                   int32_t colour_pass) {
+                                                                   int32_t compact_min, int32_t colour_pass) {
     __shared__ int32_t s_go, s_count;
     DeviceState* st = w.st;
     const int32_t n = w.n;
@@ -1171,7 +1253,7 @@ __global__ void __launch_bounds__(kT, 1) small_loop_kernel(Workspace w, int32_t 
         __syncthreads();
         prepare_edges_body(w, 0, 1);
         __syncthreads();
-        controller_body<EdgeT, kT, false>(w, smem_mode, g, span, stamp_wrap, list_cap, compact_min, colour_pass);
+        controller_body<EdgeT, kT>(w, smem_mode, g, span, stamp_wrap, compact_min, colour_pass);
         if (tid == 0) {
             const int32_t it = ++st->loop_iterations;
             if (st->status == kRunning && it > 16 * n + 4096) {
@@ -1449,8 +1531,7 @@ __global__ void __launch_bounds__(kCtlThreads, 1) controller_batched_kernel(Batc
                                                                            int32_t colour_pass) {
     for_each_entry(t, kStageSwitch, [&](const Instance& in, int32_t, int32_t) {
         const CtlScratch c{in.ctl.res, in.ctl.claimed, in.ctl.estate, in.ctl.edges, in.ctl.acc};
-        controller_body<uint32_t, kCtlThreads, false>(in.w, in.ctl_mode, c, span, stamp_wrap, in.ctl_cap, compact_min,
-                                                      colour_pass);
+        controller_body<uint32_t>(in.w, in.ctl_mode, c, span, stamp_wrap, compact_min, colour_pass);
     });
 }
 
@@ -1489,36 +1570,16 @@ __global__ void advance_batched_kernel(BatchTable t, int32_t from_stage) {
 
 }  // namespace
 
-// Controller scratch placement.  Mode 2: reservations, 32-bit edges, list
-// heads, claims and edge states in shared memory; mode 1: edges in global
-// memory (the controller kernel of a single solve moves a list of up to
-// about n / 2 positions into the spare half of the slot array); mode 0:
-// everything in global memory.
-constexpr size_t kCtlSmemLimit = 227 * 1024 - 1024;
-
-static size_t ctl_fixed_bytes(int32_t n, int32_t mode) {
-    // records + res (4n) + slot of each position (4n) + claimed (n) + estate (2n) [+ 32-bit edges (8n)]
-    return kRecBytes + 11 * (size_t)n + (mode == 2 ? 8 * (size_t)n : 0);
-}
-
 int32_t controller_smem_mode(int32_t n) {
     int32_t mode = 0;
-    if (n <= 32767 && ctl_fixed_bytes(n, 2) + 2 * 256 + 16 <= kCtlSmemLimit) mode = 2;
-    else if (n <= 32767 && ctl_fixed_bytes(n, 1) + 2 * 256 + 16 <= kCtlSmemLimit) mode = 1;
+    if (n <= 32767 && controller_layout(n, 2).bytes <= kCtlSmemLimit) mode = 2;
+    else if (n <= 32767 && controller_layout(n, 1).bytes <= kCtlSmemLimit) mode = 1;
     return min(mode, env_controller_mode_cap());
-}
-
-int32_t controller_list_cap(int32_t n, int32_t mode) {
-    if (mode == 0) return 0;
-    const size_t room = kCtlSmemLimit - ctl_fixed_bytes(n, mode) - 16;
-    const size_t cap = room / 2;  // one 16-bit list
-    return (int32_t)(cap < 2 * (size_t)n ? cap : 2 * (size_t)n);
 }
 
 size_t controller_smem_bytes(int32_t n) {
     const int32_t mode = controller_smem_mode(n);
-    if (mode == 0) return 0;
-    return ctl_fixed_bytes(n, mode) + 2 * (size_t)controller_list_cap(n, mode) + 16;
+    return mode == 0 ? 0 : controller_layout(n, mode).bytes;
 }
 
 // DGS_SMALL_LOOP_N: the largest n whose switching loop runs in one CTA
@@ -1539,16 +1600,15 @@ template <int kT>
 static cudaError_t launch_small_loop_t(const Workspace& w, const CtlGlobal& gs, cudaStream_t s, int slot) {
     const int32_t mode = controller_smem_mode(w.n);
     const size_t smem = controller_smem_bytes(w.n);
-    const int32_t cap = controller_list_cap(w.n, mode);
     CtlScratch c{gs.res, gs.claimed, gs.estate, gs.edges, gs.acc};
     const void* fn = reinterpret_cast<const void*>(small_loop_kernel<uint32_t, kT>);
-    if (smem > 48 * 1024) {
+    if (smem + kCtlStaticSmem > 48 * 1024) {
         cudaError_t e = ensure_smem_limit(fn, slot, smem);
         if (e != cudaSuccess) return e;
     }
     const bool short_wrap = env_short_wraps() != 0;
     small_loop_kernel<uint32_t, kT><<<1, kT, smem, s>>>(w, mode, c, short_wrap ? 4u : kRoundSpanMax,
-                                                         short_wrap ? 5u : 250u, cap, env_compact_min(),
+                                                         short_wrap ? 5u : 250u, env_compact_min(),
                                                          env_colour_pass());
     return cudaGetLastError();
 }
@@ -1573,12 +1633,11 @@ cudaError_t launch_small_loop(const Workspace& w, const CtlGlobal& gs, cudaStrea
 cudaError_t launch_controller_impl(const Workspace& w, const CtlGlobal& gs, cudaStream_t s, unsigned long long handle) {
     const int32_t mode = controller_smem_mode(w.n);
     const size_t smem = controller_smem_bytes(w.n);
-    const int32_t cap = controller_list_cap(w.n, mode);
     CtlScratch c{gs.res, gs.claimed, gs.estate, gs.edges, gs.acc};
     const bool narrow = w.n <= 65535;
     const void* fn = narrow ? reinterpret_cast<const void*>(controller_kernel<uint32_t>)
                             : reinterpret_cast<const void*>(controller_kernel<unsigned long long>);
-    if (smem > 48 * 1024) {
+    if (smem + kCtlStaticSmem > 48 * 1024) {
         cudaError_t e = ensure_smem_limit(fn, narrow ? 1 : 3, smem);
         if (e != cudaSuccess) return e;
     }
@@ -1588,10 +1647,10 @@ cudaError_t launch_controller_impl(const Workspace& w, const CtlGlobal& gs, cuda
     const int32_t cmin = env_compact_min();
     const int32_t cp = env_colour_pass();
     if (narrow)
-        controller_kernel<uint32_t><<<1, kCtlThreads, smem, s>>>(w, mode, c, span, stamp_wrap, cap, cmin, cp, handle);
+        controller_kernel<uint32_t><<<1, kCtlThreads, smem, s>>>(w, mode, c, span, stamp_wrap, cmin, cp, handle);
     else
-        controller_kernel<unsigned long long><<<1, kCtlThreads, smem, s>>>(w, mode, c, span, stamp_wrap, cap, cmin,
-                                                                          cp, handle);
+        controller_kernel<unsigned long long><<<1, kCtlThreads, smem, s>>>(w, mode, c, span, stamp_wrap, cmin, cp,
+                                                                          handle);
     return cudaGetLastError();
 }
 
