@@ -418,9 +418,9 @@ def run_ours(args):
     peak, peak_src = measured_hbm_peak()
     # the greedy start is the largest kernel of this workload's solve
     # (committed ncu launch list): deferred acceptance, whose algorithmic
-    # bytes are the agents' rows it rescans (4n each), the pass-1 row bests
-    # it starts from (8n) and the jobs' holder keys and benefits (12n)
-    greedy_bytes = 4 * n * stats["greedy_rescans"] + 8 * n + 12 * n
+    # bytes are the tiles of 64 jobs it looks at (4-byte benefits, 8-byte
+    # holder keys), the table of the tiles' bounds and the jobs' holders (12n)
+    greedy_bytes = 64 * 12 * stats["greedy_rescans"] + 4 * n * ((n + 63) // 64) + 12 * n
     roofline = roofline_entry("greedy_da_kernel", "greedy start (Section 3.1): deferred acceptance after pass 1",
                               greedy_bytes, statistics.mean(greedy_ms), n, args.workload, peak, peak_src)
     roofline_eval = roofline_entry("full_evaluation_kernel",

@@ -169,8 +169,10 @@ typedef struct {
     int64_t kernel_launches;  /* kernels this call launched */
     double evaluation_ms;     /* first full evaluation, when options.profile */
     double greedy_ms;         /* greedy start after pass 1, when options.profile */
-    int64_t greedy_rescans;   /* rows of a (or its transpose) the greedy start
-                                 rescanned (depends on the order of proposals) */
+    int64_t greedy_rescans;   /* greedy start: tiles of an agent's row (64 jobs;
+                                 up to n / 16 in a batch) that were looked at
+                                 (depends on the order of proposals), or the
+                                 rows the fallback rescanned */
     int32_t status;           /* the solve's outcome (a dgs_status) */
     double solve_ms;          /* everything the call enqueued, when options.profile */
 } dgs_stats;

@@ -22,13 +22,6 @@
 #include "dgs_internal.cuh"
 
 namespace dgs {
-// pass 1 over a band of tile rows (k_greedy.cu)
-cudaError_t launch_greedy_pass1_rows(const Workspace& w, int32_t cols, int32_t row_tile0, int32_t row_tile1,
-                                     cudaStream_t s);
-}  // namespace dgs
-
-
-namespace dgs {
 int32_t env_update_policy() {
     static const int32_t v = [] {
         const char* e = std::getenv("DGS_UPDATE_POLICY");
@@ -199,6 +192,7 @@ struct Plan {
     bool need_copy = false;   // a must be re-laid out (n % 4 != 0 or misaligned)
     bool need_at = true;      // transposed copy (greedy start, row tasks)
     int32_t lda = 0, ldt = 0;
+    int32_t bound_shift = kBoundShift;  // tiles of the greedy start's bounds
     size_t bytes = 0;
 };
 
@@ -210,6 +204,12 @@ size_t carve(Arena& ar, Workspace& w, const Plan& p, int32_t n, CtlGlobal* ctl, 
     const size_t nb = align_up((size_t)n, 128);
     *a_copy = p.need_copy ? ar.take<int32_t>((size_t)n * p.lda) : nullptr;
     w.at = p.need_at ? ar.take<int32_t>((size_t)n * p.ldt + 64) : nullptr;
+    // bounds of 64-job tiles are all stored by pass 1; those of wider tiles
+    // are raised from zero, so they belong to the arrays cleared before it
+    w.bound_shift = p.bound_shift;
+    w.bound_tiles = bound_tiles(n, p.bound_shift);
+    const bool wide = p.need_at && p.bound_shift != kBoundShift;
+    w.g_bound = p.need_at && !wide ? ar.take<uint32_t>((size_t)n * w.bound_tiles) : nullptr;
     w.sigma = ar.take<int32_t>(nb);
     w.tau = ar.take<int32_t>(nb);
     w.diag = ar.take<int32_t>(nb);
@@ -232,7 +232,7 @@ size_t carve(Arena& ar, Workspace& w, const Plan& p, int32_t n, CtlGlobal* ctl, 
     w.g_col = ar.take<unsigned long long>(nb);
     w.free_a = ar.take<uint8_t>(nb);
     w.free_j = ar.take<uint8_t>(nb);
-    w.g_list = ar.take<unsigned long long>(4 * nb);
+    if (wide) w.g_bound = ar.take<uint32_t>((size_t)n * w.bound_tiles);
     w.phase_ns = env_phase_timers() ? ar.take<unsigned long long>(kPtCount) : nullptr;
     w.st = ar.take<DeviceState>(1);
     *seen = ar.take<uint8_t>(4 * nb);
@@ -275,6 +275,7 @@ size_t carve_instance(char* base, int32_t n, bool need_copy, Instance* in) {
     p.need_at = true;
     p.lda = need_copy ? round_up32(n, 4) : n;
     p.ldt = round_up32(n, 64);
+    p.bound_shift = instance_bound_shift(n);
     Arena ar;
     ar.base = base;
     Workspace w{};
@@ -599,8 +600,8 @@ dgs_status sequential_pass_body(void* p, cudaStream_t cs, unsigned long long h) 
     return DGS_OK;
 }
 
-// The greedy start: pass 1, then deferred acceptance in one cooperative
-// launch; where that launch is refused, pass 1 again with the column keys and
+// The greedy start: pass 1, then deferred acceptance in one launch; where
+// that launch is refused, pass 1 again with the row and column keys and
 // the locally-dominant rounds as a device-side loop (the same assignment).
 // A matrix that arrives in row bands (dgs_solve_host): event k is recorded
 // once rows [64 k tile_rows, 64 (k + 1) tile_rows) are on the device.
@@ -612,12 +613,12 @@ struct HostBands {
 
 dgs_status run_greedy(Solve& S, EventPair* timer, const HostBands* bands = nullptr) {
     if (bands == nullptr) {
-        DGS_CUDA(launch_greedy_pass1_cols(S.w, 0, S.s), "greedy pass 1");
+        DGS_CUDA(launch_greedy_pass1_bounds(S.w, 0, (S.w.n + 63) / 64, S.s), "greedy pass 1");
         S.launches += 1;
     } else {  // pass 1 of each band as soon as it has landed, while later ones are still copied
         for (int32_t k = 0; k < bands->count; ++k) {
             DGS_CUDA(cudaStreamWaitEvent(S.s, bands->ev[k], 0), "wait for a band of the matrix");
-            DGS_CUDA(launch_greedy_pass1_rows(S.w, 0, k * bands->tile_rows, (k + 1) * bands->tile_rows, S.s),
+            DGS_CUDA(launch_greedy_pass1_bounds(S.w, k * bands->tile_rows, (k + 1) * bands->tile_rows, S.s),
                      "greedy pass 1");
             S.launches += 1;
         }
@@ -630,7 +631,7 @@ dgs_status run_greedy(Solve& S, EventPair* timer, const HostBands* bands = nullp
         return DGS_OK;
     }
     cudaGetLastError();
-    DGS_CUDA(launch_greedy_pass1_cols(S.w, 1, S.s), "greedy pass 1");
+    DGS_CUDA(launch_greedy_pass1_rounds(S.w, S.s), "greedy pass 1");
     S.launches += 1;
     LoopCtx c{S.w, S.ctl};
     DGS_TRY(enqueue_loop(S.s, greedy_round_body, &c));

@@ -53,7 +53,7 @@ struct DeviceState {
     int32_t greedy_matched;  // the last match kernel matched >= 1 pair
     int32_t update_policy;   // 0: by cost, 1: always full evaluation, 2: always row tasks
     int32_t max_abs;         // max |a| (set by the passes that check the range)
-    long long greedy_rescans;  // rows of a / at rescanned by the greedy start
+    long long greedy_rescans;  // greedy start: tiles of an agent's row looked at (rounds: rows rescanned)
     uint32_t bar_count;      // grid barrier of cooperative launches: arrivals
     uint32_t bar_gen;        //   and generation
     int32_t reeval_all;      // 1: every slot is re-evaluated after a switch (DGS_REEVAL_ALL)
@@ -99,11 +99,13 @@ struct Workspace {
     int32_t* sl_chunk;  // edges among slots 32c .. 32c + 31 (written with sl_edge)
     int32_t* ctl_slot;  // controller: slot of each edge position (priority order)
     // greedy start
-    unsigned long long* g_row;  // best free job per agent   (biased value, ~j)
+    unsigned long long* g_row;  // round form: best free job per agent (biased value, ~j)
     unsigned long long* g_col;  // round form: best free agent per job (biased value, ~i);
                                 // deferred acceptance: the key (biased value, ~i) of the job's holder
     uint8_t* free_a; uint8_t* free_j;
-    unsigned long long* g_list;  // deferred acceptance: per agent, 4 slots: the 2nd-4th jobs of its last scan
+    uint32_t* g_bound;  // deferred acceptance: per agent and tile of 2^bound_shift jobs, a bound on its best
+                        // biased benefit there (bound_tiles entries per agent)
+    int32_t bound_shift, bound_tiles;
     int32_t exact_keys;  // 1: never use the packed 32-bit keys (test knob)
     int32_t row_owner_eval;  // 1: full evaluations by row owners (A-transpose form)
     DeviceState* st;
@@ -223,6 +225,22 @@ enum : int32_t {
     kPtCtlColourRounds, kPtCtlColourWalks, kPtCtlColourEdges, kPtCount
 };
 
+// Width of the greedy start's tiles.  64 jobs, the finest that half a warp
+// reads in one load, for a single solve.  An instance of a batched or served
+// solve has at most 16 tiles (64 jobs up to n = 1024, then doubling), so that
+// the table takes at most 64 n bytes of its workspace; a look then reads up to
+// n / 16 jobs.
+constexpr int32_t kBoundShift = 6;
+constexpr int32_t kInstanceBoundTiles = 16;
+__host__ __device__ __forceinline__ int32_t bound_tiles(int32_t n, int32_t shift) {
+    return (n + (1 << shift) - 1) >> shift;
+}
+__host__ __device__ __forceinline__ int32_t instance_bound_shift(int32_t n) {
+    int32_t s = kBoundShift;
+    while (bound_tiles(n, s) > kInstanceBoundTiles) ++s;
+    return s;
+}
+
 // ------------------------------------------------------------- key packing
 // A candidate (gain > 0, index) packs into 64 bits so that unsigned max picks
 // the larger gain and, among equal gains, the LOWER index.
@@ -321,17 +339,19 @@ __device__ __forceinline__ bool grid_barrier(DeviceState* st) {
 
 // ------------------------------------------------------ host-side launchers
 // Each returns the launch error (cudaSuccess on success).
+// Pass 1: the transposed copy and the range check alone; with the bounds of
+// deferred acceptance, over the rows of tile rows [row_tile0, row_tile1) (64
+// rows each); or with the row and column keys of the locally-dominant rounds.
 cudaError_t launch_greedy_pass1(const Workspace& w, cudaStream_t s);
+cudaError_t launch_greedy_pass1_bounds(const Workspace& w, int32_t row_tile0, int32_t row_tile1, cudaStream_t s);
+cudaError_t launch_greedy_pass1_rounds(const Workspace& w, cudaStream_t s);
 cudaError_t launch_greedy_round(const Workspace& w, cudaStream_t s);
-// The greedy start by deferred acceptance (pass 1 must have run without
-// column keys, g_col zero); then the assignment is read off the jobs'
-// holders.  Returns an error (nothing launched) when the launch is refused
-// or DGS_GREEDY_ROUNDS=1; the caller then runs pass 1 with column keys and
-// the locally-dominant rounds (launch_greedy_round).
+// The greedy start by deferred acceptance (pass 1 with bounds must have run,
+// g_col zero); then the assignment is read off the jobs' holders.  Returns an
+// error (nothing launched) when the launch is refused or DGS_GREEDY_ROUNDS=1;
+// the caller then runs the rounds' pass 1 and the locally-dominant rounds
+// (launch_greedy_round).
 cudaError_t launch_greedy_da(const Workspace& w, cudaStream_t s);
-// Pass 1 with (cols = 1) or without (cols = 0) the column keys g_col that the
-// locally-dominant rounds need.
-cudaError_t launch_greedy_pass1_cols(const Workspace& w, int32_t cols, cudaStream_t s);
 cudaError_t launch_range_check(const Workspace& w, cudaStream_t s);
 cudaError_t launch_start_from_tau(const Workspace& w, const int32_t* user_tau, int32_t mode, uint8_t* seen,
                                   cudaStream_t s);
@@ -450,14 +470,16 @@ bool device_writable(const void* p, void** alias);
 // grids of the persistent and grid-stride kernels are multiples of it).
 int32_t device_sms();
 
+constexpr int kSmemSlots = 24;
+
 // Raise a kernel's dynamic shared memory limit once per device (slot = one
 // small integer per kernel).
 inline cudaError_t ensure_smem_limit(const void* func, int slot, size_t bytes) {
-    static int done[16][64] = {};
+    static int done[kSmemSlots][64] = {};
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= 64 || slot < 0 || slot >= 16) return cudaErrorInvalidValue;
+    if (dev < 0 || dev >= 64 || slot < 0 || slot >= kSmemSlots) return cudaErrorInvalidValue;
     if (done[slot][dev] >= (int)bytes) return cudaSuccess;
     e = cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (e == cudaSuccess) done[slot][dev] = (int)bytes;

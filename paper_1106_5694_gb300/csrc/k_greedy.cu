@@ -2,17 +2,19 @@
 // greedy: repeatedly take the largest remaining benefit, ties to the lowest
 // agent, then the lowest job).
 //
-// Parallel form: locally-dominant rounds.  Under the strict total order on
-// pairs (benefit desc, agent asc, job asc), every free agent finds its best
-// free job and every free job its best free agent; mutually-best pairs are
-// matched.  The globally largest remaining pair is always mutually best and
-// the matched pairs are disjoint, so the rounds produce exactly the
+// Parallel form: deferred acceptance (below), from bounds on the best benefit
+// of each agent in each tile of jobs.  Fallback (a refused launch, or the
+// DGS_GREEDY_ROUNDS=1 knob): locally-dominant rounds.  Under the strict total
+// order on pairs (benefit desc, agent asc, job asc), every free agent finds
+// its best free job and every free job its best free agent; mutually-best
+// pairs are matched.  The globally largest remaining pair is always mutually
+// best and the matched pairs are disjoint, so the rounds produce exactly the
 // sequential global-greedy assignment.
 //
 // Pass 1 reads a once in 64x64 tiles and, in the same pass, writes the
-// transposed copy at (used later for column scans), checks |a| < 2^29 and
-// computes every agent's and job's best pair.  Later rounds rescan only the
-// agents (rows of a) and jobs (rows of at) whose best partner was taken.
+// transposed copy at, checks |a| < 2^29 and computes what the greedy start
+// that follows needs: each agent's best benefit in every tile of jobs, or
+// (rounds) every agent's and job's best pair.
 #include <cstdlib>
 
 #include "dgs_internal.cuh"
@@ -22,14 +24,17 @@ namespace {
 
 constexpr int kT = 64;  // tile edge
 
+// What pass 1 computes beside the transposed copy and the range check.
+enum : int { kPass1Plain = 0, kPass1Bounds = 1, kPass1Rounds = 2 };
+
 // a_src (batched instances only): the caller's matrix with row pitch n when w.a
 // is the workspace's pitched copy still to be filled; this pass reads a_src
 // and writes the copy as it goes.  Null: w.a is read.
+template <int kMode>
 __device__ __forceinline__ void greedy_pass1_body(const Workspace& w, int32_t tiles_x, int32_t tiles_total,
-                                                  int32_t bid, int32_t nblk, const int32_t* a_src = nullptr,
-                                                  bool cols = true) {
+                                                  int32_t bid, int32_t nblk, const int32_t* a_src = nullptr) {
     __shared__ int32_t s[kT][kT + 1];
-    __shared__ unsigned long long colpart[4][kT];
+    __shared__ unsigned long long colpart[kMode == kPass1Rounds ? 4 : 1][kT];
     const int32_t n = w.n;
     const int t = threadIdx.x;
     const int lane16 = t & 15;
@@ -58,6 +63,7 @@ __device__ __forceinline__ void greedy_pass1_body(const Workspace& w, int32_t ti
             s[r][c + 0] = v.x; s[r][c + 1] = v.y; s[r][c + 2] = v.z; s[r][c + 3] = v.w;
             // row best over this tile's 4 columns of this thread
             unsigned long long best = 0;
+            uint32_t top = 0;
             const int32_t vals[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
@@ -65,16 +71,27 @@ __device__ __forceinline__ void greedy_pass1_body(const Workspace& w, int32_t ti
                     const int32_t x = vals[e];
                     bad |= (x >= kBenefitLimit) || (x <= -kBenefitLimit);
                     amax = max(amax, x == INT32_MIN ? INT32_MAX : abs(x));
-                    best = umax64(best, pack_benefit(x, (uint32_t)(j + e)));
+                    if (kMode == kPass1Rounds) best = umax64(best, pack_benefit(x, (uint32_t)(j + e)));
+                    if (kMode == kPass1Bounds) top = max(top, (uint32_t)(x + kBenefitLimit));
                 }
             }
+            if (kMode == kPass1Rounds) {
 #pragma unroll
-            for (int off = 8; off > 0; off >>= 1) best = umax64(best, __shfl_xor_sync(0xffffffffu, best, off));
-            if (lane16 == 0 && i < n && best != 0) atomicMax(&w.g_row[i], best);
+                for (int off = 8; off > 0; off >>= 1) best = umax64(best, __shfl_xor_sync(0xffffffffu, best, off));
+                if (lane16 == 0 && i < n && best != 0) atomicMax(&w.g_row[i], best);
+            } else if (kMode == kPass1Bounds) {
+#pragma unroll
+                for (int off = 8; off > 0; off >>= 1) top = max(top, __shfl_xor_sync(0xffffffffu, top, off));
+                if (lane16 == 0 && i < n) {
+                    uint32_t* ub = w.g_bound + (size_t)i * w.bound_tiles + (J0 >> w.bound_shift);
+                    if (w.bound_shift == kBoundShift) *ub = top;
+                    else atomicMax(ub, top);
+                }
+            }
         }
         __syncthreads();
         // column best: thread (group g = t/64, column c = t%64) scans 16 rows
-        if (cols) {
+        if (kMode == kPass1Rounds) {
             const int c = t & 63, g = t >> 6;
             const int32_t j = J0 + c;
             unsigned long long best = 0;
@@ -100,7 +117,7 @@ __device__ __forceinline__ void greedy_pass1_body(const Workspace& w, int32_t ti
             }
         }
         __syncthreads();
-        if (cols && t < kT) {
+        if (kMode == kPass1Rounds && t < kT) {
             const int32_t j = J0 + t;
             unsigned long long best = umax64(umax64(colpart[0][t], colpart[1][t]), umax64(colpart[2][t], colpart[3][t]));
             if (j < n && best != 0) atomicMax(&w.g_col[j], best);
@@ -117,9 +134,10 @@ __device__ __forceinline__ void greedy_pass1_body(const Workspace& w, int32_t ti
 }
 
 // tiles tile0 .. tiles_total - 1 (row-major: a band of whole tile rows)
+template <int kMode>
 __global__ void __launch_bounds__(256) greedy_pass1_kernel(Workspace w, int32_t tiles_x, int32_t tiles_total,
-                                                           int32_t cols, int32_t tile0) {
-    greedy_pass1_body(w, tiles_x, tiles_total, tile0 + blockIdx.x, gridDim.x, nullptr, cols != 0);
+                                                           int32_t tile0) {
+    greedy_pass1_body<kMode>(w, tiles_x, tiles_total, tile0 + blockIdx.x, gridDim.x);
 }
 
 // Match every mutually-best (agent, job) pair.
@@ -204,264 +222,361 @@ __global__ void __launch_bounds__(256) greedy_rescan_kernel(Workspace w, const i
 // Form: g_col[j] holds the key (biased benefit, ~agent) of the job's holder
 // and only grows (64-bit atomicMax).  Agent i beats the holder of job j iff
 // its own key (a[i][j] biased, ~i) is larger.  A free agent proposes to its
-// best job among those whose holder it beats; a proposal that raises the
-// key displaces the holder.  The first proposal of every agent is its best
-// job overall, found by pass 1 (g_row).  A later proposal takes the first
-// job of the agent's list that it still beats; the list (g_list, three
-// keys) holds the second to fourth jobs of the agent's last scan.  Holders'
-// keys only grow, so every job ranked above a list entry and left out of
-// the list was already lost at the scan and is lost still: the first list
-// entry the agent beats is its best job.  With no such entry the agent
-// rescans its row of a against the holders' keys (a stale key is lower and
-// only admits a job whose atomicMax then fails) and keeps the top four.  A
-// failed proposal tries the list, else rescans.  A group of threads takes
-// the next agent from a global counter and follows the chain of
-// displacements: the agent it displaced proposes next, by the same group,
-// until a proposal lands on a job nobody held.  Every free agent is thus in
-// exactly one group's hands, no group waits for another, and the launch
-// ends when the counter is exhausted and every chain has ended.
-constexpr int kDaThreads = 1024;
-constexpr uint64_t kDaTimeoutNs = 16000000000ull;  // bound on one group's work (internal error beyond)
-constexpr int kDaList = 3;                         // list entries per agent (g_list has 4 slots)
+// best job among those whose holder it beats; a proposal that raises the key
+// displaces the holder, who proposes next.  A failed proposal looks again.
+//
+// Bounds: g_bound[i][t] is an upper bound on the biased benefit of agent i's
+// best job in tile t among those whose holder it beats (0: none).  Pass 1
+// sets it to the tile's maximum.  Holders' keys only grow, so the jobs an
+// agent beats only become fewer, and the maximum that a look at the tile
+// finds (with holders' keys that may be stale, that is lower) stays a bound
+// for good: it is written back, and any value ever stored is valid, so the
+// bounds need no ordering between the threads that follow one agent over
+// time.  A proposal takes the tiles in the order of their bounds (ties: the
+// lower tile, which has the lower jobs) and reads their benefits and holders'
+// keys until no other tile's bound can beat the best job found (a larger
+// value, or the same value in a lower tile).
+//
+// What bounds it: round trips to memory, one chain of displacements after the
+// other (bounds, tiles, atomic), and the instructions of the looks; not bytes.
+// A look of a warp reads its four best bounds' tiles at once (3 KB).  An agent
+// displaced late has to look at most of its tiles (the good jobs are taken), so
+// a chain is followed by a group of four warps, each with its share of the
+// tiles: a proposal then takes about 1.5 microseconds when one look is enough
+// and 5 when all are needed.  Measured (single solve, greedy start after pass
+// 1), against reading an agent's whole row and every holder's key per proposal
+// with the four best jobs kept for later proposals: peer-shaped n = 10000 0.48
+// -> 0.24 ms, n = 4096 0.167 -> 0.117, uniform n = 20000 0.47 -> 0.17.  One
+// warp per chain 0.30 ms at n = 10000, two 0.26, eight 0.50; eight tiles per
+// look 0.29 (fewer CTAs fit); prefetching an agent's remaining tiles into L2:
+// no change.  A batched launch has chains enough to fill the chip, so there
+// one warp follows a chain (1024 peer-shaped instances, n in [64, 4096]: 22.4
+// -> 4.7 ms).
+//
+// A group's first agent is its number in the grid, the next ones come from a
+// counter; it follows the chain of displacements that starts with each: the
+// agent it displaced proposes next, until a proposal lands on a job nobody
+// held.  Every free agent is thus in exactly one group's hands, no group waits
+// for another, and the launch ends when every chain has ended.
+constexpr int kDaThreads = 256;
+constexpr int kDaPerSm = 4;
+constexpr int kDaGroup = 4;  // warps that follow one chain
+constexpr int kDaPicks = 4;  // 64-job tiles that one look of a warp reads
+constexpr int kDaWarps = kDaThreads / 32;
+constexpr uint64_t kDaTimeoutNs = 16000000000ull;  // bound on one warp's work (internal error beyond)
 
-template <int kGroup>
-__device__ __forceinline__ void group_bar(int grp) {
-    if (kGroup == 32) __syncwarp();
-    else asm volatile("bar.sync %0, %1;" ::"r"(grp + 1), "r"(kGroup) : "memory");
-}
-
-// 64-bit atomic max with acquire-release order at GPU scope: the proposal
-// publishes the proposer's list, and the displacer then reads the displaced
-// agent's list.
+// 64-bit atomic max with acquire-release order at GPU scope.
 __device__ __forceinline__ unsigned long long atomic_max_acq_rel(unsigned long long* p, unsigned long long v) {
     unsigned long long old;
     asm volatile("atom.acq_rel.gpu.global.max.u64 %0, [%1], %2;" : "=l"(old) : "l"(p), "l"(v) : "memory");
     return old;
 }
 
-// Insert key k into the descending t[0..3] (keys are distinct: the low word
-// is the job).
-__device__ __forceinline__ void top4_insert(unsigned long long (&t)[4], unsigned long long k) {
-    if (k <= t[3]) return;
-    t[3] = k;
-    if (t[3] > t[2]) { const unsigned long long x = t[2]; t[2] = t[3]; t[3] = x; }
-    if (t[2] > t[1]) { const unsigned long long x = t[1]; t[1] = t[2]; t[2] = x; }
-    if (t[1] > t[0]) { const unsigned long long x = t[0]; t[0] = t[1]; t[1] = x; }
+__device__ __forceinline__ unsigned long long pack_key(uint32_t hi, uint32_t lo) {
+    return ((unsigned long long)hi << 32) | lo;
 }
 
-// The four largest keys of the warp, in every lane's out[0..3].
-__device__ __forceinline__ void warp_top4(unsigned long long (&t)[4], unsigned long long (&out)[4]) {
+// What a proposal reads of an instance.
+struct DaView {
+    const int32_t* a;
+    unsigned long long* keys;
+    uint32_t* bounds;
+    int32_t n, lda, tiles, shift;
+};
+__device__ __forceinline__ DaView da_view(const Workspace& w) {
+    return DaView{w.a, w.g_col, w.g_bound, w.n, w.lda, w.bound_tiles, w.bound_shift};
+}
+
+// Barrier of a group of kGroup warps (named barriers 1.., one per group).
+template <int kGroup>
+__device__ __forceinline__ void group_bar(int grp) {
+    if (kGroup == 1) __syncwarp();
+    else asm volatile("bar.sync %0, %1;" ::"r"(grp + 1), "r"(kGroup * 32) : "memory");
+}
+
+// What the warps of a group exchange: the best job found and the best bound
+// not looked at yet, as (value, ~job) and (value, ~tile), by turns in two
+// buffers; the outcome of the proposal.
+template <int kGroup>
+struct DaShared {
+    unsigned long long best[2][kGroup], left[2][kGroup];
+    int32_t out;
+};
+
+// The value of this lane's best job of the four in x among those whose holder
+// (keys h0, h1) agent i beats; 0 when there is none.  Jobs from column c on, of
+// which those below n exist.
+__device__ __forceinline__ uint32_t da_best4(const int4& x, const ulonglong2& h0, const ulonglong2& h1, int32_t c,
+                                             int32_t n, uint32_t me_lo) {
+    const uint32_t b0 = (uint32_t)(x.x + kBenefitLimit), b1 = (uint32_t)(x.y + kBenefitLimit);
+    const uint32_t b2 = (uint32_t)(x.z + kBenefitLimit), b3 = (uint32_t)(x.w + kBenefitLimit);
+    uint32_t r = pack_key(b0, me_lo) > h0.x ? b0 : 0u;
+    if (pack_key(b1, me_lo) > h0.y && c + 1 < n) r = max(r, b1);
+    if (pack_key(b2, me_lo) > h1.x && c + 2 < n) r = max(r, b2);
+    if (pack_key(b3, me_lo) > h1.y && c + 3 < n) r = max(r, b3);
+    return r;
+}
+// The lowest of those jobs whose value is r.
+__device__ __forceinline__ int32_t da_column4(const int4& x, const ulonglong2& h0, const ulonglong2& h1, int32_t c,
+                                              uint32_t r, uint32_t me_lo) {
+    if ((uint32_t)(x.x + kBenefitLimit) == r && pack_key(r, me_lo) > h0.x) return c;
+    if ((uint32_t)(x.y + kBenefitLimit) == r && pack_key(r, me_lo) > h0.y) return c + 1;
+    if ((uint32_t)(x.z + kBenefitLimit) == r && pack_key(r, me_lo) > h1.x) return c + 2;
+    return c + 3;
+}
+
+// One look of a warp at tiles of 64 jobs (see da_propose): the kDaPicks best
+// bounds, at most one of each lane, half a warp per tile.  mv, mt: this
+// lane's largest bound left and its tile; bv, bt: value and tile of the best
+// job known.  Returns the best job found, (value, ~job), 0 when none; `mine`:
+// this lane's tile was one of them and `found` is its new bound.
+__device__ __forceinline__ unsigned long long da_look64(const DaView& d, const int32_t* row, uint32_t me_lo, uint32_t mv,
+                                                        int32_t mt, uint32_t bv, int32_t bt, bool& mine,
+                                                        uint32_t& found) {
+    constexpr uint32_t kAll = 0xffffffffu;
+    constexpr int32_t kNone = 0x7fffffff;
+    const int lane = threadIdx.x & 31, half = lane >> 4;
+    int32_t tile[kDaPicks / 2];
+    uint32_t left = (mv > bv || (mv == bv && mt < bt)) ? mv : 0u;
+    int turn = -1;
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-        unsigned long long m = t[0];
+    for (int k = 0; k < kDaPicks; ++k) {
+        const uint32_t v = __reduce_max_sync(kAll, left);
+        const int32_t t = (int32_t)__reduce_min_sync(kAll, left == v && v != 0u ? (uint32_t)mt : (uint32_t)kNone);
+        if (mt == t && v != 0u) {
+            left = 0u;
+            turn = k;
+        }
+        if ((k & 1) == 0) tile[k / 2] = t;
+        else tile[k / 2] = half ? t : tile[k / 2];
+    }
+    int4 x[kDaPicks / 2];
+    ulonglong2 h0[kDaPicks / 2], h1[kDaPicks / 2];
+    int32_t c[kDaPicks / 2];
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) m = umax64(m, __shfl_xor_sync(0xffffffffu, m, off));
-        out[r] = m;
-        if (m != 0 && t[0] == m) {  // the owner drops it
-            t[0] = t[1];
-            t[1] = t[2];
-            t[2] = t[3];
-            t[3] = 0;
+    for (int q = 0; q < kDaPicks / 2; ++q) {
+        c[q] = tile[q] == kNone ? d.n : tile[q] * kT + (lane & 15) * 4;
+        if (c[q] < d.n) {
+            x[q] = __ldg(reinterpret_cast<const int4*>(row + c[q]));
+            h0[q] = __ldcg(reinterpret_cast<const ulonglong2*>(d.keys + c[q]));
+            h1[q] = __ldcg(reinterpret_cast<const ulonglong2*>(d.keys + c[q] + 2));
         }
     }
+    uint32_t lv[kDaPicks / 2], top = 0u;
+#pragma unroll
+    for (int q = 0; q < kDaPicks / 2; ++q) {
+        lv[q] = c[q] < d.n ? da_best4(x[q], h0[q], h1[q], c[q], d.n, me_lo) : 0u;
+        top = max(top, lv[q]);
+    }
+    const uint32_t r = __reduce_max_sync(kAll, top);
+    uint32_t lc = (uint32_t)kNone;
+    if (top == r && r != 0u) {  // (few lanes)
+#pragma unroll
+        for (int q = 0; q < kDaPicks / 2; ++q)
+            if (lv[q] == r) lc = min(lc, (uint32_t)da_column4(x[q], h0[q], h1[q], c[q], r, me_lo));
+    }
+    const uint32_t rc = __reduce_min_sync(kAll, lc);
+    // each tile's maximum, to the lane whose tile it is
+#pragma unroll
+    for (int q = 0; q < kDaPicks / 2; ++q) {
+#pragma unroll
+        for (int off = 8; off > 0; off >>= 1) lv[q] = max(lv[q], __shfl_xor_sync(kAll, lv[q], off));
+        const uint32_t m = __shfl_sync(kAll, lv[q], (turn & 1) * 16);
+        if ((turn >> 1) == q) found = m;
+    }
+    mine = turn >= 0;
+    return r ? ((unsigned long long)r << 32) | ~rc : 0ull;
 }
 
-// One proposal of agent i (and its retries after failed ones), by the whole
-// group.  first: i has not proposed yet (its best job overall, from pass 1).
-// s_red: 4 keys per warp of the block; s_top: 4 keys per group.  Returns the
-// displaced agent, -1 when the job was free, -2 on an error.
+// The same at wider tiles (2^shift jobs, shift > kBoundShift; instances of a
+// batch): one tile, the warp's best bound.
+__device__ __forceinline__ unsigned long long da_look_wide(const DaView& d, const int32_t* row, uint32_t me_lo,
+                                                           uint32_t mv, int32_t mt, uint32_t bv, int32_t bt, bool& mine,
+                                                           uint32_t& found) {
+    constexpr uint32_t kAll = 0xffffffffu;
+    constexpr int32_t kNone = 0x7fffffff;
+    const int lane = threadIdx.x & 31;
+    const uint32_t left = (mv > bv || (mv == bv && mt < bt)) ? mv : 0u;
+    const uint32_t v = __reduce_max_sync(kAll, left);
+    mine = false;
+    if (v == 0u) return 0ull;
+    const int32_t t = (int32_t)__reduce_min_sync(kAll, left == v ? (uint32_t)mt : (uint32_t)kNone);
+    const int32_t end = min(d.n, (t + 1) << d.shift);
+    uint32_t top = 0u, lc = (uint32_t)kNone;
+#pragma unroll 2
+    for (int32_t c = (t << d.shift) + lane * 4; c < end; c += 128) {
+        const int4 x = __ldg(reinterpret_cast<const int4*>(row + c));
+        const ulonglong2 h0 = __ldcg(reinterpret_cast<const ulonglong2*>(d.keys + c));
+        const ulonglong2 h1 = __ldcg(reinterpret_cast<const ulonglong2*>(d.keys + c + 2));
+        const uint32_t b = da_best4(x, h0, h1, c, d.n, me_lo);
+        if (b > top) {
+            top = b;
+            lc = (uint32_t)da_column4(x, h0, h1, c, b, me_lo);
+        }
+    }
+    const uint32_t r = __reduce_max_sync(kAll, top);
+    const uint32_t rc = __reduce_min_sync(kAll, top == r ? lc : (uint32_t)kNone);
+    mine = mt == t;
+    found = r;
+    return r ? ((unsigned long long)r << 32) | ~rc : 0ull;
+}
+
+// One proposal of agent i (and its retries after failed ones) by a group of
+// kGroup warps.  Tile t belongs to lane (t / kGroup) % 32 of warp t % kGroup.
+// s_b: the group's copy of the agent's bounds (each thread reads and writes
+// only its own tiles' entries).  Returns the displaced agent, -1 when the job
+// was free, -2 on an error.
 template <int kGroup>
-__device__ __forceinline__ int32_t da_propose(const Workspace& w, int32_t i, bool first, int grp, int gt,
-                                              unsigned long long* s_red, unsigned long long* s_top,
-                                              int32_t* s_out, int32_t& scans) {
-    constexpr int kWarps = kGroup / 32;
-    constexpr unsigned long long kHi = 0xFFFFFFFF00000000ull;
-    DeviceState* st = w.st;
-    const int32_t n = w.n;
-    const int glane = gt & 31, gwarp = gt >> 5;
-    const int32_t* row = w.a + (size_t)i * w.lda;
+__device__ __forceinline__ int32_t da_propose(const DaView& d, int32_t i, uint32_t* s_b, DaShared<kGroup>& sh, int grp,
+                                              int gw, int32_t& looks) {
+    constexpr uint32_t kAll = 0xffffffffu;
+    constexpr int32_t kNone = 0x7fffffff;
+    const int lane = threadIdx.x & 31;
+    const int32_t t_first = lane * kGroup + gw;
     const uint32_t me_lo = ~(uint32_t)i;
-    unsigned long long* list = w.g_list + 4 * (size_t)i;
-    for (int32_t attempt = 0;; ++attempt) {
-        unsigned long long best = 0;
-        if (gt == 0) {
-            int32_t need_scan = 0;
-            if (attempt == 0 && first) {
-                best = w.g_row[i];
-            } else {  // the first list entry whose holder this agent beats
-                unsigned long long l[kDaList], h[kDaList];
-#pragma unroll
-                for (int m = 0; m < kDaList; ++m) l[m] = list[m];
-#pragma unroll
-                for (int m = 0; m < kDaList; ++m) h[m] = l[m] ? __ldcg(w.g_col + key_index(l[m])) : ~0ull;
-                int32_t used = kDaList;
-#pragma unroll
-                for (int m = kDaList - 1; m >= 0; --m)
-                    if (l[m] != 0 && ((l[m] & kHi) | me_lo) > h[m]) {
-                        best = l[m];
-                        used = m + 1;
-                    }
-                if (best == 0) need_scan = 1;
-#pragma unroll
-                for (int m = 0; m < kDaList; ++m)
-                    if (m < used) list[m] = 0ull;  // consumed
+    uint32_t* bounds = d.bounds + (size_t)i * d.tiles;
+    const int32_t* row = d.a + (size_t)i * d.lda;
+    int turn = 0;
+    for (int32_t attempt = 0; attempt <= 2 * d.n + 2; ++attempt) {
+        uint32_t mv = 0u;    // this lane's largest bound not looked at yet
+        int32_t mt = kNone;  // and its (lowest) tile
+        for (int32_t t = t_first; t < d.tiles; t += 32 * kGroup) {
+            const uint32_t b = __ldcg(bounds + t);
+            s_b[t] = b;
+            if (b > mv) {
+                mv = b;
+                mt = t;
             }
-            *s_out = need_scan;
         }
-        group_bar<kGroup>(grp);
-        const bool need_scan = *s_out != 0;
-        group_bar<kGroup>(grp);
-        if (need_scan) {
-            // the four best jobs whose holders this agent beats
-            ++scans;
-            unsigned long long t[4] = {0ull, 0ull, 0ull, 0ull};
-            // the whole row is requested into L2 at once (prefetches hold no
-            // registers), so that the batches below wait for L2, not DRAM
-            for (int32_t c = gt * 32; c < n; c += 32 * kGroup)
-                asm volatile("prefetch.global.L2 [%0];" ::"l"(row + c));
-            constexpr int kB = 2;  // 16-byte loads of the row (and 32 bytes of holder keys each) in flight
-            for (int32_t c0 = gt * 4; c0 < n; c0 += 4 * kGroup * kB) {
-                int4 v[kB];
-                ulonglong2 h[kB][2];
-#pragma unroll
-                for (int b = 0; b < kB; ++b) {
-                    const int32_t c = c0 + b * 4 * kGroup;
-                    if (c < n) {
-                        v[b] = __ldcs(reinterpret_cast<const int4*>(row + c));
-                        h[b][0] = __ldcg(reinterpret_cast<const ulonglong2*>(w.g_col + c));
-                        h[b][1] = __ldcg(reinterpret_cast<const ulonglong2*>(w.g_col + c + 2));
-                    }
-                }
-#pragma unroll
-                for (int b = 0; b < kB; ++b) {
-                    const int32_t c = c0 + b * 4 * kGroup;
-                    if (c >= n) continue;
-                    const int32_t vals[4] = {v[b].x, v[b].y, v[b].z, v[b].w};
-                    const unsigned long long hs[4] = {h[b][0].x, h[b][0].y, h[b][1].x, h[b][1].y};
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const unsigned long long x = (uint32_t)(vals[e] + kBenefitLimit);
-                        if (c + e < n && ((x << 32) | me_lo) > hs[e])
-                            top4_insert(t, (x << 32) | (unsigned long long)(~(uint32_t)(c + e)));
+        uint32_t bv = 0u;  // the best job found by the group: value, column
+        int32_t bc = kNone;
+        for (;;) {
+            bool mine;
+            uint32_t found = 0u;
+            const int32_t bt = bv == 0u ? kNone : bc >> d.shift;
+            unsigned long long best = d.shift == kBoundShift
+                                          ? da_look64(d, row, me_lo, mv, mt, bv, bt, mine, found)
+                                          : da_look_wide(d, row, me_lo, mv, mt, bv, bt, mine, found);
+            looks += __popc(__ballot_sync(kAll, mine));
+            // the bounds found, for good; not looked at again in this attempt
+            if (mine) {
+                if (found != mv) __stcg(bounds + mt, found);
+                s_b[mt] = 0u;
+                mv = 0u;
+                mt = kNone;
+                for (int32_t t = t_first; t < d.tiles; t += 32 * kGroup) {
+                    const uint32_t b = s_b[t];
+                    if (b > mv) {
+                        mv = b;
+                        mt = t;
                     }
                 }
             }
-            unsigned long long wt[4];
-            warp_top4(t, wt);
-            if (kWarps == 1) {
-                if (gt == 0) {
-                    best = wt[0];
-#pragma unroll
-                    for (int m = 0; m < kDaList; ++m) list[m] = wt[1 + m];
+            // (value, ~job) and (value, ~tile): larger is better
+            const uint32_t l = __reduce_max_sync(kAll, mv);
+            const uint32_t lt = __reduce_min_sync(kAll, mv == l ? (uint32_t)mt : (uint32_t)kNone);
+            unsigned long long more = ((unsigned long long)l << 32) | ~lt;
+            if (kGroup > 1) {
+                if (lane == 0) {
+                    sh.best[turn][gw] = best;
+                    sh.left[turn][gw] = more;
                 }
-            } else {
-            if (glane == 0) {
+                group_bar<kGroup>(grp);
 #pragma unroll
-                for (int r = 0; r < 4; ++r) s_red[(grp * kWarps + gwarp) * 4 + r] = wt[r];
+                for (int k = 0; k < kGroup; ++k) {
+                    best = umax64(best, sh.best[turn][k]);
+                    more = umax64(more, sh.left[turn][k]);
+                }
+                turn ^= 1;
             }
+            if ((uint32_t)(best >> 32) > bv || ((uint32_t)(best >> 32) == bv && (int32_t)(~(uint32_t)best) < bc)) {
+                bv = (uint32_t)(best >> 32);
+                bc = (int32_t)(~(uint32_t)best);
+            }
+            const uint32_t v = (uint32_t)(more >> 32);
+            if (v == 0u || bv > v || (bv == v && (bc >> d.shift) < (int32_t)(~(uint32_t)more))) break;
+        }
+        // some job always accepts a free agent, and every failed proposal
+        // rules a job out, so an agent needs at most 2 n + 2 attempts
+        if (bv == 0u || bc >= d.n) return -2;
+        int32_t out = -2;
+        if (gw == 0) {
+            const unsigned long long mine = ((unsigned long long)bv << 32) | me_lo;
+            unsigned long long old = 0ull;
+            if (lane == 0) old = atomic_max_acq_rel(d.keys + bc, mine);
+            old = __shfl_sync(kAll, old, 0);
+            out = old < mine ? (old == 0ull ? -1 : key_index(old)) : -3;  // -3: taken meanwhile, look again
+        }
+        if (kGroup > 1) {
+            if (gw == 0 && lane == 0) sh.out = out;
             group_bar<kGroup>(grp);
-            if (gwarp == 0) {  // the group's first warp merges its warps' candidates
-                unsigned long long c4[4] = {0ull, 0ull, 0ull, 0ull};
-                for (int q = glane; q < kWarps * 4; q += 32) top4_insert(c4, s_red[grp * kWarps * 4 + q]);
-                unsigned long long gt4[4];
-                warp_top4(c4, gt4);
-                if (glane == 0) {
-#pragma unroll
-                    for (int r = 0; r < 4; ++r) s_top[grp * 4 + r] = gt4[r];
-                }
-            }
+            out = sh.out;
             group_bar<kGroup>(grp);
-            if (gt == 0) {
-                best = s_top[grp * 4];
-#pragma unroll
-                for (int m = 0; m < kDaList; ++m) list[m] = s_top[grp * 4 + 1 + m];
-            }
-            }
         }
-        if (gt == 0) {
-            int32_t out = -1;
-            const int32_t j = key_index(best);
-            // some job always accepts a free agent, and every failed proposal
-            // or rejected list entry rules a job out, so an agent needs at
-            // most 2 n + 2 attempts
-            if (best == 0 || j < 0 || j >= n || attempt > 2 * n + 2) {
-                st->error = kErrInternal;
-                st->status = kError;
-                out = -2;
-            } else {
-                const unsigned long long mine = (best & kHi) | me_lo;
-                const unsigned long long old = atomic_max_acq_rel(w.g_col + j, mine);
-                if (old < mine) {
-                    out = old == 0 ? -1 : key_index(old);
-                } else {
-                    out = -3;  // the job was taken meanwhile: the list, else a rescan
-                }
-            }
-            *s_out = out;
-        }
-        group_bar<kGroup>(grp);
-        const int32_t out = *s_out;
-        group_bar<kGroup>(grp);
         if (out != -3) return out;
     }
+    return -2;
 }
 
 template <int kGroup>
-__global__ void __launch_bounds__(kDaThreads, 1) greedy_da_kernel(Workspace w) {
-    constexpr int kGroups = kDaThreads / kGroup;
+__global__ void __launch_bounds__(kDaThreads, kDaPerSm) greedy_da_kernel(Workspace w) {
+    extern __shared__ __align__(16) uint32_t s_bounds[];
+    constexpr int kGroups = kDaWarps / kGroup;
+    __shared__ DaShared<kGroup> s_sh[kGroups];
     DeviceState* st = w.st;
-    __shared__ unsigned long long s_red[kDaThreads / 32 * 4];
-    __shared__ unsigned long long s_top[kGroups * 4];
-    __shared__ int32_t s_out[kGroups];
-    __shared__ int32_t s_status;
+    __shared__ int32_t s_status, s_next[kGroups];
     if (threadIdx.x == 0) s_status = *(volatile int32_t*)&st->status;
     __syncthreads();
     if (s_status != kRunning) return;
-    const int32_t n = w.n;
-    const int tid = threadIdx.x, grp = tid / kGroup, gt = tid % kGroup;
-    int32_t scans = 0, longest = 0;
-    bool worked = false;
+    const DaView d = da_view(w);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, grp = warp / kGroup, gw = warp % kGroup;
+    const bool leader = gw == 0 && lane == 0;
+    uint32_t* s_b = s_bounds + (size_t)grp * d.tiles;
+    const int32_t groups = (int32_t)gridDim.x * kGroups;
+    int32_t looks = 0, longest = 0;
     const uint64_t t_start = globaltimer_ns();
-    for (;;) {
-        if (gt == 0) s_out[grp] = atomicAdd(&st->da_next, 1);
-        group_bar<kGroup>(grp);
-        int32_t a = s_out[grp];
-        group_bar<kGroup>(grp);
-        if (a >= n) break;
-        bool first = true;
-        int32_t d, steps = 0;
-        worked = true;
+    // (neighbouring agents on different SMs)
+    int32_t next = grp * (int32_t)gridDim.x + (int32_t)blockIdx.x;
+    while (next < d.n) {
+        int32_t a = next, r, steps = 1;
         // the chain of displacements that starts with agent a
-        while ((d = da_propose<kGroup>(w, a, first, grp, gt, s_red, s_top, &s_out[grp], scans)) >= 0) {
-            a = d;
-            first = false;
+        while ((r = da_propose<kGroup>(d, a, s_b, s_sh[grp], grp, gw, looks)) >= 0) {
+            a = r;
             ++steps;
-            longest = max(longest, steps);
-            if (gt == 0 && globaltimer_ns() - t_start > kDaTimeoutNs) {
-                st->error = kErrWaitTimeout;
-                st->status = kError;
-                s_out[grp] = 1;
-            } else if (gt == 0) {
-                s_out[grp] = 0;
-            }
-            group_bar<kGroup>(grp);
-            const bool late = s_out[grp] != 0;
-            group_bar<kGroup>(grp);
-            if (late) {
-                d = -2;
-                break;
+            if ((steps & 63) == 0) {  // bounded in time
+                if (leader) s_next[grp] = globaltimer_ns() - t_start > kDaTimeoutNs;
+                group_bar<kGroup>(grp);
+                const bool late = s_next[grp] != 0;
+                group_bar<kGroup>(grp);
+                if (late) {
+                    r = -3;
+                    break;
+                }
             }
         }
-        if (d == -2) break;
+        longest = max(longest, steps);
+        if (r < -1) {
+            if (leader) {
+                st->error = r == -3 ? kErrWaitTimeout : kErrInternal;
+                st->status = kError;
+            }
+            break;
+        }
+        if (leader) s_next[grp] = groups + atomicAdd(&st->da_next, 1);
+        group_bar<kGroup>(grp);
+        next = s_next[grp];
+        group_bar<kGroup>(grp);
     }
-    if (gt == 0 && scans) atomicAdd((unsigned long long*)&st->greedy_rescans, (unsigned long long)scans);
-    if (gt == 0 && worked) atomicMax(&st->greedy_rounds, longest + 1);  // proposals along the longest chain
-    if (gt == 0 && w.phase_ns) {  // diagnostics (DGS_PHASE_TIMERS=1)
+    if (lane == 0 && looks) {
+        atomicAdd((unsigned long long*)&st->greedy_rescans, (unsigned long long)looks);
+        atomicMax(&st->greedy_rounds, longest);  // proposals along the longest chain
+    }
+    if (leader && w.phase_ns) {  // diagnostics (DGS_PHASE_TIMERS=1)
         const uint64_t t = globaltimer_ns() - t_start;
         atomicMax(w.phase_ns + kPtDaLastNs, (unsigned long long)t);
         atomicAdd(w.phase_ns + kPtDaSumNs, (unsigned long long)t);
         atomicMax(w.phase_ns + kPtDaChain, (unsigned long long)longest);
-        atomicMax(w.phase_ns + kPtDaGroupScans, (unsigned long long)scans);
+        atomicMax(w.phase_ns + kPtDaGroupScans, (unsigned long long)looks);
     }
 }
 
@@ -525,55 +640,71 @@ __global__ void range_check_kernel(Workspace w) {
 __global__ void __launch_bounds__(256) greedy_pass1_batched_kernel(BatchQueues q) {
     for_each_item(q.inst, q.q0, q.cap, [&](const Instance& in, int32_t bid, int32_t nblk) {
         const int32_t tx = (in.w.n + kT - 1) / kT;
-        greedy_pass1_body(in.w, tx, tx * tx, bid, nblk, in.a_src, false);
+        greedy_pass1_body<kPass1Bounds>(in.w, tx, tx * tx, bid, nblk, in.a_src);
     });
 }
 
 // Deferred acceptance of every instance in kStageGreedy in one launch: the
 // agents of all those instances form one index space (prefix offsets q0 of
 // the kScanGreedyDA scan, which also zeroes q1[0], the shared counter); a
-// group takes the next agent of that space and follows its chain of
-// displacements inside its instance, exactly as greedy_da_kernel does for a
-// single solve.
-template <int kGroup>
-__global__ void __launch_bounds__(kDaThreads, 1) greedy_da_batched_kernel(BatchQueues q) {
-    constexpr int kGroups = kDaThreads / kGroup;
-    __shared__ unsigned long long s_red[kDaThreads / 32 * 4];
-    __shared__ unsigned long long s_top[kGroups * 4];
-    __shared__ int32_t s_out[kGroups];
+// warp takes its first agents of that space by its number, later ones from
+// the counter, and follows each one's chain of displacements inside its
+// instance, exactly as greedy_da_kernel does for a single solve.
+__global__ void __launch_bounds__(kDaThreads, kDaPerSm) greedy_da_batched_kernel(BatchQueues q) {
+    __shared__ uint32_t s_bounds[kDaWarps][kInstanceBoundTiles];
+    __shared__ DaShared<1> s_sh[kDaWarps];
     const int32_t total = q.q0[q.cap];
     if (total <= 0) return;
-    const int tid = threadIdx.x, grp = tid / kGroup, gt = tid % kGroup;
-    int32_t scans = 0, k_last = -1;
-    for (;;) {
-        if (gt == 0) s_out[grp] = atomicAdd(q.q1, 1);
-        group_bar<kGroup>(grp);
-        const int32_t g = s_out[grp];
-        group_bar<kGroup>(grp);
-        if (g >= total) break;
-        int32_t lo = 0, hi = q.cap;  // q0[lo] <= g < q0[hi]
-        while (hi - lo > 1) {
-            const int32_t mid = (lo + hi) >> 1;
-            if (q.q0[mid] <= g) lo = mid;
-            else hi = mid;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t* s_b = s_bounds[warp];
+    const int32_t warps = (int32_t)gridDim.x * kDaWarps;
+    int32_t looks = 0, longest = 0, k_last = -1, first = 0, end = 0;
+    DaView d{};
+    auto flush = [&] {  // looks and chains are counted per instance
+        if (k_last >= 0 && lane == 0 && looks) {
+            DeviceState* st = q.inst[k_last].w.st;
+            atomicAdd((unsigned long long*)&st->greedy_rescans, (unsigned long long)looks);
+            atomicMax(&st->greedy_rounds, longest);
         }
-        const Instance& in = q.inst[lo];
-        if (k_last != lo && k_last >= 0 && gt == 0 && scans)  // rescans are counted per instance
-            atomicAdd((unsigned long long*)&q.inst[k_last].w.st->greedy_rescans, (unsigned long long)scans);
-        if (k_last != lo) scans = 0;
-        k_last = lo;
-        int32_t a = g - q.q0[lo];
-        bool first = true;
-        int32_t d, steps = 1;
-        while ((d = da_propose<kGroup>(in.w, a, first, grp, gt, s_red, s_top, &s_out[grp], scans)) >= 0) {
-            a = d;
-            first = false;
-            ++steps;
+        looks = longest = 0;
+    };
+    const int32_t per = total >= 4 * warps ? 4 : 1;  // agents taken at a time (one look-up of their instance)
+    int32_t chunk = warp * (int32_t)gridDim.x + (int32_t)blockIdx.x;
+    while ((int64_t)chunk * per < total) {
+        const int32_t g_end = min(total, (chunk + 1) * per);
+        for (int32_t g = chunk * per; g < g_end; ++g) {
+            if (g < first || g >= end) {  // another instance: q0[lo] <= g < q0[lo + 1], 32 probes at a time
+                flush();
+                int32_t lo = 0, hi = q.cap;
+                while (hi - lo > 1) {
+                    const int32_t step = (hi - lo + 31) / 32;
+                    const int32_t probe = lo + (lane + 1) * step;
+                    const uint32_t above = __ballot_sync(0xffffffffu, probe >= hi || q.q0[probe] > g);
+                    const int k = __ffs(above) - 1;  // (the last probe is at or past hi)
+                    hi = min(hi, lo + (k + 1) * step);
+                    lo += k * step;
+                }
+                k_last = lo;
+                first = q.q0[lo];
+                end = q.q0[lo + 1];
+                d = da_view(q.inst[lo].w);
+            }
+            int32_t a = g - first, r, steps = 1;
+            while ((r = da_propose<1>(d, a, s_b, s_sh[warp], warp, 0, looks)) >= 0) {
+                a = r;
+                ++steps;
+            }
+            longest = max(longest, steps);
+            if (r == -2 && lane == 0) {
+                DeviceState* st = q.inst[k_last].w.st;
+                st->error = kErrInternal;
+                st->status = kError;
+            }
         }
-        if (gt == 0 && d == -1) atomicMax(&in.w.st->greedy_rounds, steps);
+        if (lane == 0) chunk = warps + atomicAdd(q.q1, 1);
+        chunk = __shfl_sync(0xffffffffu, chunk, 0);
     }
-    if (k_last >= 0 && gt == 0 && scans)
-        atomicAdd((unsigned long long*)&q.inst[k_last].w.st->greedy_rescans, (unsigned long long)scans);
+    flush();
 }
 
 // The assignment of every instance in kStageGreedy from its jobs' holders
@@ -609,22 +740,28 @@ cudaError_t launch_range_check(const Workspace& w, cudaStream_t s) {
 
 // Pass 1 over the rows of tile rows [row_tile0, row_tile1) (64 rows each):
 // the bands of a matrix that arrives in pieces can be processed as they land.
-cudaError_t launch_greedy_pass1_rows(const Workspace& w, int32_t cols, int32_t row_tile0, int32_t row_tile1,
+cudaError_t launch_greedy_pass1_rows(const Workspace& w, int32_t mode, int32_t row_tile0, int32_t row_tile1,
                                      cudaStream_t s) {
     const int32_t tx = (w.n + kT - 1) / kT;
     const int32_t t0 = row_tile0 * tx, t1 = (row_tile1 < tx ? row_tile1 : tx) * tx;
     const int32_t count = t1 - t0;
     if (count <= 0) return cudaSuccess;
     const int32_t grid = count < dgs::device_sms() * 8 ? count : dgs::device_sms() * 8;
-    greedy_pass1_kernel<<<grid, 256, 0, s>>>(w, tx, t1, cols, t0);
+    if (mode == kPass1Bounds) greedy_pass1_kernel<kPass1Bounds><<<grid, 256, 0, s>>>(w, tx, t1, t0);
+    else if (mode == kPass1Rounds) greedy_pass1_kernel<kPass1Rounds><<<grid, 256, 0, s>>>(w, tx, t1, t0);
+    else greedy_pass1_kernel<kPass1Plain><<<grid, 256, 0, s>>>(w, tx, t1, t0);
     return cudaGetLastError();
 }
 
-cudaError_t launch_greedy_pass1_cols(const Workspace& w, int32_t cols, cudaStream_t s) {
-    return launch_greedy_pass1_rows(w, cols, 0, (w.n + kT - 1) / kT, s);
+cudaError_t launch_greedy_pass1_bounds(const Workspace& w, int32_t row_tile0, int32_t row_tile1, cudaStream_t s) {
+    return launch_greedy_pass1_rows(w, kPass1Bounds, row_tile0, row_tile1, s);
 }
-
-cudaError_t launch_greedy_pass1(const Workspace& w, cudaStream_t s) { return launch_greedy_pass1_cols(w, 1, s); }
+cudaError_t launch_greedy_pass1_rounds(const Workspace& w, cudaStream_t s) {
+    return launch_greedy_pass1_rows(w, kPass1Rounds, 0, (w.n + kT - 1) / kT, s);
+}
+cudaError_t launch_greedy_pass1(const Workspace& w, cudaStream_t s) {
+    return launch_greedy_pass1_rows(w, kPass1Plain, 0, (w.n + kT - 1) / kT, s);
+}
 
 cudaError_t launch_greedy_loop_cond(const Workspace& w, unsigned long long handle, cudaStream_t s) {
     greedy_loop_cond_kernel<<<1, 1, 0, s>>>(w, handle);
@@ -647,27 +784,13 @@ cudaError_t launch_b_pass1(const BatchQueues& q, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-// Threads per proposal of the deferred acceptance (DGS_DA_GROUP = 32, 128,
-// 256 or 512; results do not depend on it).  Groups of more than one warp
-// synchronise on named barriers 1..15, one per group of the block.
-int32_t da_group_env() {
-    static const int32_t v = [] {
-        const char* e = std::getenv("DGS_DA_GROUP");
-        const int32_t x = e ? std::atoi(e) : 256;
-        return (x == 32 || x == 128 || x == 512) ? x : 256;
-    }();
-    return v;
+// CTAs of a deferred acceptance launch with `smem` bytes of bounds per CTA: as
+// many per SM as fit, so that all are resident.
+int32_t da_grid(size_t smem) {
+    int32_t per_sm = kDaPerSm;
+    while (per_sm > 1 && per_sm * (smem + 2048) > 227 * 1024) --per_sm;
+    return dgs::device_sms() * per_sm;
 }
-
-template <template <int> class K>
-const void* da_kernel_for(int32_t g) {
-    return g == 32 ? reinterpret_cast<const void*>(K<32>::fn)
-         : g == 128 ? reinterpret_cast<const void*>(K<128>::fn)
-         : g == 512 ? reinterpret_cast<const void*>(K<512>::fn)
-                    : reinterpret_cast<const void*>(K<256>::fn);
-}
-template <int G> struct SingleDa { static constexpr auto fn = greedy_da_kernel<G>; };
-template <int G> struct BatchedDa { static constexpr auto fn = greedy_da_batched_kernel<G>; };
 
 // The greedy start of every instance in kStageGreedy (deferred acceptance:
 // queue the agents, one launch, then the assignments; the advance kernel
@@ -675,10 +798,8 @@ template <int G> struct BatchedDa { static constexpr auto fn = greedy_da_batched
 cudaError_t launch_b_greedy(const BatchTable& rows, const BatchQueues& q, cudaStream_t s) {
     cudaError_t e = launch_b_scan(q, kScanGreedyDA, 0, s);
     if (e != cudaSuccess) return e;
-    BatchQueues arg = q;
-    void* args[] = {&arg};
-    e = cudaLaunchKernel(da_kernel_for<BatchedDa>(da_group_env()), dim3(dgs::device_sms()), dim3(kDaThreads), args,
-                         0, s);
+    greedy_da_batched_kernel<<<da_grid(0), kDaThreads, 0, s>>>(q);
+    e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     greedy_da_finish_batched_kernel<<<dgs::device_sms() * 8, 256, 0, s>>>(rows);
     return cudaGetLastError();
@@ -694,11 +815,15 @@ int32_t greedy_rounds_env() {
 }
 
 cudaError_t launch_greedy_da(const Workspace& w, cudaStream_t s) {
-    if (greedy_rounds_env() || w.g_list == nullptr) return cudaErrorNotSupported;
-    const void* kernel = da_kernel_for<SingleDa>(da_group_env());
-    Workspace arg = w;
-    void* args[] = {&arg};
-    cudaError_t e = cudaLaunchKernel(kernel, dim3(dgs::device_sms()), dim3(kDaThreads), args, 0, s);
+    if (greedy_rounds_env() || w.g_bound == nullptr) return cudaErrorNotSupported;
+    constexpr int kGroups = kDaWarps / kDaGroup;
+    const size_t smem = sizeof(uint32_t) * kGroups * (size_t)w.bound_tiles;
+    cudaError_t e = ensure_smem_limit(reinterpret_cast<const void*>(greedy_da_kernel<kDaGroup>), 16, smem);
+    if (e != cudaSuccess) return e;
+    const int32_t most = (w.n + kGroups - 1) / kGroups;
+    const int32_t grid = most < da_grid(smem) ? most : da_grid(smem);
+    greedy_da_kernel<kDaGroup><<<grid, kDaThreads, smem, s>>>(w);
+    e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const int32_t nb = (w.n + 255) / 256;
     greedy_da_finish_kernel<<<nb < dgs::device_sms() * 4 ? nb : dgs::device_sms() * 4, 256, 0, s>>>(w);
