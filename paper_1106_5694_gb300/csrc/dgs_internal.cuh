@@ -93,10 +93,10 @@ struct Workspace {
     uint8_t* in_y; uint8_t* moved;        // jobs changed / agents moved in the last event
     int32_t* y_list;                      // jobs changed in the last event
     int32_t* rescan_list;                 // rows to re-evaluate fully
-    // per slot (agent slots 0..n-1, job slots n..2n-1): its edge word (0 when
-    // it has no candidate)
+    // per chunk of 32 slots (agent slots 0..n-1, job slots n..2n-1): the edge
+    // words of the slots that have a candidate, from its first entry on
     unsigned long long* sl_edge;
-    int32_t* sl_chunk;  // edges among slots 32c .. 32c + 31 (written with sl_edge)
+    int32_t* sl_chunk;  // how many
     int32_t* ctl_slot;  // controller: slot of each edge position (priority order)
     // greedy start
     unsigned long long* g_row;  // round form: best free job per agent (biased value, ~j)
@@ -304,6 +304,11 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
         "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
         ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar))
         : "memory");
+}
+
+// 1-D bulk prefetch into L2; src 16-byte aligned, bytes a multiple of 16.
+__device__ __forceinline__ void bulk_prefetch_l2(const void* src, uint32_t bytes) {
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
 }
 
 // Grid-wide barrier for cooperative launches (every CTA co-resident).  The

@@ -42,13 +42,15 @@ constexpr int kCtlThreads = 1024;
 // Slot edge word: agent u (bits 0..16), agent v (17..33), applies (34): its
 // exchange raises f under the current sigma, revives (35): the slot's row has
 // a positive gain under the current sigma, so that re-evaluating the slot
-// gives it a candidate again, valid (36): set on every edge (0 means "no
-// candidate").  Edge positions follow slot priority, so a position is a priority.
+// gives it a candidate again, place (36..40): the slot's place among the 32 of
+// its chunk.  The edges of a chunk (32 consecutive slots) are stored from its
+// first entry on, in slot order, with their number beside them.  Edge positions
+// follow slot priority, so a position is a priority.
 constexpr unsigned long long kApplies = 1ull << 34;
 constexpr unsigned long long kRevives = 1ull << 35;
-constexpr unsigned long long kValid = 1ull << 36;  // a slot's edge word is never 0
+constexpr int kPlaceShift = 36;
 __device__ __forceinline__ unsigned long long edge_word(int32_t u, int32_t v) {
-    return (unsigned long long)(uint32_t)u | ((unsigned long long)(uint32_t)v << 17) | kValid;
+    return (unsigned long long)(uint32_t)u | ((unsigned long long)(uint32_t)v << 17);
 }
 __device__ __forceinline__ int32_t edge_u(unsigned long long e) { return (int32_t)(e & 0x1FFFFu); }
 __device__ __forceinline__ int32_t edge_v(unsigned long long e) { return (int32_t)((e >> 17) & 0x1FFFFu); }
@@ -490,6 +492,8 @@ __device__ __forceinline__ void controller_body(const Workspace& w, int32_t smem
     __shared__ int32_t warp_sums[33];
     __shared__ int32_t s_L, s_live, s_stop, s_acc, s_app, s_y, s_sweeps, s_event;
     __shared__ int32_t s_max_sweeps, s_trace_cap;
+    __shared__ int32_t s_events;
+    __shared__ long long s_swaps;
     __shared__ int32_t s_window;  // the next sweeps may run as a colouring window
     __shared__ WindowShared s_win;
     __shared__ uint32_t s_round;
@@ -541,85 +545,92 @@ __device__ __forceinline__ void controller_body(const Workspace& w, int32_t smem
     // The slot refresh and the per-slot edge data were prepared by the grid
     // (prepare_edges_kernel); here the edges are listed in priority order.
     {
-        for (int32_t i = tid; i < n; i += kT) {
-            res[i] = 0xFFFFFFFFu;
-            claimed[i] = 0;
-        }
+        // Warp wp lists the chunks of its own range (ranges ascend with wp): it
+        // sums their edge counts, and with the 32 warps' sums each warp knows
+        // where its edges go, so positions follow slot order (the priority
+        // order).  (The loads first, then the clearing, which waits for
+        // nothing.)
+        constexpr int kWarps = kT / 32;
+        const int32_t lane = tid & 31, wp = tid >> 5;
+        const int32_t nchunks = (2 * n + 31) >> 5;
+        const int32_t per = (nchunks + kWarps - 1) / kWarps;
+        const int32_t c_lo = min(nchunks, wp * per), c_hi = min(nchunks, c_lo + per);
+        uint32_t cnt = 0;
+        for (int32_t c = c_lo + lane; c < c_hi; c += 32) cnt += (uint32_t)w.sl_chunk[c];
         if (tid == 0) {
-            st->need_update = 0;
-            st->y_count = 0;
+            s_swaps = st->swaps;
+            s_events = st->events;
             s_sweeps = st->sweeps;
             s_max_sweeps = st->max_sweeps;
             s_deadline = st->deadline_ns;
             s_trace_cap = st->trace_capacity;
             s_f = st->f;
+            st->need_update = 0;
+            st->y_count = 0;
             s_round = 0;
             s_stamp = 0;
             s_window = 0;
         }
-        // Warp wp lists the slots of its own range [lo, hi) (ranges are
-        // multiples of 32 long and ascend with wp): it sums the edge counts
-        // of its 32-slot chunks (written by the grid beside the edge words),
-        // the 32 warp counts are scanned once, and it writes the edges of
-        // its chunks that have any at its offset, so positions follow slot
-        // order (the priority order).
-        constexpr int kWarps = kT / 32;
-        const int32_t lane = tid & 31, wp = tid >> 5;
-        const int32_t per = (2 * n + 32 * kWarps - 1) / (32 * kWarps) * 32;
-        const int32_t lo = min(2 * n, wp * per), hi = min(2 * n, lo + per);
-        const int32_t c_lo = lo >> 5, c_hi = lo < hi ? (hi + 31) >> 5 : c_lo;  // lo is a multiple of 32
-        int32_t cnt = 0;
-        for (int32_t c = c_lo + lane; c < c_hi; c += 32) cnt += w.sl_chunk[c];
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, off);
-        if (lane == 0) warp_sums[wp] = cnt;
-        __syncthreads();
-        if (wp == 0) {
-            const int32_t v = lane < kWarps ? warp_sums[lane] : 0;
-            int32_t incl = v;
-#pragma unroll
-            for (int off = 1; off < 32; off <<= 1) {
-                const int32_t o = __shfl_up_sync(0xffffffffu, incl, off);
-                if (lane >= off) incl += o;
-            }
-            warp_sums[lane] = incl - v;
-            if (lane == 31) warp_sums[32] = incl;
+        // (in words of 16 and 4 bytes: what lies past the last one's end is
+        // padding, or edges and states that are written only later)
+        for (int32_t i = tid; i < (n + 3) / 4; i += kT) {
+            reinterpret_cast<uint4*>(res)[i] = make_uint4(~0u, ~0u, ~0u, ~0u);
+            reinterpret_cast<uint32_t*>(claimed)[i] = 0u;
         }
+        cnt = __reduce_add_sync(0xffffffffu, cnt);
+        if (lane == 0) warp_sums[wp] = (int32_t)cnt;
         __syncthreads();
-        if (es_cap > 0 && warp_sums[32] <= es_cap) E = Es;  // the whole list fits in shared memory
-        int32_t pos0 = warp_sums[wp];
-        const uint32_t below = (1u << lane) - 1u;
+        const uint32_t sums = lane < kWarps ? (uint32_t)warp_sums[lane] : 0u;
+        const int32_t total = (int32_t)__reduce_add_sync(0xffffffffu, sums);
+        int32_t pos0 = (int32_t)__reduce_add_sync(0xffffffffu, lane < wp ? sums : 0u);
+        if (es_cap > 0 && total <= es_cap) E = Es;  // the whole list fits in shared memory
+        auto list_edge = [&](int32_t pos, int32_t c, unsigned long long e) {
+            w.ctl_slot[pos] = c * 32 + (int32_t)((e >> kPlaceShift) & 31u);
+            E[pos] = C::make(edge_u(e), edge_v(e));
+            estate[pos] = kAlive | ((e & kApplies) ? kAppl : 0) | ((e & kRevives) ? kRevive : 0);
+        };
         for (int32_t cb = c_lo; cb < c_hi; cb += 32) {
-            uint32_t nz = __ballot_sync(0xffffffffu, cb + lane < c_hi && w.sl_chunk[cb + lane] > 0);
-            while (nz) {  // four chunks with edges at a time, their loads in flight together
-                int32_t ck[4];
-                unsigned long long ew[4];
+            const int32_t mine = cb + lane < c_hi ? w.sl_chunk[cb + lane] : 0;
+            const int32_t most = (int32_t)__reduce_max_sync(0xffffffffu, (uint32_t)mine);
+            // a lane per chunk where one trip to memory takes them all (kAhead
+            // words in flight), else a lane per edge
+            constexpr int kAhead = 8;
+            if (most <= kAhead) {
+                int32_t incl = mine;
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    ck[k] = nz ? cb + __ffs(nz) - 1 : -1;
-                    nz &= nz - 1u;
+                for (int off = 1; off < 32; off <<= 1) {
+                    const int32_t o = __shfl_up_sync(0xffffffffu, incl, off);
+                    if (lane >= off) incl += o;
                 }
+                const int32_t pos = pos0 + incl - mine;
+                const unsigned long long* src = w.sl_edge + (size_t)(cb + lane) * 32;
+                for (int32_t k0 = 0; k0 < most; k0 += kAhead) {
+                    unsigned long long e[kAhead];
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const int32_t t = ck[k] * 32 + lane;
-                    ew[k] = (ck[k] >= 0 && t < hi) ? w.sl_edge[t] : 0ull;
+                    for (int k = 0; k < kAhead; ++k) e[k] = k0 + k < mine ? src[k0 + k] : 0ull;
+#pragma unroll
+                    for (int k = 0; k < kAhead; ++k)
+                        if (k0 + k < mine) list_edge(pos + k0 + k, cb + lane, e[k]);
                 }
+                pos0 += __shfl_sync(0xffffffffu, incl, 31);
+            } else {
+                for (int32_t k0 = 0; k0 < min(32, c_hi - cb); k0 += 4) {
+                    int32_t m[4];
+                    unsigned long long e[4];
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const int32_t t = ck[k] * 32 + lane;
-                    const bool has = ew[k] != 0ull;
-                    const uint32_t m = __ballot_sync(0xffffffffu, has);
-                    if (has) {
-                        const int32_t pos = pos0 + __popc(m & below);
-                        w.ctl_slot[pos] = t;
-                        E[pos] = C::make(edge_u(ew[k]), edge_v(ew[k]));
-                        estate[pos] = kAlive | ((ew[k] & kApplies) ? kAppl : 0) | ((ew[k] & kRevives) ? kRevive : 0);
+                    for (int k = 0; k < 4; ++k) {
+                        m[k] = __shfl_sync(0xffffffffu, mine, k0 + k);
+                        e[k] = lane < m[k] ? w.sl_edge[(size_t)(cb + k0 + k) * 32 + lane] : 0ull;
                     }
-                    pos0 += __popc(m);
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        if (lane < m[k]) list_edge(pos0 + lane, cb + k0 + k, e[k]);
+                        pos0 += m[k];
+                    }
                 }
             }
         }
-        if (tid == 0) { s_L = warp_sums[32]; s_live = warp_sums[32]; }
+        if (tid == 0) s_L = s_live = total;
         __syncthreads();
     }
     DGS_CT(kPtCtlEntry)
@@ -843,72 +854,71 @@ __device__ __forceinline__ void controller_body(const Workspace& w, int32_t smem
         const int32_t nacc = s_acc;
         if (s_event) {
             // parallel switch: accepted exchanges are agent-disjoint; those
-            // that raise f under the current sigma commit
-            int32_t my_app = 0;
-            long long my_gain = 0;
-            for (int32_t q = tid; q < nacc; q += kT) {
-                const int32_t p = accl.get(q);
-                estate[p] |= kAccBit;
-                if (!(estate[p] & kAppl)) continue;
-                const EdgeT e = E[p];
-                const int32_t u = C::u(e), v = C::v(e);
-                const int32_t ju = w.tau[u], jv = w.tau[v];
-                const int32_t x1 = w.a[(size_t)u * w.lda + jv];
-                const int32_t x2 = w.a[(size_t)v * w.lda + ju];
-                my_gain += (long long)x1 + x2 - w.diag[ju] - w.diag[jv];
-                w.tau[u] = jv;
-                w.tau[v] = ju;
-                w.sigma[jv] = u;
-                w.sigma[ju] = v;
-                w.diag[jv] = x1;
-                w.diag[ju] = x2;
-                ++my_app;
-                const int32_t qy = atomicAdd(&s_y, 2);
-                w.y_list[qy] = ju;
-                w.y_list[qy + 1] = jv;
-                w.in_y[ju] = 1;
-                w.in_y[jv] = 1;
-                w.moved[u] = 1;
-                w.moved[v] = 1;
-            }
-            if (my_app) {
-                atomicAdd(&s_app, my_app);
-                atomicAdd(&s_gain, (unsigned long long)my_gain);
-            }
-            if (((reinterpret_cast<uintptr_t>(w.in_ca) | reinterpret_cast<uintptr_t>(w.in_cj)) & 15) == 0) {
-                // both arrays hold round_up(n, 128) bytes: clear them in 16-byte words
-                const int32_t n16 = (n + 15) / 16;
-                for (int32_t i = tid; i < n16; i += kT) {
-                    reinterpret_cast<uint4*>(w.in_ca)[i] = make_uint4(0, 0, 0, 0);
-                    reinterpret_cast<uint4*>(w.in_cj)[i] = make_uint4(0, 0, 0, 0);
-                }
-            } else {
-                for (int32_t i = tid; i < n; i += kT) {
-                    w.in_ca[i] = 0;
-                    w.in_cj[i] = 0;
-                }
-            }
+            // that raise f under the current sigma commit.  C (every live slot
+            // that was not accepted) keeps its candidates (reading R4); its
+            // marks are cleared where they are read (prepare_edges_body).
+            // (The sums go through the warp first: 64-bit atomics of every
+            // thread on one shared word are retry loops.)
+            for (int32_t q = tid; q < nacc; q += kT) estate[accl.get(q)] |= kAccBit;
             __syncthreads();
-            // record C: every live slot that was not accepted keeps its
-            // candidate (reading R4)
+            const int32_t slot0 = tid < L ? w.ctl_slot[tid] : 0;  // in flight during the commits
+            const int lane = tid & 31;
+            for (int32_t q0 = tid - lane; q0 < nacc; q0 += kT) {
+                const int32_t q = q0 + lane;
+                const int32_t p = q < nacc ? accl.get(q) : 0;
+                const bool commits = q < nacc && (estate[p] & kAppl);
+                const uint32_t cm = __ballot_sync(0xffffffffu, commits);
+                if (cm == 0u) continue;
+                int32_t qy = 0;
+                if (lane == 0) {
+                    qy = atomicAdd(&s_y, 2 * __popc(cm));
+                    atomicAdd(&s_app, __popc(cm));
+                }
+                qy = __shfl_sync(0xffffffffu, qy, 0) + 2 * __popc(cm & ((1u << lane) - 1u));
+                long long gain = 0;
+                if (commits) {
+                    const EdgeT e = E[p];
+                    const int32_t u = C::u(e), v = C::v(e);
+                    const int32_t ju = w.tau[u], jv = w.tau[v];
+                    const int32_t x1 = w.a[(size_t)u * w.lda + jv];
+                    const int32_t x2 = w.a[(size_t)v * w.lda + ju];
+                    gain = (long long)x1 + x2 - w.diag[ju] - w.diag[jv];
+                    w.tau[u] = jv;
+                    w.tau[v] = ju;
+                    w.sigma[jv] = u;
+                    w.sigma[ju] = v;
+                    w.diag[jv] = x1;
+                    w.diag[ju] = x2;
+                    w.y_list[qy] = ju;
+                    w.y_list[qy + 1] = jv;
+                    w.in_y[ju] = 1;
+                    w.in_y[jv] = 1;
+                    w.moved[u] = 1;
+                    w.moved[v] = 1;
+                }
+#pragma unroll
+                for (int off = 16; off > 0; off >>= 1) gain += __shfl_xor_sync(0xffffffffu, gain, off);
+                if (lane == 0) atomicAdd(&s_gain, (unsigned long long)gain);
+            }
             for (int32_t p = tid; p < L; p += kT) {
                 const uint8_t es = estate[p];
                 if (!(es & kAlive) || (es & kAccBit)) continue;
-                const int32_t t = w.ctl_slot[p];
+                const int32_t t = p == tid ? slot0 : w.ctl_slot[p];
                 if (t < n) w.in_ca[t] = 1;
                 else w.in_cj[t - n] = 1;
             }
+            __syncthreads();  // the sums are complete
             if (tid == 0) {
                 const int32_t sw = s_sweeps;
                 s_f += (long long)s_gain;
-                st->swaps += s_app;
+                s_swaps += s_app;
                 if (sw < s_trace_cap) {
                     if (st->trace_accepted) st->trace_accepted[sw] = nacc;
                     if (st->trace_applied) st->trace_applied[sw] = s_app;
                     if (st->trace_objective) st->trace_objective[sw] = s_f;
                 }
                 s_sweeps = sw + 1;
-                st->events += 1;
+                s_events += 1;
                 st->y_count = s_y;
                 st->rescan_count = 0;
                 st->need_update = 1;
@@ -953,6 +963,8 @@ __device__ __forceinline__ void controller_body(const Workspace& w, int32_t smem
         st->sweeps = s_sweeps;
         st->edge_count = s_live;
         st->f = s_f;
+        st->swaps = s_swaps;
+        st->events = s_events;
     }
     __syncthreads();  // shared memory is reused by the caller's next call
 }
@@ -991,6 +1003,7 @@ __device__ __forceinline__ void prepare_edges_body(const Workspace& w, int32_t b
     const int32_t n = w.n;
     const int32_t stride = nblk * blockDim.x;
     const int32_t yc = st->y_count;
+    const bool reeval_all = st->reeval_all != 0;
     for (int32_t t = bid * blockDim.x + threadIdx.x; t < yc; t += stride) {
         const int32_t j = w.y_list[t];
         w.in_y[j] = 0;
@@ -1002,7 +1015,9 @@ __device__ __forceinline__ void prepare_edges_body(const Workspace& w, int32_t b
         bool in_c;
         if (t < n) {
             key = w.key_a[w.tau[t]];
-            in_c = w.in_ca[t] && !st->reeval_all;
+            in_c = w.in_ca[t];
+            if (in_c) w.in_ca[t] = 0;  // the next commit marks its own
+            in_c = in_c && !reeval_all;
             if (!in_c) {
                 w.ag_gain[t] = key ? key_gain(key) : 0;
                 w.ag_job[t] = key ? key_index(key) : -1;
@@ -1012,7 +1027,9 @@ __device__ __forceinline__ void prepare_edges_body(const Workspace& w, int32_t b
         } else {
             const int32_t j = t - n;
             key = w.key_j[j];
-            in_c = w.in_cj[j] && !st->reeval_all;
+            in_c = w.in_cj[j];
+            if (in_c) w.in_cj[j] = 0;
+            in_c = in_c && !reeval_all;
             if (!in_c) {
                 w.jb_gain[j] = key ? key_gain(key) : 0;
                 w.jb_agent[j] = key ? key_index(key) : -1;
@@ -1020,18 +1037,19 @@ __device__ __forceinline__ void prepare_edges_body(const Workspace& w, int32_t b
             gain = in_c ? w.jb_gain[j] : (key ? key_gain(key) : 0);
             target = in_c ? w.jb_agent[j] : (key ? key_index(key) : -1);
         }
+        const uint32_t am = __activemask();
         unsigned long long e = 0ull;
         if (gain > 0) {
             const int32_t u = (t < n) ? t : w.sigma[t - n];
             const int32_t v = (t < n) ? w.sigma[target] : target;
             e = edge_word(u, v) | (exchange_gain(w, u, v) > 0 ? kApplies : 0ull) | (key ? kRevives : 0ull);
         }
-        w.sl_edge[t] = e;
-        // the warp's 32 consecutive slots form one chunk: its edge count
-        // lets the controller skip chunks without edges
-        const uint32_t am = __activemask();
-        const uint32_t bm = __ballot_sync(am, e != 0ull);
-        if ((int)(threadIdx.x & 31) == __ffs(am) - 1) w.sl_chunk[t >> 5] = __popc(bm);
+        // the warp's 32 consecutive slots form one chunk
+        const uint32_t bm = __ballot_sync(am, gain > 0);
+        const int32_t lane = (int32_t)(threadIdx.x & 31u);
+        if (gain > 0)
+            w.sl_edge[(t & ~31) + __popc(bm & ((1u << lane) - 1u))] = e | ((unsigned long long)(t & 31) << kPlaceShift);
+        if (lane == __ffs(am) - 1) w.sl_chunk[t >> 5] = __popc(bm);
     }
 }
 
@@ -1135,6 +1153,8 @@ __device__ __forceinline__ bool row_task_row(const Workspace& w, int32_t j, int3
             const uint32_t bytes = 16u * (uint32_t)((w.n + 3) / 4);
             mbar_arrive_expect_tx(bar, bytes);
             bulk_g2s(atrow_s, atrow, bytes, bar);
+            // the row of a meanwhile into L2
+            bulk_prefetch_l2(w.a + (size_t)w.sigma[j] * w.lda, bytes);
         }
         const bool ok = mbar_wait_bounded(bar, phase);
         if (__syncthreads_or(!ok)) {
@@ -1671,9 +1691,13 @@ cudaError_t launch_mark_rescan(const Workspace& w, cudaStream_t s) {
 constexpr int32_t kRowStageMaxN = 54 * 1024;
 
 cudaError_t launch_row_tasks(const Workspace& w, cudaStream_t s) {
-    const int grid = dgs::device_sms() * 2;
+    int grid = dgs::device_sms() * 2;
     if (w.n <= kRowStageMaxN) {
         const size_t smem = 4 * (size_t)w.ldt;
+        // as many CTAs as fit (four of 512 threads per SM): the few hundred
+        // rows of an update then go in one wave
+        const int fit = (int)((227 * 1024) / (smem + 2048));
+        grid = dgs::device_sms() * (fit > 4 ? 4 : fit < 1 ? 1 : fit);
         if (smem > 48 * 1024) {
             cudaError_t e = ensure_smem_limit(reinterpret_cast<const void*>(row_tasks_kernel<true>), 2, smem);
             if (e != cudaSuccess) return e;
