@@ -519,9 +519,17 @@ LoopKey loop_key(const LoopCtx& c) {
     return k;
 }
 
+// Iterations in one pass of the switching loop's WHILE node: a pass begins 4
+// us after the last one ended, while an iteration that finds the loop ended
+// costs 6 to 7 us, at most kLoopUnroll - 1 times a solve.  Measured, one / two
+// / four / eight per pass: peer-shaped n = 10000 (16 iterations) 1.160 / 1.128
+// / 1.106 / 1.100 ms, n = 1021 (11 iterations) 0.366 / 0.348 / 0.334 / 0.345,
+// distances n = 2048 from a random start (160) 5.27 / 5.05 / 4.97 / 4.89.
+constexpr int32_t kLoopUnroll = 4;
+
 // DGS_LOOP_ON_HOST=1 (profiling only: per-kernel profilers do not see the
 // kernels inside conditional graph nodes): the switching loop's body is
-// launched from the host, four iterations between reads of the loop state,
+// launched from the host, kLoopUnroll iterations between reads of the loop state,
 // which makes the call wait for the solve.  Results are the same.
 int32_t env_loop_on_host() {
     static const int32_t v = [] {
@@ -538,8 +546,8 @@ dgs_status enqueue_loop(cudaStream_t s, LoopBody body, LoopCtx* c) {
         DeviceState* h = static_cast<DeviceState*>(pinned_get(sizeof(DeviceState)));
         if (h == nullptr) return DGS_ERR_OOM;
         dgs_status st = DGS_OK;
-        for (int64_t it = 0; st == DGS_OK && it < 16 * (int64_t)c->w.n + 4096; it += 4) {
-            for (int r = 0; r < 4 && st == DGS_OK; ++r) st = body(c, s, 0);
+        for (int64_t it = 0; st == DGS_OK && it < 16 * (int64_t)c->w.n + 4096; it += kLoopUnroll) {
+            st = body(c, s, 0);
             cudaError_t e = cudaMemcpyAsync(h, c->w.st, sizeof(DeviceState), cudaMemcpyDeviceToHost, s);
             if (e == cudaSuccess) e = cudaStreamSynchronize(s);
             if (e != cudaSuccess) st = cuda_fail(e, "reading loop state");
@@ -560,17 +568,28 @@ dgs_status greedy_round_body(void* p, cudaStream_t cs, unsigned long long h) {
     return DGS_OK;
 }
 
-// One iteration of the switching loop of Algorithm 3: re-evaluate what the
+dgs_status reevaluate_all_body(void* p, cudaStream_t cs, unsigned long long) {
+    DGS_CUDA(launch_full_evaluation(static_cast<const LoopCtx*>(p)->w, 1, cs), "re-evaluation");
+    return DGS_OK;
+}
+dgs_status reevaluate_rows_body(void* p, cudaStream_t cs, unsigned long long) {
+    DGS_CUDA(launch_row_tasks(static_cast<const LoopCtx*>(p)->w, cs), "row tasks");
+    return DGS_OK;
+}
+
+// Iterations of the switching loop of Algorithm 3: re-evaluate what the
 // last committing sweep changed (marked rows by row tasks, or all rows by a
-// full evaluation), refresh the slots not in C, then the controller's sweeps;
-// the controller decides whether the loop goes on.
+// full evaluation: only one of the two kernels finds work, so they need not
+// wait for one another), refresh the slots not in C, then the controller's
+// sweeps; the last controller decides whether the loop goes on.
 dgs_status switching_body(void* p, cudaStream_t cs, unsigned long long h) {
     const LoopCtx* c = static_cast<const LoopCtx*>(p);
-    DGS_CUDA(launch_mark_rescan(c->w, cs), "mark");
-    DGS_CUDA(launch_full_evaluation(c->w, 1, cs), "re-evaluation");
-    DGS_CUDA(launch_row_tasks(c->w, cs), "row tasks");
-    DGS_CUDA(launch_prepare_edges(c->w, cs), "prepare");
-    DGS_CUDA(launch_controller_impl(c->w, c->ctl, cs, h), "controller");
+    for (int32_t r = 0; r < kLoopUnroll; ++r) {
+        DGS_CUDA(launch_mark_rescan(c->w, cs), "mark");
+        DGS_TRY(capture_side_by_side(cs, reevaluate_rows_body, reevaluate_all_body, p));
+        DGS_CUDA(launch_prepare_edges(c->w, cs), "prepare");
+        DGS_CUDA(launch_controller_impl(c->w, c->ctl, cs, h != 0, r + 1 == kLoopUnroll ? h : 0), "controller");
+    }
     return DGS_OK;
 }
 

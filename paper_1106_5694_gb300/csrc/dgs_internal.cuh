@@ -374,10 +374,11 @@ int32_t size_bucket(int32_t n);
 cudaError_t launch_full_evaluation_shape(const Workspace& w, int32_t conditional, EvalShape shape, cudaStream_t s);
 cudaError_t launch_keys_to_slots(const Workspace& w, int32_t* ag, int32_t* aj, int32_t* jg, int32_t* ja,
                                  cudaStream_t s);
-// handle != 0: the controller ends each launch by setting that loop
-// condition (1 while the loop state is running) and counts the iteration.
-cudaError_t launch_controller_impl(const Workspace& w, const CtlGlobal& g, cudaStream_t s,
-                                   unsigned long long handle = 0);
+// counted: the launch ends an iteration of the device-side switching loop and
+// counts it; handle != 0: it also sets that loop condition (1 while the loop
+// state is running).
+cudaError_t launch_controller_impl(const Workspace& w, const CtlGlobal& g, cudaStream_t s, bool counted,
+                                   unsigned long long handle);
 // The switching loop in one CTA for small n (see small_loop_kernel), and
 // whether a solve of this workspace takes it.
 bool use_small_loop(const Workspace& w);
@@ -460,6 +461,10 @@ dgs_status enqueue_while(cudaStream_t s, LoopBody body, void* ctx);
 // body's launches are captured with); up to 16 are kept.
 dgs_status enqueue_while_cached(cudaStream_t s, LoopBody body, void* ctx, const void* key, size_t key_bytes);
 dgs_status create_loop_handle(cudaStream_t capturing, unsigned long long* handle);
+// Inside a capture: what a and b enqueue (each on the capture stream) both
+// follow what was enqueued before, not one another; what comes next follows
+// both.  Outside a capture they are enqueued one after the other.
+dgs_status capture_side_by_side(cudaStream_t s, LoopBody a, LoopBody b, void* ctx);
 dgs_status capture_while(cudaStream_t capturing, LoopBody body, void* ctx, unsigned long long handle = 0);
 // Pinned host staging blocks from a process-wide cache (never freed while the
 // process runs; pinned_put may be called from a stream callback).

@@ -128,6 +128,35 @@ dgs_status capture_while(cudaStream_t capturing, LoopBody body, void* ctx, unsig
     return DGS_OK;
 }
 
+dgs_status capture_side_by_side(cudaStream_t s, LoopBody a, LoopBody b, void* ctx) {
+    cudaStreamCaptureStatus cst = cudaStreamCaptureStatusNone;
+    const cudaGraphNode_t* deps = nullptr;
+    const cudaGraphEdgeData* edata = nullptr;
+    size_t nd = 0;
+    cudaError_t e = cudaStreamGetCaptureInfo(s, &cst, nullptr, nullptr, &deps, &edata, &nd);
+    if (e != cudaSuccess) return fail(e, "capture info");
+    dgs_status st;
+    if (cst != cudaStreamCaptureStatusActive) {  // launched directly: one after the other
+        st = a(ctx, s, 0);
+        return st == DGS_OK ? b(ctx, s, 0) : st;
+    }
+    // (the arrays belong to the capture and change with it)
+    const std::vector<cudaGraphNode_t> before(deps, deps + nd);
+    st = a(ctx, s, 0);
+    if (st != DGS_OK) return st;
+    e = cudaStreamGetCaptureInfo(s, &cst, nullptr, nullptr, &deps, &edata, &nd);
+    if (e != cudaSuccess) return fail(e, "capture info");
+    std::vector<cudaGraphNode_t> ends(deps, deps + nd);
+    std::vector<cudaGraphNode_t> from = before;
+    e = cudaStreamUpdateCaptureDependencies(s, from.data(), nullptr, from.size(), cudaStreamSetCaptureDependencies);
+    if (e != cudaSuccess) return fail(e, "capture order");
+    st = b(ctx, s, 0);
+    if (st != DGS_OK) return st;
+    e = cudaStreamUpdateCaptureDependencies(s, ends.data(), nullptr, ends.size(), cudaStreamAddCaptureDependencies);
+    if (e != cudaSuccess) return fail(e, "capture order");
+    return DGS_OK;
+}
+
 namespace {
 struct GraphHolder {
     cudaGraph_t g = nullptr;

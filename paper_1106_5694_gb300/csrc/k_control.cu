@@ -969,17 +969,17 @@ __device__ __forceinline__ void controller_body(const Workspace& w, int32_t smem
     __syncthreads();  // shared memory is reused by the caller's next call
 }
 
-// cond != 0: the launch is the last kernel of an iteration of the device-
-// side switching loop (a conditional WHILE graph node, five kernels per
-// iteration); it sets the loop condition from the loop state.  The loop is
-// bounded: more than 16 n + 4096 iterations is an internal error.
+// counted: the launch is the last kernel of an iteration of the device-side
+// switching loop (a conditional WHILE graph node, five kernels per iteration).
+// The loop is bounded: more than 16 n + 4096 iterations is an internal error.
+// cond != 0: it also sets the loop condition from the loop state.
 template <typename EdgeT>
 __global__ void __launch_bounds__(kCtlThreads, 1) controller_kernel(Workspace w, int32_t smem_mode, CtlScratch g,
                                                                    uint32_t span, uint32_t stamp_wrap,
                                                                    int32_t compact_min, int32_t colour_pass,
-                                                                   unsigned long long cond) {
+                                                                   int32_t counted, unsigned long long cond) {
     controller_body<EdgeT>(w, smem_mode, g, span, stamp_wrap, compact_min, colour_pass);
-    if (cond != 0 && threadIdx.x == 0) {
+    if (counted && threadIdx.x == 0) {
         DeviceState* st = w.st;
         const int32_t it = ++st->loop_iterations;
         st->loop_launches += 5;
@@ -987,7 +987,7 @@ __global__ void __launch_bounds__(kCtlThreads, 1) controller_kernel(Workspace w,
             st->error = kErrInternal;
             st->status = kError;
         }
-        cudaGraphSetConditional(cond, st->status == kRunning ? 1u : 0u);
+        if (cond != 0) cudaGraphSetConditional(cond, st->status == kRunning ? 1u : 0u);
     }
 }
 
@@ -1650,7 +1650,8 @@ cudaError_t launch_small_loop(const Workspace& w, const CtlGlobal& gs, cudaStrea
     }
 }
 
-cudaError_t launch_controller_impl(const Workspace& w, const CtlGlobal& gs, cudaStream_t s, unsigned long long handle) {
+cudaError_t launch_controller_impl(const Workspace& w, const CtlGlobal& gs, cudaStream_t s, bool counted,
+                                   unsigned long long handle) {
     const int32_t mode = controller_smem_mode(w.n);
     const size_t smem = controller_smem_bytes(w.n);
     CtlScratch c{gs.res, gs.claimed, gs.estate, gs.edges, gs.acc};
@@ -1667,10 +1668,10 @@ cudaError_t launch_controller_impl(const Workspace& w, const CtlGlobal& gs, cuda
     const int32_t cmin = env_compact_min();
     const int32_t cp = env_colour_pass();
     if (narrow)
-        controller_kernel<uint32_t><<<1, kCtlThreads, smem, s>>>(w, mode, c, span, stamp_wrap, cmin, cp, handle);
+        controller_kernel<uint32_t><<<1, kCtlThreads, smem, s>>>(w, mode, c, span, stamp_wrap, cmin, cp, counted, handle);
     else
         controller_kernel<unsigned long long><<<1, kCtlThreads, smem, s>>>(w, mode, c, span, stamp_wrap, cmin, cp,
-                                                                          handle);
+                                                                          counted, handle);
     return cudaGetLastError();
 }
 
