@@ -257,21 +257,20 @@ class Engine {
     } while (0)
         const BatchTable rows = table(kTabRows), one = table(kTabOne);
         const BatchQueues q{d_inst_, cap_, d_q_, d_q_ + cap_ + 1};
-        const int32_t strip = evaluation_strip();
         B_LAUNCH(launch_b_init(rows, s), 1, "init");
-        B_LAUNCH(launch_b_scan(q, kScanPass1, strip, s), 1, "scan");
+        B_LAUNCH(launch_b_scan(q, kScanPass1, s), 1, "scan");
         B_LAUNCH(launch_b_pass1(q, s), 1, "pass 1");
         B_LAUNCH(launch_b_advance(one, kStageNew, s), 1, "advance");
         B_LAUNCH(launch_b_greedy(rows, q, s), 3, "greedy start");
         B_LAUNCH(launch_b_advance(one, kStageGreedy, s), 1, "advance");
         B_LAUNCH(launch_b_start(rows, s), 1, "start");
-        B_LAUNCH(launch_b_scan(q, kScanStart, strip, s), 1, "scan");
-        B_LAUNCH(launch_b_evaluation(q, strip, s), 1, "evaluation");
+        B_LAUNCH(launch_b_scan(q, kScanStart, s), 1, "scan");
+        B_LAUNCH(launch_b_evaluation(q, s), 1, "evaluation");
         B_LAUNCH(launch_b_advance(one, kStageStart, s), 1, "advance");
         for (int32_t i = 0; i < kSwitchPerStep; ++i) {
             B_LAUNCH(launch_b_mark_rescan(rows, s), 1, "mark");
-            B_LAUNCH(launch_b_scan(q, kScanSwitch, strip, s), 1, "scan");
-            B_LAUNCH(launch_b_evaluation(q, strip, s), 1, "re-evaluation");
+            B_LAUNCH(launch_b_scan(q, kScanSwitch, s), 1, "scan");
+            B_LAUNCH(launch_b_evaluation(q, s), 1, "re-evaluation");
             B_LAUNCH(launch_b_row_tasks(q, max_n_, s), 1, "row tasks");
             B_LAUNCH(launch_b_prepare_edges(rows, s), 1, "prepare");
             B_LAUNCH(launch_b_controller(one, s), 1, "controller");
@@ -565,7 +564,7 @@ struct dgs_server {
     int32_t* h_sigma = nullptr;      // pinned staging for results (worker only)
     size_t h_sigma_cap = 0;
 
-    explicit dgs_server(int32_t cap) : eng(cap, DGS_BATCH_MAX_N), slots(cap) {}
+    explicit dgs_server(int32_t cap) : eng(cap, std::min(DGS_BATCH_MAX_N, solo_min_n() - 1)), slots(cap) {}
 
     // Layout of a large request's memory: the n x n matrix, the result,
     // the start.

@@ -198,22 +198,57 @@ __device__ __forceinline__ void for_each_item(const Instance* inst, const int32_
     }
 }
 
-// Blocks (work items) of the batched pass 1 and evaluation of an instance of
-// size n.  Only the scan kernel uses them; any count is correct (items are
-// spread over whatever grid consumes the queue), the caps only bound how
-// finely one instance is split.
+// The slot k with off[k] <= g < off[k + 1] (off as above, 0 <= g < off[cap]):
+// 32 probes at a time, by a whole warp, every lane with the same g.
+__device__ __forceinline__ int32_t find_slot(const int32_t* off, int32_t cap, int32_t g) {
+    const int lane = threadIdx.x & 31;
+    int32_t lo = 0, hi = cap;
+    while (hi - lo > 1) {
+        const int32_t step = (hi - lo + 31) / 32;
+        const int32_t probe = lo + (lane + 1) * step;
+        const uint32_t above = __ballot_sync(0xffffffffu, probe >= hi || off[probe] > g);
+        const int k = __ffs(above) - 1;  // (the last probe is at or past hi)
+        hi = min(hi, lo + (k + 1) * step);
+        lo += k * step;
+    }
+    return lo;
+}
+
+// The units of every slot's work (off as above) split into `parts` equal
+// contiguous ranges: f(instance, lo, hi) for the units [lo, hi) of each
+// instance that range `part` covers.  Called by whole warps.
+template <typename F>
+__device__ __forceinline__ void for_each_range(const Instance* inst, const int32_t* off, int32_t cap, int32_t part,
+                                               int32_t parts, F&& f) {
+    const int64_t total = off[cap];
+    int32_t lo = (int32_t)(total * part / parts);
+    const int32_t end = (int32_t)(total * (part + 1) / parts);
+    if (lo >= end) return;
+    for (int32_t k = find_slot(off, cap, lo); lo < end; ++k) {
+        const int32_t first = off[k], next = min(end, off[k + 1]);
+        if (next <= lo) continue;
+        f(inst[k], lo - first, next - first);
+        lo = next;
+    }
+}
+
+// Blocks (work items) of the batched pass 1 of an instance of size n.  Only
+// the scan kernel uses them; any count is correct (items are spread over
+// whatever grid consumes the queue), the cap only bounds how finely one
+// instance is split.
 constexpr int32_t kBatchPass1MaxBlocks = 1216;
-constexpr int32_t kBatchEvalMaxBlocks = 152;
 __host__ __device__ __forceinline__ int32_t batch_blocks_pass1(int32_t n) {
     const int32_t t = (n + 63) / 64;
     const int32_t b = (t * t + 3) / 4;
     return b < 1 ? 1 : (b > kBatchPass1MaxBlocks ? kBatchPass1MaxBlocks : b);
 }
-__host__ __device__ __forceinline__ int32_t batch_blocks_eval(int32_t n, int32_t strip) {
-    const int32_t nb = (n + 63) / 64, chunks = (nb + strip - 1) / strip;
-    const int32_t b = (nb * chunks + 1) / 2;
-    return b < 1 ? 1 : (b > kBatchEvalMaxBlocks ? kBatchEvalMaxBlocks : b);
+// Units of the evaluation (64 x 64 tile pairs) and of one row task (n / 32
+// columns, and the latency that any row costs).
+__host__ __device__ __forceinline__ int32_t eval_tiles(int32_t n) {
+    const int32_t nb = (n + 63) / 64;
+    return nb * (nb + 1) / 2;
 }
+__host__ __device__ __forceinline__ int32_t row_weight(int32_t n) { return 16 + (n + 31) / 32; }
 
 // Phases whose work counts the scan kernel computes.
 enum : int32_t { kScanPass1 = 0, kScanGreedyDA = 1, kScanStart = 2, kScanSwitch = 3 };
@@ -386,7 +421,6 @@ cudaError_t launch_small_loop(const Workspace& w, const CtlGlobal& g, cudaStream
 int32_t controller_smem_mode(int32_t n);
 size_t controller_smem_bytes(int32_t n);
 size_t full_evaluation_smem_bytes();
-int32_t evaluation_strip();
 cudaError_t launch_mark_rescan(const Workspace& w, cudaStream_t s);
 cudaError_t launch_prepare_edges(const Workspace& w, cudaStream_t s);
 cudaError_t launch_row_tasks(const Workspace& w, cudaStream_t s);
@@ -429,12 +463,12 @@ struct BatchQueues {
     int32_t* q0;
     int32_t* q1;
 };
-cudaError_t launch_b_scan(const BatchQueues& q, int32_t phase, int32_t strip, cudaStream_t s);
+cudaError_t launch_b_scan(const BatchQueues& q, int32_t phase, cudaStream_t s);
 cudaError_t launch_b_init(const BatchTable& rows, cudaStream_t s);
 cudaError_t launch_b_pass1(const BatchQueues& q, cudaStream_t s);
 cudaError_t launch_b_greedy(const BatchTable& rows, const BatchQueues& q, cudaStream_t s);
 cudaError_t launch_b_start(const BatchTable& rows, cudaStream_t s);
-cudaError_t launch_b_evaluation(const BatchQueues& q, int32_t strip, cudaStream_t s);
+cudaError_t launch_b_evaluation(const BatchQueues& q, cudaStream_t s);
 cudaError_t launch_b_mark_rescan(const BatchTable& rows, cudaStream_t s);
 cudaError_t launch_b_row_tasks(const BatchQueues& q, int32_t max_n, cudaStream_t s);
 cudaError_t launch_b_prepare_edges(const BatchTable& rows, cudaStream_t s);

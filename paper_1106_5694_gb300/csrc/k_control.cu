@@ -1112,11 +1112,9 @@ __device__ __forceinline__ void row_task_compute(const Workspace& w, int32_t j, 
             bs = gt ? sk : (eq ? min(bs, sk) : bs);
             bc = gt ? k : bc;
             bg = max(bg, g);
-            if (scatter && g > 0 && k != j) {
-                if (g >= key_gain(w.key_a[k])) {
-                    atomicMax(&w.key_a[k], pack_gain(g, (uint32_t)j));
-                    atomicMax(&w.key_j[k], pack_gain(g, (uint32_t)sjj));
-                }
+            if (scatter && g > 0 && k != j && g >= key_gain(w.key_a[k])) {
+                atomicMax(&w.key_a[k], pack_gain(g, (uint32_t)j));
+                atomicMax(&w.key_j[k], pack_gain(g, (uint32_t)sjj));
             }
         }
     }
@@ -1203,10 +1201,10 @@ __global__ void __launch_bounds__(512) row_tasks_kernel(Workspace w) {
 }
 
 // Row j of G re-evaluated in full by one warp (the row task of the
-// single-CTA switching loop): the same gains, tie-breaks and scatter into
-// the other rows' keys as row_task_compute, with lane-strided columns (each
-// lane sees its columns in ascending order, so its first maximum is its
-// lowest column, and the packed keys combine across lanes).
+// single-CTA switching loop and of batches): the same gains, tie-breaks and
+// scatter into the other rows' keys as row_task_compute, four columns per lane
+// and step (each lane sees its columns in ascending order, so its first
+// maximum is its lowest column, and the packed keys combine across lanes).
 __device__ __forceinline__ void row_task_warp(const Workspace& w, int32_t j) {
     const int lane = threadIdx.x & 31;
     const int32_t n = w.n;
@@ -1216,15 +1214,27 @@ __device__ __forceinline__ void row_task_warp(const Workspace& w, int32_t j) {
     const int32_t* arow = w.a + (size_t)sjj * w.lda;
     const int32_t* atrow = w.at + (size_t)j * w.ldt;
     int32_t bg = 0, bc = -1, bs = 0x7fffffff;
-    for (int32_t k = lane; k < n; k += 32) {
-        const int32_t sk = w.sigma[k];
-        const int32_t g = arow[k] + atrow[sk] - dj - w.diag[k];
-        const bool gt = g > bg, eq = g == bg;
-        bs = gt ? sk : (eq ? min(bs, sk) : bs);
-        bc = gt ? k : bc;
-        bg = max(bg, g);
-        if (scatter && g > 0 && k != j) {
-            if (g >= key_gain(w.key_a[k])) {
+#pragma unroll 2
+    for (int32_t k0 = lane * 4; k0 < n; k0 += 128) {
+        const int4 x4 = *reinterpret_cast<const int4*>(arow + k0);
+        const int4 s4 = *reinterpret_cast<const int4*>(w.sigma + k0);
+        const int4 d4 = *reinterpret_cast<const int4*>(w.diag + k0);
+        const int32_t xs[4] = {x4.x, x4.y, x4.z, x4.w};
+        const int32_t ss[4] = {s4.x, s4.y, s4.z, s4.w};
+        const int32_t ds[4] = {d4.x, d4.y, d4.z, d4.w};
+        int32_t ys[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) ys[e] = k0 + e < n ? atrow[ss[e]] : 0;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const int32_t k = k0 + e;
+            if (k >= n) break;
+            const int32_t g = xs[e] + ys[e] - dj - ds[e];
+            const bool gt = g > bg, eq = g == bg;
+            bs = gt ? ss[e] : (eq ? min(bs, ss[e]) : bs);
+            bc = gt ? k : bc;
+            bg = max(bg, g);
+            if (scatter && g > 0 && k != j && g >= key_gain(w.key_a[k])) {
                 atomicMax(&w.key_a[k], pack_gain(g, (uint32_t)j));
                 atomicMax(&w.key_j[k], pack_gain(g, (uint32_t)sjj));
             }
@@ -1457,13 +1467,23 @@ __global__ void mark_rescan_batched_kernel(BatchTable t) {
     });
 }
 
-// The rows queued by the kScanSwitch scan (q1): one row task per item, the
-// at row staged by TMA; one mbarrier for the CTA's whole sequence of rows.
-__global__ void __launch_bounds__(512) row_tasks_batched_kernel(BatchQueues q) {
+// The rows queued by the kScanSwitch scan (q1: their weights), every CTA an
+// equal share of the weight; a row by the whole CTA, the at row staged by TMA;
+// one mbarrier for the CTA's whole sequence of rows.  What bounds a row is
+// latency (staging, loads, reduction: 4 to 5 microseconds), and below that the
+// 8 n bytes, so CTAs are small and many per SM where their rows are short
+// (launch_b_row_tasks).  The gather through sigma has to come from shared
+// memory: from L1 it takes a cycle per column (1024 peer-shaped instances, n in
+// [64, 4096], 562k rows: 4.1 ms with a warp per row, 3.7 now; 8.2 ms with
+// 512 threads per row and equal numbers of rows per CTA).
+template <int kT>
+__global__ void __launch_bounds__(kT) row_tasks_batched_kernel(BatchQueues q) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     int32_t* atrow_s = reinterpret_cast<int32_t*>(smem_raw);
     __shared__ unsigned long long red_a[16], red_j[16];
     __shared__ __align__(8) uint64_t bar;
+    __shared__ Workspace w;
+    if (q.q1[q.cap] <= 0) return;
     if (threadIdx.x == 0) {
         mbar_init(&bar, 1);
         fence_mbar_init();
@@ -1471,12 +1491,18 @@ __global__ void __launch_bounds__(512) row_tasks_batched_kernel(BatchQueues q) {
     __syncthreads();
     uint32_t phase = 0;
     bool dead = false;
-    for_each_item(q.inst, q.q1, q.cap, [&](const Instance& in, int32_t t, int32_t) {
+    for_each_range(q.inst, q.q1, q.cap, blockIdx.x, gridDim.x, [&](const Instance& in, int32_t lo, int32_t hi) {
         if (dead) return;
-        const Workspace& w = in.w;
-        if (!row_task_row<true>(w, w.rescan_list[t], atrow_s, &bar, phase, red_a, red_j)) {
-            if (threadIdx.x == 0) { w.st->error = kErrWaitTimeout; w.st->status = kError; }
-            dead = true;  // the buffer may still be written: no further copies into it
+        __syncthreads();  // the copy is no longer read
+        if (threadIdx.x == 0) w = in.w;
+        __syncthreads();
+        const int32_t weight = row_weight(w.n);  // the rows that begin in [lo, hi)
+        for (int32_t r = (lo + weight - 1) / weight; r * weight < hi; ++r) {
+            if (!row_task_row<true>(w, w.rescan_list[r], atrow_s, &bar, phase, red_a, red_j)) {
+                if (threadIdx.x == 0) { w.st->error = kErrWaitTimeout; w.st->status = kError; }
+                dead = true;  // the buffer may still be written: no further copies into it
+                return;
+            }
         }
     });
 }
@@ -1487,10 +1513,10 @@ __global__ void __launch_bounds__(512) row_tasks_batched_kernel(BatchQueues q) {
 //   kScanPass1:  q0 = pass-1 blocks of instances in kStageNew
 //   kScanGreedyDA: q0 = agents of the instances in kStageGreedy (every q1
 //                entry is 0: q1[0] is the deferred acceptance's shared counter)
-//   kScanStart:  q0 = evaluation blocks of instances in kStageStart
-//   kScanSwitch: q0 = evaluation blocks of the updates that re-evaluate every
-//                row, q1 = rows of the updates that use row tasks
-__global__ void __launch_bounds__(1024) scan_batched_kernel(BatchQueues q, int32_t phase, int32_t strip) {
+//   kScanStart:  q0 = evaluation tiles of instances in kStageStart
+//   kScanSwitch: q0 = evaluation tiles of the updates that re-evaluate every
+//                row, q1 = weight of the rows of the updates that use row tasks
+__global__ void __launch_bounds__(1024) scan_batched_kernel(BatchQueues q, int32_t phase) {
     __shared__ int32_t warp_sums[33];
     int32_t carry0 = 0, carry1 = 0;
     for (int32_t c0 = 0; c0 < q.cap; c0 += 1024) {
@@ -1508,15 +1534,15 @@ __global__ void __launch_bounds__(1024) scan_batched_kernel(BatchQueues q, int32
                 } else if (phase == kScanGreedyDA) {
                     if (stage == kStageGreedy && running && st->greedy_remaining > 0) x0 = n;
                 } else if (phase == kScanStart) {
-                    if (stage == kStageStart && running) x0 = batch_blocks_eval(n, strip);
+                    if (stage == kStageStart && running) x0 = eval_tiles(n);
                 } else if (phase == kScanSwitch) {
                     if (stage == kStageSwitch && running && st->need_update) {
                         const int32_t count = st->rescan_count;
                         if (use_full_update(count, n, st->update_policy)) {
-                            x0 = batch_blocks_eval(n, strip);
+                            x0 = eval_tiles(n);
                             st->full_evals += 1;
                         } else {
-                            x1 = count;
+                            x1 = count * row_weight(n);
                             st->row_updates += 1;
                             st->rows_recomputed += count;
                         }
@@ -1756,20 +1782,26 @@ cudaError_t launch_b_mark_rescan(const BatchTable& rows, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-// The row tasks queued in q.q1; max_n bounds every queued instance's n.
-cudaError_t launch_b_row_tasks(const BatchQueues& q, int32_t max_n, cudaStream_t s) {
-    const size_t smem = 4 * (size_t)((max_n + 63) / 64 * 64);
-    if (smem > 48 * 1024) {
-        cudaError_t e = ensure_smem_limit(reinterpret_cast<const void*>(row_tasks_batched_kernel), 6, smem);
-        if (e != cudaSuccess) return e;
-    }
-    const int per_sm = (int)std::min<size_t>(4, (227 * 1024) / (smem + 1024));  // 512 threads, 2048 per SM
-    row_tasks_batched_kernel<<<dgs::device_sms() * (per_sm < 1 ? 1 : per_sm), 512, smem, s>>>(q);
+// max_n: no queued instance is larger.  128 threads per row up to n = 4096 (a
+// row is then at most 16 KB, 13 CTAs per SM), else 512.
+template <int kT>
+static cudaError_t launch_b_row_tasks_t(const BatchQueues& q, size_t smem, int slot, cudaStream_t s) {
+    const void* fn = reinterpret_cast<const void*>(row_tasks_batched_kernel<kT>);
+    cudaError_t e = ensure_smem_limit(fn, slot, smem);
+    if (e != cudaSuccess) return e;
+    const int by_smem = (int)((227 * 1024) / (smem + 2048)), by_threads = 2048 / kT;
+    const int per_sm = std::max(1, std::min({by_smem, by_threads, 13}));
+    row_tasks_batched_kernel<kT><<<dgs::device_sms() * per_sm, kT, smem, s>>>(q);
     return cudaGetLastError();
 }
 
-cudaError_t launch_b_scan(const BatchQueues& q, int32_t phase, int32_t strip, cudaStream_t s) {
-    scan_batched_kernel<<<1, 1024, 0, s>>>(q, phase, strip);
+cudaError_t launch_b_row_tasks(const BatchQueues& q, int32_t max_n, cudaStream_t s) {
+    const size_t smem = 4 * (size_t)((max_n + 63) / 64 * 64);
+    return max_n <= 4096 ? launch_b_row_tasks_t<128>(q, smem, 6, s) : launch_b_row_tasks_t<512>(q, smem, 17, s);
+}
+
+cudaError_t launch_b_scan(const BatchQueues& q, int32_t phase, cudaStream_t s) {
+    scan_batched_kernel<<<1, 1024, 0, s>>>(q, phase);
     return cudaGetLastError();
 }
 

@@ -76,10 +76,14 @@ struct TileCursor {
 //  strip > 0 (strided items): item (J, c) = tiles J + strip*c .. + strip - 1
 //    of row block J, numbered J * chunks + c; block b walks items b, b +
 //    nblk, ...; items past the last tile are empty and skipped.
-//  strip == 0 (contiguous): the tiles in row-major order, split into nblk
-//    equal contiguous ranges; block b walks range b, one row run per row
-//    block it touches.
+//  strip == 0 (contiguous): the tiles [lo, hi) in row-major order, one row run
+//    per row block they touch; a single solve splits all tiles into nblk equal
+//    ranges, a batch the tiles of all its instances.
 // Either way every tile is visited by exactly one block.
+struct Schedule {
+    int32_t strip, bid, nblk;  // strided
+    int32_t lo, hi;            // contiguous
+};
 __device__ __forceinline__ bool cursor_strided(TileCursor& c, int32_t item, int32_t nb, int32_t strip,
                                                int32_t nblk) {
     const int32_t chunks = (nb + strip - 1) / strip;
@@ -102,11 +106,10 @@ __device__ __forceinline__ bool cursor_strided(TileCursor& c, int32_t item, int3
 // first tile of row block J in row-major upper-triangle order
 __device__ __forceinline__ int32_t tri_offset(int32_t J, int32_t nb) { return J * nb - J * (J - 1) / 2; }
 
-__device__ __forceinline__ bool cursor_first(TileCursor& c, int32_t nb, int32_t strip, int32_t bid, int32_t nblk) {
-    if (strip > 0) return cursor_strided(c, bid, nb, strip, nblk);
-    const int64_t total = tri_offset(nb, nb);
-    c.lin = (int32_t)(total * bid / nblk);
-    c.lend = (int32_t)(total * (bid + 1) / nblk);
+__device__ __forceinline__ bool cursor_first(TileCursor& c, int32_t nb, const Schedule& sc) {
+    if (sc.strip > 0) return cursor_strided(c, sc.bid, nb, sc.strip, sc.nblk);
+    c.lin = sc.lo;
+    c.lend = sc.hi;
     if (c.lin >= c.lend) return false;
     int32_t lo = 0, hi = nb;  // tri_offset(lo) <= lin < tri_offset(hi)
     while (hi - lo > 1) {
@@ -120,10 +123,10 @@ __device__ __forceinline__ bool cursor_first(TileCursor& c, int32_t nb, int32_t 
     return true;
 }
 
-__device__ __forceinline__ bool cursor_next(TileCursor& c, int32_t nb, int32_t strip, int32_t nblk) {
-    if (strip > 0) {
+__device__ __forceinline__ bool cursor_next(TileCursor& c, int32_t nb, const Schedule& sc) {
+    if (sc.strip > 0) {
         if (++c.k < c.kend) return true;
-        return cursor_strided(c, c.item + nblk, nb, strip, nblk);
+        return cursor_strided(c, c.item + sc.nblk, nb, sc.strip, sc.nblk);
     }
     if (++c.lin >= c.lend) return false;
     if (++c.k >= nb) {
@@ -476,8 +479,8 @@ constexpr size_t eval_smem_bytes() {
 // tiles arrive by TMA gathers (tm: tensor map over a) tracked by one mbarrier
 // per stage; the Y tiles and the sigma / D rows by 16-byte cp.async.
 template <int kRows, bool kPacked, bool kTma>
-__device__ __forceinline__ void evaluation_loop(const Workspace& w, int32_t strip, int32_t bid, int32_t nblk,
-                                                const Packing& pk, const CUtensorMap* tm) {
+__device__ __forceinline__ void evaluation_loop(const Workspace& w, const Schedule& sc, const Packing& pk,
+                                                const CUtensorMap* tm) {
     constexpr int kGroups = Geo<kRows>::kGroups;
     constexpr int kStages = stages_for(kRows);
     extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -503,7 +506,7 @@ __device__ __forceinline__ void evaluation_loop(const Workspace& w, int32_t stri
     // producer cursor: kStages - 1 tiles ahead of the consumer; the rows
     // (sigma) it will copy are loaded two tiles before they are needed
     TileCursor prod;
-    bool prod_ok = cursor_first(prod, nb, strip, bid, nblk);
+    bool prod_ok = cursor_first(prod, nb, sc);
     for (int s = 0; s < kStages - 1; ++s) {
         if (prod_ok) {
             if (!kTma && prod.j != xr_j) {
@@ -519,17 +522,17 @@ __device__ __forceinline__ void evaluation_loop(const Workspace& w, int32_t stri
                 }
                 gather_x(&stages[s], tm, prod.k * kT, xs, &s_bar[s]);
             }
-            prod_ok = cursor_next(prod, nb, strip, nblk);
+            prod_ok = cursor_next(prod, nb, sc);
         }
         cp_async_commit();
     }
     TileCursor ahead = prod;  // one tile after prod
-    bool ahead_ok = prod_ok && cursor_next(ahead, nb, strip, nblk);
+    bool ahead_ok = prod_ok && cursor_next(ahead, nb, sc);
     CopyRows<kRows> rows_now = prod_ok ? copy_rows<kRows, kTma>(w, prod.j, prod.k) : no_rows<kRows>();
     CopyRows<kRows> rows_next = ahead_ok ? copy_rows<kRows, kTma>(w, ahead.j, ahead.k) : no_rows<kRows>();
 
     TileCursor cons;
-    bool cons_ok = cursor_first(cons, nb, strip, bid, nblk);
+    bool cons_ok = cursor_first(cons, nb, sc);
     Rows<kRows, kPacked> rs;
     bool item_start = true;
     int32_t t = 0, prev_k0 = -1;
@@ -579,7 +582,7 @@ __device__ __forceinline__ void evaluation_loop(const Workspace& w, int32_t stri
             prod_ok = ahead_ok;
             rows_now = rows_next;
             if (ahead_ok) {
-                ahead_ok = cursor_next(ahead, nb, strip, nblk);
+                ahead_ok = cursor_next(ahead, nb, sc);
                 if (ahead_ok) rows_next = copy_rows<kRows, kTma>(w, ahead.j, ahead.k);
             }
         }
@@ -596,7 +599,7 @@ __device__ __forceinline__ void evaluation_loop(const Workspace& w, int32_t stri
             cs = 0;
             cph ^= 1u;
         }
-        cons_ok = cursor_next(cons, nb, strip, nblk);
+        cons_ok = cursor_next(cons, nb, sc);
         item_start = run_end;
     }
     cp_async_wait<0>();
@@ -610,31 +613,42 @@ __device__ __forceinline__ void evaluation_loop(const Workspace& w, int32_t stri
 // it (a CTA of the single-instance launch, or one item of a batched queue).
 // All threads of the CTA call it together.
 template <int kRows, bool kTma = false>
-__device__ __forceinline__ void full_evaluation_body(const Workspace& w, int32_t conditional, int32_t strip,
-                                                     int32_t bid, int32_t nblk, const CUtensorMap* tm = nullptr) {
+__device__ __forceinline__ void full_evaluation_body(const Workspace& w, int32_t conditional, const Schedule& sc,
+                                                     const CUtensorMap* tm = nullptr) {
     DeviceState* st = w.st;
     if (st->status != kRunning) return;
     if (conditional && !(st->need_update && use_full_update(st->rescan_count, w.n, st->update_policy))) return;
-    if (conditional && bid == 0 && threadIdx.x == 0) st->full_evals += 1;
+    if (conditional && blockIdx.x == 0 && threadIdx.x == 0) st->full_evals += 1;
     const Packing pk = packing_for(w.n, st->max_abs);
-    if (pk.pw != 0 && !w.exact_keys) evaluation_loop<kRows, true, kTma>(w, strip, bid, nblk, pk, tm);
-    else evaluation_loop<kRows, false, kTma>(w, strip, bid, nblk, pk, tm);
+    if (pk.pw != 0 && !w.exact_keys) evaluation_loop<kRows, true, kTma>(w, sc, pk, tm);
+    else evaluation_loop<kRows, false, kTma>(w, sc, pk, tm);
 }
 
 template <int kRows, bool kTma>
 __global__ void __launch_bounds__(Geo<kRows>::kThreads, 1) full_evaluation_kernel(Workspace w, int32_t conditional,
                                                                                   int32_t strip,
                                                                                   const __grid_constant__ CUtensorMap tm) {
-    full_evaluation_body<kRows, kTma>(w, conditional, strip, blockIdx.x, gridDim.x, &tm);
+    const int64_t total = eval_tiles(w.n);
+    const Schedule sc{strip, (int32_t)blockIdx.x, (int32_t)gridDim.x, (int32_t)(total * blockIdx.x / gridDim.x),
+                      (int32_t)(total * (blockIdx.x + 1) / gridDim.x)};
+    full_evaluation_body<kRows, kTma>(w, conditional, sc, &tm);
 }
 
-// Batched: each queue item is one block of one instance's evaluation (the
-// scan kernel queued exactly the instances that need one).
+// Batched: the tiles of every instance that needs an evaluation (queued by the
+// scan kernel) in one order, an equal contiguous range of them per CTA, so
+// that the pipeline is filled once per instance and CTA.  (Items of two strips
+// of eight tiles, equal numbers of items per CTA: 1024 peer-shaped instances,
+// n in [64, 4096], 5.6 ms, now 3.5.)
 template <int kRows>
-__global__ void __launch_bounds__(Geo<kRows>::kThreads, 1) full_evaluation_batched_kernel(BatchQueues q,
-                                                                                          int32_t strip) {
-    for_each_item(q.inst, q.q0, q.cap, [&](const Instance& in, int32_t bid, int32_t nblk) {
-        full_evaluation_body<kRows>(in.w, 0, strip, bid, nblk);
+__global__ void __launch_bounds__(Geo<kRows>::kThreads, 1) full_evaluation_batched_kernel(BatchQueues q) {
+    // (a copy: pointers read from global memory would be read again after
+    // every key update, which might have changed them)
+    __shared__ Workspace w;
+    for_each_range(q.inst, q.q0, q.cap, blockIdx.x, gridDim.x, [&](const Instance& in, int32_t lo, int32_t hi) {
+        __syncthreads();  // the copy is no longer read
+        if (threadIdx.x == 0) w = in.w;
+        __syncthreads();
+        full_evaluation_body<kRows>(w, 0, Schedule{0, 0, 1, lo, hi});
     });
 }
 
@@ -758,16 +772,13 @@ cudaError_t launch_full_evaluation(const Workspace& w, int32_t conditional, cuda
     return launch_full_evaluation_shape(w, conditional, evaluation_shape(w.n), s);
 }
 
-int32_t evaluation_strip() { return kStrip; }
-
-// The evaluations queued in q.q0 (batch_blocks_eval(n, strip) blocks each),
-// 512 threads per CTA (the 1024-thread variant would spill the instance's
+// The evaluations queued in q.q0 (eval_tiles(n) units each), 512 threads per CTA (the 1024-thread variant would spill the instance's
 // workspace pointers it reads from global memory).
-cudaError_t launch_b_evaluation(const BatchQueues& q, int32_t strip, cudaStream_t s) {
+cudaError_t launch_b_evaluation(const BatchQueues& q, cudaStream_t s) {
     constexpr size_t smem = eval_smem_bytes<8>();
     cudaError_t e = ensure_smem_limit(reinterpret_cast<const void*>(full_evaluation_batched_kernel<8>), 4, smem);
     if (e != cudaSuccess) return e;
-    full_evaluation_batched_kernel<8><<<dgs::device_sms(), Geo<8>::kThreads, smem, s>>>(q, strip);
+    full_evaluation_batched_kernel<8><<<dgs::device_sms(), Geo<8>::kThreads, smem, s>>>(q);
     return cudaGetLastError();
 }
 

@@ -27,6 +27,13 @@ constexpr int kT = 64;  // tile edge
 // What pass 1 computes beside the transposed copy and the range check.
 enum : int { kPass1Plain = 0, kPass1Bounds = 1, kPass1Rounds = 2 };
 
+// The maximum `top` of agent i's biased benefits in the 64 columns from J0 on.
+__device__ __forceinline__ void put_bound(const Workspace& w, int32_t i, int32_t J0, uint32_t top) {
+    uint32_t* b = w.g_bound + (size_t)i * w.bound_tiles + (J0 >> w.bound_shift);
+    if (w.bound_shift == kBoundShift) *b = top;
+    else atomicMax(b, top);
+}
+
 // a_src (batched instances only): the caller's matrix with row pitch n when w.a
 // is the workspace's pitched copy still to be filled; this pass reads a_src
 // and writes the copy as it goes.  Null: w.a is read.
@@ -43,23 +50,46 @@ __device__ __forceinline__ void greedy_pass1_body(const Workspace& w, int32_t ti
     for (int32_t tile = bid; tile < tiles_total; tile += nblk) {
         const int32_t I0 = (tile / tiles_x) * kT;
         const int32_t J0 = (tile % tiles_x) * kT;
+        if (a_src != nullptr) {
+            // rows of n int32 from any 4-byte boundary: a warp per row, two
+            // loads of 32 consecutive columns; the pitched copy (padding
+            // columns 0) is written from shared memory below
+            const int lane = t & 31;
+            int32_t x[8][2];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                const int32_t i = I0 + (t >> 5) + 8 * q;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int32_t j = J0 + lane + 32 * h;
+                    x[q][h] = i < n && j < n ? a_src[(size_t)i * n + j] : 0;
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                const int r = (t >> 5) + 8 * q;
+                uint32_t top = 0;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    s[r][lane + 32 * h] = x[q][h];
+                    if (J0 + lane + 32 * h < n) {
+                        bad |= (x[q][h] >= kBenefitLimit) || (x[q][h] <= -kBenefitLimit);
+                        amax = max(amax, x[q][h] == INT32_MIN ? INT32_MAX : abs(x[q][h]));
+                        top = max(top, (uint32_t)(x[q][h] + kBenefitLimit));
+                    }
+                }
+                top = __reduce_max_sync(0xffffffffu, top);
+                if (kMode == kPass1Bounds && lane == 0 && I0 + r < n) put_bound(w, I0 + r, J0, top);
+            }
+        }
         // load 64 rows x 64 cols with int4, 16 threads per row, 4 passes
 #pragma unroll
-        for (int p = 0; p < 4; ++p) {
+        for (int p = 0; p < 4 && a_src == nullptr; ++p) {
             const int r = (t >> 4) + 16 * p;
             const int c = lane16 * 4;
             const int32_t i = I0 + r, j = J0 + c;
             int4 v = make_int4(0, 0, 0, 0);
-            if (a_src == nullptr) {
-                if (i < n && j < w.lda) v = *reinterpret_cast<const int4*>(w.a + (size_t)i * w.lda + j);
-            } else if (i < n && j < w.lda) {  // re-pitch: unaligned reads, padding columns 0
-                const int32_t* src = a_src + (size_t)i * n + j;
-                v.x = j < n ? src[0] : 0;
-                v.y = j + 1 < n ? src[1] : 0;
-                v.z = j + 2 < n ? src[2] : 0;
-                v.w = j + 3 < n ? src[3] : 0;
-                *reinterpret_cast<int4*>(const_cast<int32_t*>(w.a) + (size_t)i * w.lda + j) = v;
-            }
+            if (i < n && j < w.lda) v = *reinterpret_cast<const int4*>(w.a + (size_t)i * w.lda + j);
             s[r][c + 0] = v.x; s[r][c + 1] = v.y; s[r][c + 2] = v.z; s[r][c + 3] = v.w;
             // row best over this tile's 4 columns of this thread
             unsigned long long best = 0;
@@ -82,11 +112,7 @@ __device__ __forceinline__ void greedy_pass1_body(const Workspace& w, int32_t ti
             } else if (kMode == kPass1Bounds) {
 #pragma unroll
                 for (int off = 8; off > 0; off >>= 1) top = max(top, __shfl_xor_sync(0xffffffffu, top, off));
-                if (lane16 == 0 && i < n) {
-                    uint32_t* ub = w.g_bound + (size_t)i * w.bound_tiles + (J0 >> w.bound_shift);
-                    if (w.bound_shift == kBoundShift) *ub = top;
-                    else atomicMax(ub, top);
-                }
+                if (lane16 == 0 && i < n) put_bound(w, i, J0, top);
             }
         }
         __syncthreads();
@@ -104,6 +130,15 @@ __device__ __forceinline__ void greedy_pass1_body(const Workspace& w, int32_t ti
             }
             colpart[g][c] = best;
         }
+        if (a_src != nullptr) {
+#pragma unroll
+            for (int p = 0; p < 4; ++p) {
+                const int r = (t >> 4) + 16 * p, c = lane16 * 4;
+                if (I0 + r < n && J0 + c < w.lda)
+                    *reinterpret_cast<int4*>(const_cast<int32_t*>(w.a) + (size_t)(I0 + r) * w.lda + J0 + c) =
+                        make_int4(s[r][c], s[r][c + 1], s[r][c + 2], s[r][c + 3]);
+            }
+        }
         // transposed store: at row j = J0 + jr, 4 agents per thread
 #pragma unroll
         for (int p = 0; p < 4; ++p) {
@@ -117,7 +152,8 @@ __device__ __forceinline__ void greedy_pass1_body(const Workspace& w, int32_t ti
             }
         }
         __syncthreads();
-        if (kMode == kPass1Rounds && t < kT) {
+        if (kMode != kPass1Rounds) continue;
+        if (t < kT) {
             const int32_t j = J0 + t;
             unsigned long long best = umax64(umax64(colpart[0][t], colpart[1][t]), umax64(colpart[2][t], colpart[3][t]));
             if (j < n && best != 0) atomicMax(&w.g_col[j], best);
@@ -639,8 +675,9 @@ __global__ void range_check_kernel(Workspace w) {
 
 __global__ void __launch_bounds__(256) greedy_pass1_batched_kernel(BatchQueues q) {
     for_each_item(q.inst, q.q0, q.cap, [&](const Instance& in, int32_t bid, int32_t nblk) {
-        const int32_t tx = (in.w.n + kT - 1) / kT;
-        greedy_pass1_body<kPass1Bounds>(in.w, tx, tx * tx, bid, nblk, in.a_src);
+        const Workspace w = in.w;
+        const int32_t tx = (w.n + kT - 1) / kT;
+        greedy_pass1_body<kPass1Bounds>(w, tx, tx * tx, bid, nblk, in.a_src);
     });
 }
 
@@ -673,21 +710,12 @@ __global__ void __launch_bounds__(kDaThreads, kDaPerSm) greedy_da_batched_kernel
     while ((int64_t)chunk * per < total) {
         const int32_t g_end = min(total, (chunk + 1) * per);
         for (int32_t g = chunk * per; g < g_end; ++g) {
-            if (g < first || g >= end) {  // another instance: q0[lo] <= g < q0[lo + 1], 32 probes at a time
+            if (g < first || g >= end) {  // another instance
                 flush();
-                int32_t lo = 0, hi = q.cap;
-                while (hi - lo > 1) {
-                    const int32_t step = (hi - lo + 31) / 32;
-                    const int32_t probe = lo + (lane + 1) * step;
-                    const uint32_t above = __ballot_sync(0xffffffffu, probe >= hi || q.q0[probe] > g);
-                    const int k = __ffs(above) - 1;  // (the last probe is at or past hi)
-                    hi = min(hi, lo + (k + 1) * step);
-                    lo += k * step;
-                }
-                k_last = lo;
-                first = q.q0[lo];
-                end = q.q0[lo + 1];
-                d = da_view(q.inst[lo].w);
+                k_last = find_slot(q.q0, q.cap, g);
+                first = q.q0[k_last];
+                end = q.q0[k_last + 1];
+                d = da_view(q.inst[k_last].w);
             }
             int32_t a = g - first, r, steps = 1;
             while ((r = da_propose<1>(d, a, s_b, s_sh[warp], warp, 0, looks)) >= 0) {
@@ -796,7 +824,7 @@ int32_t da_grid(size_t smem) {
 // queue the agents, one launch, then the assignments; the advance kernel
 // moves the instances on once greedy_remaining is 0).
 cudaError_t launch_b_greedy(const BatchTable& rows, const BatchQueues& q, cudaStream_t s) {
-    cudaError_t e = launch_b_scan(q, kScanGreedyDA, 0, s);
+    cudaError_t e = launch_b_scan(q, kScanGreedyDA, s);
     if (e != cudaSuccess) return e;
     greedy_da_batched_kernel<<<da_grid(0), kDaThreads, 0, s>>>(q);
     e = cudaGetLastError();
