@@ -438,8 +438,10 @@ DGS_API dgs_status dgs_read_bandwidth(const void* buffer, size_t bytes, int32_t 
  * their device memory from the library's own stream-ordered pool on the
  * current device, which keeps freed memory cached for the next call instead of
  * returning it to the device (back-to-back solves then reuse their workspace
- * instead of mapping it again).  dgs_release_cached_memory returns every
- * cached byte of those pools to the device; memory still in use by a call in
+ * instead of mapping it again); dgs_solve_batched also keeps up to four of its
+ * engines (work tables, pinned staging and step graph, about 3 KB per
+ * instance).  dgs_release_cached_memory returns every cached byte of those
+ * pools and engines to the device; memory still in use by a call in
  * flight stays with it.  Errors: DGS_ERR_CUDA if a trim failed. */
 DGS_API dgs_status dgs_release_cached_memory(void);
 

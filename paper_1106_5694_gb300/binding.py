@@ -85,6 +85,12 @@ class dgs_stats(ctypes.Structure):
         ("solve_ms", ctypes.c_double),
     ]
 
+    @classmethod
+    def dicts(cls, array):
+        """The elements of a ctypes array of dgs_stats as dicts (as as_dict gives one)."""
+        names = [name for name, _ in cls._fields_]
+        return [dict(zip(names, row)) for row in np.frombuffer(array, dtype=np.dtype(cls)).tolist()]
+
     def as_dict(self):
         return {name: (float if name.endswith("_ms") else int)(getattr(self, name)) for name, _ in self._fields_}
 
@@ -423,7 +429,7 @@ def dgs_solve_batched(benefits, sigma_outs=None, stream=None, **opts):
     o = _options(**opts)
     st = load().dgs_solve_batched(a_ptrs, ns, count, o_ptrs, objs, ctypes.byref(o), statuses, stats,
                                   _stream(benefits[0], stream))
-    return st, sigma_outs, [int(x) for x in objs], [int(x) for x in statuses], [s.as_dict() for s in stats]
+    return st, sigma_outs, list(objs), list(statuses), dgs_stats.dicts(stats)
 
 
 def dgs_server_request_bytes(n: int) -> int:

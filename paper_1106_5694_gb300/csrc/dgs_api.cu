@@ -1160,6 +1160,7 @@ const char* dgs_last_cuda_error(void) { return g_last_error; }
 }  // extern "C"
 
 extern "C" dgs_status dgs_release_cached_memory(void) {
+    dgs::release_cached_engines();
     std::lock_guard<std::mutex> lock(dgs::g_pool_mutex);
     dgs_status st = DGS_OK;
     for (int d = 0; d < 64; ++d) {

@@ -32,6 +32,7 @@
 #include <mutex>
 #include <thread>
 #include <unordered_map>
+#include <utility>
 #include <vector>
 
 #include "../../include/dgs.h"
@@ -229,6 +230,13 @@ class Engine {
 
     int64_t steps() const { return steps_; }
 
+    // Every slot free again, for another batch (nothing may be in flight).
+    void clear() {
+        for (int32_t k = 0; k < cap_; ++k)
+            if (used_[k]) vacate(k);
+        steps_ = 0;
+    }
+
   private:
     BatchTable table(int32_t t) const {
         return BatchTable{d_inst_, d_ent_ + off_[t], d_cnt_ + t};
@@ -338,6 +346,95 @@ class Engine {
     int64_t steps_ = 0;
 };
 
+// Engines of finished dgs_solve_batched calls, kept for later ones of the same
+// device, capacity and size class (their tables, pinned staging and step graph
+// took 1.5 ms to set up and tear down, most of a small batch).  An engine
+// belongs to one call at a time, so calls from several threads run on engines
+// of their own; at most kKeep wait here, none of more than kKeepCapacity
+// slots (about 3 KB each), and dgs_release_cached_memory gives them back.  (Not
+// destroyed at exit, when the CUDA runtime may be gone.)
+class EngineCache {
+  public:
+    struct Key {
+        int dev;
+        int32_t cap, max_n, colour;  // colour: a knob that the step graph bakes in
+        bool operator==(const Key& o) const {
+            return dev == o.dev && cap == o.cap && max_n == o.max_n && colour == o.colour;
+        }
+    };
+    static EngineCache& get() {
+        static EngineCache* c = new EngineCache();
+        return *c;
+    }
+    Engine* take(const Key& key) {
+        std::lock_guard<std::mutex> lock(mu_);
+        for (size_t i = 0; i < free_.size(); ++i)
+            if (free_[i].first == key) {
+                Engine* e = free_[i].second;
+                free_.erase(free_.begin() + (long)i);
+                return e;
+            }
+        return nullptr;
+    }
+    void put(const Key& key, Engine* e) {  // the longest waiting one goes
+        e->clear();
+        Engine* drop = key.cap > kKeepCapacity ? e : nullptr;
+        if (drop == nullptr) {
+            std::lock_guard<std::mutex> lock(mu_);
+            free_.emplace_back(key, e);
+            if (free_.size() > kKeep) {
+                drop = free_.front().second;
+                free_.erase(free_.begin());
+            }
+        }
+        delete drop;
+    }
+    void release() {
+        std::vector<std::pair<Key, Engine*>> all;
+        {
+            std::lock_guard<std::mutex> lock(mu_);
+            all.swap(free_);
+        }
+        for (auto& x : all) delete x.second;
+    }
+
+  private:
+    static constexpr size_t kKeep = 4;
+    static constexpr int32_t kKeepCapacity = 4096;
+    std::mutex mu_;
+    std::vector<std::pair<Key, Engine*>> free_;
+};
+
+// The engine of one call: from the cache, or new; back to the cache when the
+// call has finished with it, destroyed when the call failed.
+struct EngineLease {
+    EngineCache::Key key{};
+    Engine* e = nullptr;
+    bool finished = false;
+    dgs_status acquire(int32_t count, int32_t max_n) {
+        // classes: 16 slots, then steps of a half or a third; sizes likewise
+        const auto round = [](int32_t x, int32_t from) {
+            int32_t c = from;
+            for (int i = 0; c < x; ++i) c = (i & 1) ? c / 3 * 4 : c / 2 * 3;
+            return c;
+        };
+        cudaError_t err = cudaGetDevice(&key.dev);
+        if (err != cudaSuccess) return fail(err, "cudaGetDevice");
+        key.cap = round(count, 16);
+        key.max_n = std::min(round(max_n, 256), (int32_t)DGS_BATCH_MAX_N);
+        key.colour = env_colour_pass();
+        e = EngineCache::get().take(key);
+        if (e != nullptr) return DGS_OK;
+        e = new Engine(key.cap, key.max_n);
+        return e->init();
+    }
+    ~EngineLease() {
+        if (e == nullptr) return;
+        if (finished) EngineCache::get().put(key, e);
+        else delete e;
+    }
+};
+
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 // Upper bound on the steps of one instance: the greedy start ends within its
@@ -366,6 +463,8 @@ int64_t now_ns() {
 }
 
 }  // namespace
+
+void release_cached_engines() { EngineCache::get().release(); }
 }  // namespace dgs
 
 using namespace dgs;
@@ -389,9 +488,10 @@ extern "C" dgs_status dgs_solve_batched(const int32_t* const* benefits, const in
         max_n = std::max(max_n, ns[k]);
     }
     cudaStream_t user = reinterpret_cast<cudaStream_t>(stream);
-    Engine eng(count, max_n);
-    dgs_status st = eng.init();
+    EngineLease lease;
+    dgs_status st = lease.acquire(count, max_n);
     if (st != DGS_OK) return st;
+    Engine& eng = *lease.e;
     cudaStream_t s = eng.stream();
     // the private stream starts after the caller's stream
     cudaEvent_t ev = nullptr;
@@ -476,6 +576,7 @@ extern "C" dgs_status dgs_solve_batched(const int32_t* const* benefits, const in
     }
     dgs_status first = DGS_OK;
     const int64_t launches = eng.launches_per_step() * eng.steps();
+    lease.finished = true;  // (its states are read until the lease ends)
     for (int32_t k = 0; k < count; ++k) {
         const DeviceState& h = eng.state(k);
         const dgs_status sk = status_of(h);

@@ -444,6 +444,8 @@ cudaError_t launch_seq_pass_end(const Workspace& w, unsigned long long outer, cu
 cudaError_t launch_slots_from_keys(const Workspace& w, cudaStream_t s);
 cudaError_t launch_sequential(const Workspace& w, cudaStream_t s);
 
+// Engines kept by finished batched calls, given back (dgs_release_cached_memory).
+void release_cached_engines();
 size_t carve_instance(char* base, int32_t n, bool need_copy, Instance* in);
 // One stream-ordered single solve (dgs_solve_ex) for the server's large
 // requests; *final_status gets the outcome when the stream reaches it.
