@@ -312,6 +312,7 @@ struct Solve {
     Workspace w{};
     Plan plan;
     int32_t* a_copy = nullptr;
+    const int32_t* a_src = nullptr;  // not null: the caller's matrix, from which pass 1 fills w.a
     CtlGlobal ctl{};
     uint8_t* seen = nullptr;
     int64_t launches = 0;
@@ -344,24 +345,12 @@ struct Solve {
         w.lda = plan.lda;
         w.ldt = plan.ldt;
         w.exact_keys = env_exact_keys();
-        if (plan.need_copy) {
-            e = cudaMemsetAsync(a_copy, 0, (size_t)n * plan.lda * sizeof(int32_t), s);
-            if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync");
-            e = cudaMemcpy2DAsync(a_copy, (size_t)plan.lda * 4, a, (size_t)n * 4, (size_t)n * 4, n,
-                                  cudaMemcpyDeviceToDevice, s);
-            if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpy2DAsync");
-            w.a = a_copy;
-        } else {
-            w.a = a;
-        }
+        w.a = plan.need_copy ? a_copy : a;  // (the copy is filled by the pass that reads the matrix anyway)
+        a_src = plan.need_copy ? a : nullptr;
         // zero every small array in one go (they follow a/at in the arena)
         char* small_begin = reinterpret_cast<char*>(w.sigma);
         const size_t small_bytes = (size_t)(ar.base + ar.used - small_begin);
         e = cudaMemsetAsync(small_begin, 0, small_bytes, s);
-        if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync");
-        const size_t nb = align_up((size_t)n, 128);
-        e = cudaMemsetAsync(w.free_a, 1, nb, s);
-        if (e == cudaSuccess) e = cudaMemsetAsync(w.free_j, 1, nb, s);
         if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync");
         return DGS_OK;
     }
@@ -449,14 +438,22 @@ __global__ void arm_deadline_kernel(DeviceState* st, int64_t deadline_us) {
     st->deadline_ns = now + (uint64_t)deadline_us * 1000ull;
 }
 
-__global__ void record_initial_objective_kernel(DeviceState* st) { st->f_initial = st->f; }
-
 // Rectangular instance -> square instance of size s (zero-benefit dummies).
-__global__ void pad_square_kernel(const int32_t* a, int32_t n, int32_t m, int32_t s, int32_t* sq) {
-    const size_t total = (size_t)s * s;
-    for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < total; q += (size_t)gridDim.x * blockDim.x) {
-        const int32_t i = (int32_t)(q / s), j = (int32_t)(q - (size_t)i * s);
-        sq[q] = (i < n && j < m) ? a[(size_t)i * m + j] : 0;
+// A warp per row, 32 consecutive columns at a time.
+__global__ void __launch_bounds__(256) pad_square_kernel(const int32_t* a, int32_t n, int32_t m, int32_t s,
+                                                         int32_t* sq) {
+    const int32_t lane = threadIdx.x & 31, warps = gridDim.x * (blockDim.x / 32);
+    for (int32_t i = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5); i < s; i += warps) {
+        const int32_t real = i < n ? m : 0;
+        constexpr int kAhead = 8;
+        for (int32_t j = lane; j < s; j += 32 * kAhead) {
+            int32_t x[kAhead];
+#pragma unroll
+            for (int k = 0; k < kAhead; ++k) x[k] = j + 32 * k < real ? a[(size_t)i * m + j + 32 * k] : 0;
+#pragma unroll
+            for (int k = 0; k < kAhead; ++k)
+                if (j + 32 * k < s) sq[(size_t)i * s + j + 32 * k] = x[k];
+        }
     }
 }
 
@@ -630,14 +627,16 @@ struct HostBands {
     int32_t tile_rows;
 };
 
-dgs_status run_greedy(Solve& S, EventPair* timer, const HostBands* bands = nullptr) {
+// *started: the start (sigma, D, f) is there too; else only tau and sigma are.
+dgs_status run_greedy(Solve& S, EventPair* timer, bool* started, const HostBands* bands = nullptr) {
+    *started = true;
     if (bands == nullptr) {
-        DGS_CUDA(launch_greedy_pass1_bounds(S.w, 0, (S.w.n + 63) / 64, S.s), "greedy pass 1");
+        DGS_CUDA(launch_greedy_pass1_bounds(S.w, 0, (S.w.n + 63) / 64, S.a_src, S.s), "greedy pass 1");
         S.launches += 1;
     } else {  // pass 1 of each band as soon as it has landed, while later ones are still copied
         for (int32_t k = 0; k < bands->count; ++k) {
             DGS_CUDA(cudaStreamWaitEvent(S.s, bands->ev[k], 0), "wait for a band of the matrix");
-            DGS_CUDA(launch_greedy_pass1_bounds(S.w, k * bands->tile_rows, (k + 1) * bands->tile_rows, S.s),
+            DGS_CUDA(launch_greedy_pass1_bounds(S.w, k * bands->tile_rows, (k + 1) * bands->tile_rows, nullptr, S.s),
                      "greedy pass 1");
             S.launches += 1;
         }
@@ -650,6 +649,10 @@ dgs_status run_greedy(Solve& S, EventPair* timer, const HostBands* bands = nullp
         return DGS_OK;
     }
     cudaGetLastError();
+    *started = false;
+    const size_t nb = align_up((size_t)S.w.n, 128);
+    DGS_CUDA(cudaMemsetAsync(S.w.free_a, 1, nb, S.s), "free agents");
+    DGS_CUDA(cudaMemsetAsync(S.w.free_j, 1, nb, S.s), "free jobs");
     DGS_CUDA(launch_greedy_pass1_rounds(S.w, S.s), "greedy pass 1");
     S.launches += 1;
     LoopCtx c{S.w, S.ctl};
@@ -802,15 +805,17 @@ dgs_status solve_impl(const int32_t* benefit, int32_t n, int32_t* sigma_out, int
         S.launches += 1;
     }
     EventPair gev;
+    bool started = false;
     if (o.init == DGS_INIT_GREEDY) {
-        DGS_TRY(run_greedy(S, o.profile ? &gev : nullptr, bands));
+        DGS_TRY(run_greedy(S, o.profile ? &gev : nullptr, &started, bands));
     } else {
-        DGS_CUDA(launch_greedy_pass1(S.w, stream), "pass 1");  // transpose + range check
+        DGS_CUDA(launch_greedy_pass1(S.w, S.a_src, stream), "pass 1");  // transpose + range check
         S.launches += 1;
     }
-    DGS_CUDA(launch_start_from_tau(S.w, o.init_sigma, o.init, S.seen, stream), "start");
-    record_initial_objective_kernel<<<1, 1, 0, stream>>>(S.w.st);
-    S.launches += 2;
+    if (!started) {
+        DGS_CUDA(launch_start_from_tau(S.w, o.init_sigma, o.init, S.seen, stream), "start");
+        S.launches += 1;
+    }
     EventPair ev;
     LoopCtx lc{S.w, S.ctl};
     if (o.algorithm == DGS_ALG_SEQUENTIAL) {
@@ -1014,7 +1019,7 @@ dgs_status dgs_evaluate(const int32_t* benefit, int32_t n, const int32_t* sigma_
     Solve S(s);
     DGS_TRY(S.setup(benefit, n, false));
     DGS_TRY(S.init_state(0, nullptr));
-    DGS_CUDA(launch_range_check(S.w, s), "range check");
+    DGS_CUDA(launch_range_check(S.w, S.a_src, s), "range check");
     DGS_CUDA(launch_start_from_tau(S.w, sigma_in, DGS_INIT_USER, S.seen, s), "start");
     DGS_CUDA(launch_full_evaluation(S.w, 0, s), "evaluation");
     DGS_CUDA(launch_keys_to_slots(S.w, agent_gain, agent_job, job_gain, job_agent, s), "keys to slots");
@@ -1030,7 +1035,8 @@ dgs_status dgs_greedy_init(const int32_t* benefit, int32_t n, int32_t* sigma_out
     Solve S(s);
     DGS_TRY(S.setup(benefit, n, true));
     DGS_TRY(S.init_state(0, nullptr));
-    DGS_TRY(run_greedy(S, nullptr));
+    bool started;
+    DGS_TRY(run_greedy(S, nullptr, &started));
     DGS_CUDA(launch_finish(S.w, sigma_out, s), "finish");
     DeviceState h;
     DGS_TRY(S.read_state(&h));
@@ -1072,7 +1078,7 @@ dgs_status dgs_autotune(int32_t n, dgs_tuning* result, dgs_stream_t stream) {
         if (e != cudaSuccess) st = cuda_fail(e, "copy assignment");
         if (st == DGS_OK) st = S.setup_pitched(a, n, lda);
         if (st == DGS_OK) st = S.init_state(0, nullptr);
-        if (st == DGS_OK && (e = launch_range_check(S.w, s)) != cudaSuccess) st = cuda_fail(e, "range check");
+        if (st == DGS_OK && (e = launch_range_check(S.w, nullptr, s)) != cudaSuccess) st = cuda_fail(e, "range check");
         if (st == DGS_OK && (e = launch_start_from_tau(S.w, sigma, DGS_INIT_USER, S.seen, s)) != cudaSuccess)
             st = cuda_fail(e, "start");
         // candidate shapes: 8 and 16 rows per thread with every strip (0:

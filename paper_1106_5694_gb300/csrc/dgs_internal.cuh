@@ -295,6 +295,22 @@ __device__ __forceinline__ unsigned long long umax64(unsigned long long x, unsig
     return x > y ? x : y;
 }
 
+// f += the sum of every thread's x over the CTA, by one atomic (the whole CTA
+// calls it, at most 1024 threads).
+__device__ __forceinline__ void add_objective(DeviceState* st, long long x) {
+    __shared__ long long s_sum[32];
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
+    if ((threadIdx.x & 31) == 0) s_sum[threadIdx.x >> 5] = x;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        long long f = 0;
+        for (int q = 0; q < (int)(blockDim.x >> 5); ++q) f += s_sum[q];
+        if (f != 0) atomicAdd(reinterpret_cast<unsigned long long*>(&st->f), (unsigned long long)f);
+    }
+    __syncthreads();  // s_sum may be written again
+}
+
 __device__ __forceinline__ uint64_t globaltimer_ns() {
     uint64_t t;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
@@ -382,17 +398,22 @@ __device__ __forceinline__ bool grid_barrier(DeviceState* st) {
 // Pass 1: the transposed copy and the range check alone; with the bounds of
 // deferred acceptance, over the rows of tile rows [row_tile0, row_tile1) (64
 // rows each); or with the row and column keys of the locally-dominant rounds.
-cudaError_t launch_greedy_pass1(const Workspace& w, cudaStream_t s);
-cudaError_t launch_greedy_pass1_bounds(const Workspace& w, int32_t row_tile0, int32_t row_tile1, cudaStream_t s);
+// a_src (where given, not null): the caller's rows of n int32, from which the
+// pass fills the pitched copy w.a.
+cudaError_t launch_greedy_pass1(const Workspace& w, const int32_t* a_src, cudaStream_t s);
+cudaError_t launch_greedy_pass1_bounds(const Workspace& w, int32_t row_tile0, int32_t row_tile1, const int32_t* a_src,
+                                       cudaStream_t s);
 cudaError_t launch_greedy_pass1_rounds(const Workspace& w, cudaStream_t s);
 cudaError_t launch_greedy_round(const Workspace& w, cudaStream_t s);
 // The greedy start by deferred acceptance (pass 1 with bounds must have run,
-// g_col zero); then the assignment is read off the jobs' holders.  Returns an
+// g_col zero); then the start (sigma, tau, D, f) is read off the jobs' holders.
+// Returns an
 // error (nothing launched) when the launch is refused or DGS_GREEDY_ROUNDS=1;
 // the caller then runs the rounds' pass 1 and the locally-dominant rounds
 // (launch_greedy_round).
 cudaError_t launch_greedy_da(const Workspace& w, cudaStream_t s);
-cudaError_t launch_range_check(const Workspace& w, cudaStream_t s);
+// The range check alone (a_src as for pass 1).
+cudaError_t launch_range_check(const Workspace& w, const int32_t* a_src, cudaStream_t s);
 cudaError_t launch_start_from_tau(const Workspace& w, const int32_t* user_tau, int32_t mode, uint8_t* seen,
                                   cudaStream_t s);
 cudaError_t launch_full_evaluation(const Workspace& w, int32_t conditional, cudaStream_t s);

@@ -114,7 +114,7 @@ extern "C" DGS_API dgs_status dgs_evaluate_static(const int32_t* benefit, int32_
     }
     static_state_kernel<<<1, 1, 0, s>>>(w.st);
     e = cudaGetLastError();
-    if (e == cudaSuccess) e = launch_range_check(w, s);
+    if (e == cudaSuccess) e = launch_range_check(w, nullptr, s);
     if (e == cudaSuccess) e = launch_start_from_tau(w, sigma_in, DGS_INIT_USER, seen, s);
     if (e == cudaSuccess) e = launch_full_evaluation(w, 0, s);
     if (e == cudaSuccess) e = launch_keys_to_slots(w, agent_gain, agent_job, job_gain, job_agent, s);

@@ -1311,6 +1311,7 @@ __global__ void __launch_bounds__(512) row_owner_evaluation_kernel(Workspace w, 
     if (st->status != kRunning) return;
     if (conditional && !(st->need_update && use_full_update(st->rescan_count, w.n, st->update_policy))) return;
     if (conditional && blockIdx.x == 0 && threadIdx.x == 0) st->full_evals += 1;
+    if (!conditional && blockIdx.x == 0 && threadIdx.x == 0 && st->sweeps == 0) st->f_initial = st->f;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ unsigned long long red_a[16], red_j[16];
     __shared__ __align__(8) uint64_t bar[2];
@@ -1366,7 +1367,9 @@ __global__ void __launch_bounds__(512) row_owner_evaluation_kernel(Workspace w, 
 __device__ __forceinline__ void start_from_tau_body(const Workspace& w, const int32_t* user_tau, int32_t mode,
                                                     uint8_t* seen, int32_t bid, int32_t nblk) {
     DeviceState* st = w.st;
-    if (st->status != kRunning) return;
+    // (uniform for the CTA: another CTA may report a bad start meanwhile)
+    if (__syncthreads_or(st->status != kRunning)) return;
+    long long f = 0;
     for (int32_t i = bid * blockDim.x + threadIdx.x; i < w.n; i += nblk * blockDim.x) {
         int32_t j;
         if (mode == 2) j = i;                 // identity
@@ -1381,8 +1384,9 @@ __device__ __forceinline__ void start_from_tau_body(const Workspace& w, const in
         w.sigma[j] = i;
         const int32_t d = w.a[(size_t)i * w.lda + j];
         w.diag[j] = d;
-        atomicAdd(reinterpret_cast<unsigned long long*>(&st->f), (unsigned long long)(long long)d);
+        f += d;
     }
+    add_objective(st, f);
 }
 
 __global__ void start_from_tau_kernel(Workspace w, const int32_t* user_tau, int32_t mode, uint8_t* seen) {

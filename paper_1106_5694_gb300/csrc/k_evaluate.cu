@@ -631,6 +631,8 @@ __global__ void __launch_bounds__(Geo<kRows>::kThreads, 1) full_evaluation_kerne
     const int64_t total = eval_tiles(w.n);
     const Schedule sc{strip, (int32_t)blockIdx.x, (int32_t)gridDim.x, (int32_t)(total * blockIdx.x / gridDim.x),
                       (int32_t)(total * (blockIdx.x + 1) / gridDim.x)};
+    // the first evaluation follows the start
+    if (!conditional && blockIdx.x == 0 && threadIdx.x == 0 && w.st->sweeps == 0) w.st->f_initial = w.st->f;
     full_evaluation_body<kRows, kTma>(w, conditional, sc, &tm);
 }
 

@@ -34,9 +34,9 @@ __device__ __forceinline__ void put_bound(const Workspace& w, int32_t i, int32_t
     else atomicMax(b, top);
 }
 
-// a_src (batched instances only): the caller's matrix with row pitch n when w.a
-// is the workspace's pitched copy still to be filled; this pass reads a_src
-// and writes the copy as it goes.  Null: w.a is read.
+// a_src: the caller's matrix with row pitch n when w.a is the workspace's
+// pitched copy still to be filled; this pass reads a_src and writes the copy as
+// it goes.  Null: w.a is read.
 template <int kMode>
 __device__ __forceinline__ void greedy_pass1_body(const Workspace& w, int32_t tiles_x, int32_t tiles_total,
                                                   int32_t bid, int32_t nblk, const int32_t* a_src = nullptr) {
@@ -172,8 +172,8 @@ __device__ __forceinline__ void greedy_pass1_body(const Workspace& w, int32_t ti
 // tiles tile0 .. tiles_total - 1 (row-major: a band of whole tile rows)
 template <int kMode>
 __global__ void __launch_bounds__(256) greedy_pass1_kernel(Workspace w, int32_t tiles_x, int32_t tiles_total,
-                                                           int32_t tile0) {
-    greedy_pass1_body<kMode>(w, tiles_x, tiles_total, tile0 + blockIdx.x, gridDim.x);
+                                                           int32_t tile0, const int32_t* a_src) {
+    greedy_pass1_body<kMode>(w, tiles_x, tiles_total, tile0 + blockIdx.x, gridDim.x, a_src);
 }
 
 // Match every mutually-best (agent, job) pair.
@@ -630,47 +630,86 @@ __global__ void greedy_loop_cond_kernel(Workspace w, unsigned long long cond) {
     cudaGraphSetConditional(cond, (st->status == kRunning && st->greedy_remaining > 0) ? 1u : 0u);
 }
 
-// The assignment from the jobs' holders.
-__global__ void greedy_da_finish_kernel(Workspace w) {
+// The start from the jobs' holders: both maps, D (the holder's key has the
+// benefit) and f.
+__global__ void __launch_bounds__(256) greedy_da_start_kernel(Workspace w) {
     DeviceState* st = w.st;
     if (st->status != kRunning) return;
     if (blockIdx.x == 0 && threadIdx.x == 0) st->greedy_remaining = 0;
+    long long f = 0;
     for (int32_t j = blockIdx.x * blockDim.x + threadIdx.x; j < w.n; j += gridDim.x * blockDim.x) {
-        const int32_t i = key_index(w.g_col[j]);
+        const unsigned long long key = w.g_col[j];
+        const int32_t i = key_index(key);
         if (i < 0 || i >= w.n) {
             st->error = kErrInternal;
             st->status = kError;
             continue;
         }
+        const int32_t d = (int32_t)(key >> 32) - kBenefitLimit;
         w.sigma[j] = i;
         w.tau[i] = j;
+        w.diag[j] = d;
+        f += d;
+    }
+    add_objective(st, f);
+}
+
+// |a| < 2^29 check alone (for entry points that do not run pass 1).  The pitched
+// rows are read as one array (padding columns are 0, which changes nothing),
+// four 16-byte loads in flight per thread: HBM-bound (n = 10000, 400 MB: 115
+// us with one load in flight and a column test per element, now 62).
+__device__ __forceinline__ void report_range(const Workspace& w, int32_t lo, int32_t hi) {
+    // the largest |x| of lo <= x <= hi, without the overflow of -INT32_MIN
+    int32_t amax = max(hi, lo == INT32_MIN ? INT32_MAX : -lo);
+    amax = (int32_t)__reduce_max_sync(0xffffffffu, (uint32_t)max(amax, 0));
+    if ((threadIdx.x & 31) == 0 && amax) {
+        atomicMax(&w.st->max_abs, amax);
+        if (amax >= kBenefitLimit) {
+            atomicExch(&w.st->error, kErrRange);
+            atomicExch(&w.st->status, kError);
+        }
     }
 }
 
-// |a| < 2^29 check alone (for entry points that do not run pass 1).
-__global__ void range_check_kernel(Workspace w) {
-    bool bad = false;
-    int32_t amax = 0;
-    const size_t total4 = (size_t)w.n * (size_t)(w.lda / 4);
-    const int32_t row4 = w.lda / 4;
-    for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < total4; q += (size_t)gridDim.x * blockDim.x) {
-        const int32_t c = (int32_t)(q % row4) * 4;
-        const int4 v = reinterpret_cast<const int4*>(w.a)[q];
-        const int32_t vals[4] = {v.x, v.y, v.z, v.w};
+__global__ void __launch_bounds__(256) range_check_kernel(Workspace w) {
+    const int4* a = reinterpret_cast<const int4*>(w.a);
+    const size_t total = (size_t)w.n * (size_t)(w.lda / 4), stride = (size_t)gridDim.x * blockDim.x;
+    int32_t lo = 0, hi = 0;
+    constexpr int kAhead = 4;
+    for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < total; q += kAhead * stride) {
+        int4 v[kAhead];
 #pragma unroll
-        for (int e = 0; e < 4; ++e)
-            if (c + e < w.n) {
-                bad |= (vals[e] >= kBenefitLimit) || (vals[e] <= -kBenefitLimit);
-                amax = max(amax, vals[e] == INT32_MIN ? INT32_MAX : abs(vals[e]));
+        for (int k = 0; k < kAhead; ++k) v[k] = q + k * stride < total ? a[q + k * stride] : make_int4(0, 0, 0, 0);
+#pragma unroll
+        for (int k = 0; k < kAhead; ++k) {
+            lo = min(lo, min(min(v[k].x, v[k].y), min(v[k].z, v[k].w)));
+            hi = max(hi, max(max(v[k].x, v[k].y), max(v[k].z, v[k].w)));
+        }
+    }
+    report_range(w, lo, hi);
+}
+
+// The same, filling the pitched copy w.a from the caller's rows of n int32.
+__global__ void __launch_bounds__(256) repitch_check_kernel(Workspace w, const int32_t* a_src) {
+    const int lane = threadIdx.x & 31;
+    int32_t lo = 0, hi = 0;
+    for (int32_t i = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5); i < w.n; i += gridDim.x * (blockDim.x / 32)) {
+        const int32_t* src = a_src + (size_t)i * w.n;
+        int32_t* dst = const_cast<int32_t*>(w.a) + (size_t)i * w.lda;
+        constexpr int kAhead = 8;
+        for (int32_t j = lane; j < w.lda; j += 32 * kAhead) {
+            int32_t x[kAhead];
+#pragma unroll
+            for (int k = 0; k < kAhead; ++k) x[k] = j + 32 * k < w.n ? src[j + 32 * k] : 0;
+#pragma unroll
+            for (int k = 0; k < kAhead; ++k) {
+                if (j + 32 * k < w.lda) dst[j + 32 * k] = x[k];
+                lo = min(lo, x[k]);
+                hi = max(hi, x[k]);
             }
+        }
     }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) amax = max(amax, __shfl_xor_sync(0xffffffffu, amax, off));
-    if ((threadIdx.x & 31) == 0 && amax) atomicMax(&w.st->max_abs, amax);
-    if (bad) {
-        atomicExch(&w.st->error, kErrRange);
-        atomicExch(&w.st->status, kError);
-    }
+    report_range(w, lo, hi);
 }
 
 __global__ void __launch_bounds__(256) greedy_pass1_batched_kernel(BatchQueues q) {
@@ -761,34 +800,36 @@ __global__ void greedy_da_finish_batched_kernel(BatchTable t) {
 
 }  // namespace
 
-cudaError_t launch_range_check(const Workspace& w, cudaStream_t s) {
-    range_check_kernel<<<dgs::device_sms() * 4, 256, 0, s>>>(w);
+cudaError_t launch_range_check(const Workspace& w, const int32_t* a_src, cudaStream_t s) {
+    if (a_src != nullptr) repitch_check_kernel<<<dgs::device_sms() * 8, 256, 0, s>>>(w, a_src);
+    else range_check_kernel<<<dgs::device_sms() * 8, 256, 0, s>>>(w);
     return cudaGetLastError();
 }
 
 // Pass 1 over the rows of tile rows [row_tile0, row_tile1) (64 rows each):
 // the bands of a matrix that arrives in pieces can be processed as they land.
 cudaError_t launch_greedy_pass1_rows(const Workspace& w, int32_t mode, int32_t row_tile0, int32_t row_tile1,
-                                     cudaStream_t s) {
+                                     const int32_t* a_src, cudaStream_t s) {
     const int32_t tx = (w.n + kT - 1) / kT;
     const int32_t t0 = row_tile0 * tx, t1 = (row_tile1 < tx ? row_tile1 : tx) * tx;
     const int32_t count = t1 - t0;
     if (count <= 0) return cudaSuccess;
     const int32_t grid = count < dgs::device_sms() * 8 ? count : dgs::device_sms() * 8;
-    if (mode == kPass1Bounds) greedy_pass1_kernel<kPass1Bounds><<<grid, 256, 0, s>>>(w, tx, t1, t0);
-    else if (mode == kPass1Rounds) greedy_pass1_kernel<kPass1Rounds><<<grid, 256, 0, s>>>(w, tx, t1, t0);
-    else greedy_pass1_kernel<kPass1Plain><<<grid, 256, 0, s>>>(w, tx, t1, t0);
+    if (mode == kPass1Bounds) greedy_pass1_kernel<kPass1Bounds><<<grid, 256, 0, s>>>(w, tx, t1, t0, a_src);
+    else if (mode == kPass1Rounds) greedy_pass1_kernel<kPass1Rounds><<<grid, 256, 0, s>>>(w, tx, t1, t0, a_src);
+    else greedy_pass1_kernel<kPass1Plain><<<grid, 256, 0, s>>>(w, tx, t1, t0, a_src);
     return cudaGetLastError();
 }
 
-cudaError_t launch_greedy_pass1_bounds(const Workspace& w, int32_t row_tile0, int32_t row_tile1, cudaStream_t s) {
-    return launch_greedy_pass1_rows(w, kPass1Bounds, row_tile0, row_tile1, s);
+cudaError_t launch_greedy_pass1_bounds(const Workspace& w, int32_t row_tile0, int32_t row_tile1, const int32_t* a_src,
+                                       cudaStream_t s) {
+    return launch_greedy_pass1_rows(w, kPass1Bounds, row_tile0, row_tile1, a_src, s);
 }
 cudaError_t launch_greedy_pass1_rounds(const Workspace& w, cudaStream_t s) {
-    return launch_greedy_pass1_rows(w, kPass1Rounds, 0, (w.n + kT - 1) / kT, s);
+    return launch_greedy_pass1_rows(w, kPass1Rounds, 0, (w.n + kT - 1) / kT, nullptr, s);
 }
-cudaError_t launch_greedy_pass1(const Workspace& w, cudaStream_t s) {
-    return launch_greedy_pass1_rows(w, kPass1Plain, 0, (w.n + kT - 1) / kT, s);
+cudaError_t launch_greedy_pass1(const Workspace& w, const int32_t* a_src, cudaStream_t s) {
+    return launch_greedy_pass1_rows(w, kPass1Plain, 0, (w.n + kT - 1) / kT, a_src, s);
 }
 
 cudaError_t launch_greedy_loop_cond(const Workspace& w, unsigned long long handle, cudaStream_t s) {
@@ -854,7 +895,7 @@ cudaError_t launch_greedy_da(const Workspace& w, cudaStream_t s) {
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const int32_t nb = (w.n + 255) / 256;
-    greedy_da_finish_kernel<<<nb < dgs::device_sms() * 4 ? nb : dgs::device_sms() * 4, 256, 0, s>>>(w);
+    greedy_da_start_kernel<<<nb < dgs::device_sms() * 4 ? nb : dgs::device_sms() * 4, 256, 0, s>>>(w);
     return cudaGetLastError();
 }
 
