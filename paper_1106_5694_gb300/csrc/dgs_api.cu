@@ -628,7 +628,8 @@ struct HostBands {
 };
 
 // *started: the start (sigma, D, f) is there too; else only tau and sigma are.
-dgs_status run_greedy(Solve& S, EventPair* timer, bool* started, const HostBands* bands = nullptr) {
+dgs_status run_greedy(Solve& S, EventPair* timer, bool* started, int32_t real_n, int32_t real_m,
+                      const HostBands* bands = nullptr) {
     *started = true;
     if (bands == nullptr) {
         DGS_CUDA(launch_greedy_pass1_bounds(S.w, 0, (S.w.n + 63) / 64, S.a_src, S.s), "greedy pass 1");
@@ -642,9 +643,9 @@ dgs_status run_greedy(Solve& S, EventPair* timer, bool* started, const HostBands
         }
     }
     if (timer) DGS_TRY(timer->begin(S.s));
-    const cudaError_t pe = launch_greedy_da(S.w, S.s);
+    const cudaError_t pe = launch_greedy_da(S.w, real_n, real_m, S.s);
     if (pe == cudaSuccess) {
-        S.launches += 2;
+        S.launches += real_n == S.w.n && real_m == S.w.n ? 2 : 4;
         if (timer) DGS_TRY(timer->end(S.s));
         return DGS_OK;
     }
@@ -744,11 +745,12 @@ struct PinnedStart {
 
 // One solve, enqueued on `stream`.  final_status (host, may be null): set to
 // the solve's status when the stream reaches its end.  extra_launches: kernels
-// the caller launches around the solve (counted in the stats).
+// the caller launches around the solve (counted in the stats).  real_n, real_m
+// (0: n): the real agents and jobs of an instance padded with zeros.
 dgs_status solve_impl(const int32_t* benefit, int32_t n, int32_t* sigma_out, int64_t* objective_out,
                       const dgs_options* opt, dgs_stats* stats, cudaStream_t stream,
                       dgs_status* final_status = nullptr, int64_t extra_launches = 0,
-                      const HostBands* bands = nullptr) {
+                      const HostBands* bands = nullptr, int32_t real_n = 0, int32_t real_m = 0) {
     DGS_TRY(check_common(benefit, n));
     if (sigma_out == nullptr || objective_out == nullptr) return DGS_ERR_INVALID;
     dgs_options o;
@@ -807,7 +809,8 @@ dgs_status solve_impl(const int32_t* benefit, int32_t n, int32_t* sigma_out, int
     EventPair gev;
     bool started = false;
     if (o.init == DGS_INIT_GREEDY) {
-        DGS_TRY(run_greedy(S, o.profile ? &gev : nullptr, &started, bands));
+        DGS_TRY(run_greedy(S, o.profile ? &gev : nullptr, &started, real_n > 0 ? real_n : n, real_m > 0 ? real_m : n,
+                           bands));
     } else {
         DGS_CUDA(launch_greedy_pass1(S.w, S.a_src, stream), "pass 1");  // transpose + range check
         S.launches += 1;
@@ -1005,7 +1008,7 @@ dgs_status dgs_solve_rect(const int32_t* benefit, int32_t n_agents, int32_t m_jo
     int32_t* tau = reinterpret_cast<int32_t*>(static_cast<char*>(buf.p) + sq_bytes);
     pad_square_kernel<<<dgs::device_sms() * 8, 256, 0, s>>>(benefit, n_agents, m_jobs, sz, sq);
     DGS_CUDA(cudaGetLastError(), "pad");
-    DGS_TRY(solve_impl(sq, sz, tau, objective_out, &o, stats, s, nullptr, 2));
+    DGS_TRY(solve_impl(sq, sz, tau, objective_out, &o, stats, s, nullptr, 2, nullptr, n_agents, m_jobs));
     trim_assignment_kernel<<<(n_agents + 255) / 256, 256, 0, s>>>(tau, n_agents, m_jobs, assign_out);
     DGS_CUDA(cudaGetLastError(), "trim");
     return DGS_OK;
@@ -1036,7 +1039,7 @@ dgs_status dgs_greedy_init(const int32_t* benefit, int32_t n, int32_t* sigma_out
     DGS_TRY(S.setup(benefit, n, true));
     DGS_TRY(S.init_state(0, nullptr));
     bool started;
-    DGS_TRY(run_greedy(S, nullptr, &started));
+    DGS_TRY(run_greedy(S, nullptr, &started, n, n));
     DGS_CUDA(launch_finish(S.w, sigma_out, s), "finish");
     DeviceState h;
     DGS_TRY(S.read_state(&h));

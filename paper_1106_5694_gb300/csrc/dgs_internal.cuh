@@ -74,7 +74,7 @@ struct DeviceState {
     int32_t seq_passes;      // Algorithm 1: passes so far
     int64_t f_pass;          // Algorithm 1: objective at the start of the current pass
     int32_t da_next;         // greedy start (deferred acceptance): next agent to take
-    int32_t pad_state2;
+    int32_t da_wait;         // padded instances: agents that wait for the second phase of proposals
 };
 
 // Pointers to every array of one solve (passed by value to kernels).
@@ -411,7 +411,10 @@ cudaError_t launch_greedy_round(const Workspace& w, cudaStream_t s);
 // error (nothing launched) when the launch is refused or DGS_GREEDY_ROUNDS=1;
 // the caller then runs the rounds' pass 1 and the locally-dominant rounds
 // (launch_greedy_round).
-cudaError_t launch_greedy_da(const Workspace& w, cudaStream_t s);
+// real_n / real_m: the agents and jobs that are real (below n: the others are
+// the zero rows or columns of a padded instance; at most one of the two).
+// (free_a has to be zero, rescan_list is written.)
+cudaError_t launch_greedy_da(const Workspace& w, int32_t real_n, int32_t real_m, cudaStream_t s);
 // The range check alone (a_src as for pass 1).
 cudaError_t launch_range_check(const Workspace& w, const int32_t* a_src, cudaStream_t s);
 cudaError_t launch_start_from_tau(const Workspace& w, const int32_t* user_tau, int32_t mode, uint8_t* seen,

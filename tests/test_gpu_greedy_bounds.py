@@ -56,3 +56,24 @@ def test_batched_greedy_start_equals_oracle(kind):
         ref_st, ref_sig, ref_obj, _ = B.dgs_solve_ex(torch.from_numpy(a).cuda())
         assert ref_st == B.DGS_OK and obj == ref_obj
         np.testing.assert_array_equal(out.cpu().numpy(), ref_sig.cpu().numpy())
+
+
+@pytest.mark.parametrize("kind", ["negative", "zeros", "ties", "mixed"])
+@pytest.mark.parametrize("n,m", [(1, 2), (2, 1), (5, 70), (70, 5), (64, 65), (200, 130), (130, 300), (700, 40)])
+def test_padded_start_equals_oracle(kind, n, m):
+    """Rectangular instances: benefits below, at and above the dummies' zero,
+    with ties between real and dummy pairs."""
+    rng = np.random.default_rng(n * 1000 + m)
+    lo, hi = {"negative": (-50, 0), "zeros": (0, 1), "ties": (-1, 2), "mixed": (-500, 500)}[kind]
+    a = rng.integers(lo, hi, size=(n, m), dtype=np.int32)
+    st_o, assign_o, f_o, sweeps_o = oracle.dgs_rect(a)
+    assert st_o == oracle.OK
+    st, assign, f, stats = B.dgs_solve_rect(torch.from_numpy(a).cuda())
+    assert st == B.DGS_OK, B.dgs_last_cuda_error()
+    np.testing.assert_array_equal(assign.cpu().numpy(), assign_o)
+    assert f == f_o and stats["sweeps"] == sweeps_o
+    s = max(n, m)
+    square = np.zeros((s, s), np.int32)
+    square[:n, :m] = a
+    tau = oracle.greedy_init(square)
+    assert stats["initial_objective"] == int(square[np.arange(s), tau].astype(np.int64).sum())
