@@ -617,7 +617,7 @@ dgs_status sequential_pass_body(void* p, cudaStream_t cs, unsigned long long h) 
 }
 
 // The greedy start: pass 1, then deferred acceptance in one launch; where
-// that launch is refused, pass 1 again with the row and column keys and
+// that launch is refused, the best pairs and
 // the locally-dominant rounds as a device-side loop (the same assignment).
 // A matrix that arrives in row bands (dgs_solve_host): event k is recorded
 // once rows [64 k tile_rows, 64 (k + 1) tile_rows) are on the device.
@@ -654,8 +654,8 @@ dgs_status run_greedy(Solve& S, EventPair* timer, bool* started, int32_t real_n,
     const size_t nb = align_up((size_t)S.w.n, 128);
     DGS_CUDA(cudaMemsetAsync(S.w.free_a, 1, nb, S.s), "free agents");
     DGS_CUDA(cudaMemsetAsync(S.w.free_j, 1, nb, S.s), "free jobs");
-    DGS_CUDA(launch_greedy_pass1_rounds(S.w, S.s), "greedy pass 1");
-    S.launches += 1;
+    DGS_CUDA(launch_greedy_best(S.w, S.s), "best pairs");
+    S.launches += 2;
     LoopCtx c{S.w, S.ctl};
     DGS_TRY(enqueue_loop(S.s, greedy_round_body, &c));
     if (timer) DGS_TRY(timer->end(S.s));

@@ -395,22 +395,23 @@ __device__ __forceinline__ bool grid_barrier(DeviceState* st) {
 
 // ------------------------------------------------------ host-side launchers
 // Each returns the launch error (cudaSuccess on success).
-// Pass 1: the transposed copy and the range check alone; with the bounds of
+// Pass 1: the transposed copy and the range check alone, or with the bounds of
 // deferred acceptance, over the rows of tile rows [row_tile0, row_tile1) (64
-// rows each); or with the row and column keys of the locally-dominant rounds.
+// rows each).
 // a_src (where given, not null): the caller's rows of n int32, from which the
 // pass fills the pitched copy w.a.
 cudaError_t launch_greedy_pass1(const Workspace& w, const int32_t* a_src, cudaStream_t s);
 cudaError_t launch_greedy_pass1_bounds(const Workspace& w, int32_t row_tile0, int32_t row_tile1, const int32_t* a_src,
                                        cudaStream_t s);
-cudaError_t launch_greedy_pass1_rounds(const Workspace& w, cudaStream_t s);
+// Locally-dominant rounds: the best pair of every agent and job (after pass 1),
+// and one round.
+cudaError_t launch_greedy_best(const Workspace& w, cudaStream_t s);
 cudaError_t launch_greedy_round(const Workspace& w, cudaStream_t s);
 // The greedy start by deferred acceptance (pass 1 with bounds must have run,
 // g_col zero); then the start (sigma, tau, D, f) is read off the jobs' holders.
 // Returns an
 // error (nothing launched) when the launch is refused or DGS_GREEDY_ROUNDS=1;
-// the caller then runs the rounds' pass 1 and the locally-dominant rounds
-// (launch_greedy_round).
+// the caller then runs the locally-dominant rounds.
 // real_n / real_m: the agents and jobs that are real (below n: the others are
 // the zero rows or columns of a padded instance; at most one of the two).
 // (free_a has to be zero, rescan_list is written.)

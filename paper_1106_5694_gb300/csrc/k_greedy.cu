@@ -13,8 +13,7 @@
 //
 // Pass 1 reads a once in 64x64 tiles and, in the same pass, writes the
 // transposed copy at, checks |a| < 2^29 and computes what the greedy start
-// that follows needs: each agent's best benefit in every tile of jobs, or
-// (rounds) every agent's and job's best pair.
+// that follows needs: each agent's best benefit in every tile of jobs.
 #include <cstdlib>
 
 #include "dgs_internal.cuh"
@@ -24,36 +23,61 @@ namespace {
 
 constexpr int kT = 64;  // tile edge
 
-// What pass 1 computes beside the transposed copy and the range check.
-enum : int { kPass1Plain = 0, kPass1Bounds = 1, kPass1Rounds = 2 };
-
-// The maximum `top` of agent i's biased benefits in the 64 columns from J0 on.
-__device__ __forceinline__ void put_bound(const Workspace& w, int32_t i, int32_t J0, uint32_t top) {
-    uint32_t* b = w.g_bound + (size_t)i * w.bound_tiles + (J0 >> w.bound_shift);
-    if (w.bound_shift == kBoundShift) *b = top;
-    else atomicMax(b, top);
+// |x| of lo <= x <= hi: raises the largest one seen and reports values out of
+// range (whole warps call it).
+__device__ __forceinline__ void report_range(const Workspace& w, int32_t lo, int32_t hi) {
+    // without the overflow of -INT32_MIN
+    int32_t amax = max(hi, lo == INT32_MIN ? INT32_MAX : -lo);
+    amax = (int32_t)__reduce_max_sync(0xffffffffu, (uint32_t)max(amax, 0));
+    if ((threadIdx.x & 31) == 0 && amax) {
+        atomicMax(&w.st->max_abs, amax);
+        if (amax >= kBenefitLimit) {
+            atomicExch(&w.st->error, kErrRange);
+            atomicExch(&w.st->status, kError);
+        }
+    }
 }
 
+// Pass 1 over 64 x 64 tiles, 256 threads.  A tile's rows go to shared memory in
+// 16-byte chunks, chunk c of row r at place c ^ (r / 4 mod 16): a row's chunks
+// fill all banks, and so do the chunks c of eight rows 4l that the transposing
+// read takes together.  Each thread then reads the 4 x 4 block of rows 4l ..
+// and columns 4c .., writes its columns as 16 bytes of four rows of at, and
+// (kBounds) raises the tile's maxima of its rows.  Rows and columns past n read
+// as 0, which changes no range and leaves bounds valid.  What bounds it: HBM
+// (read a, write at); with one element per shared-memory instruction and the
+// row maxima by shuffles it was 465 instructions a warp and tile, 55% of the
+// issue slots (n = 10000, under ncu: 147 us, now 128, 92% of the measured
+// copy rate).
+//
 // a_src: the caller's matrix with row pitch n when w.a is the workspace's
-// pitched copy still to be filled; this pass reads a_src and writes the copy as
-// it goes.  Null: w.a is read.
-template <int kMode>
+// pitched copy still to be filled; this pass reads a_src (a warp per row, 32
+// consecutive columns per load, from any 4-byte boundary) and writes the copy
+// as it goes.  Null: w.a is read.
+template <bool kBounds>
 __device__ __forceinline__ void greedy_pass1_body(const Workspace& w, int32_t tiles_x, int32_t tiles_total,
                                                   int32_t bid, int32_t nblk, const int32_t* a_src = nullptr) {
-    __shared__ int32_t s[kT][kT + 1];
-    __shared__ unsigned long long colpart[kMode == kPass1Rounds ? 4 : 1][kT];
+    __shared__ __align__(16) int32_t s[kT * kT];
+    __shared__ uint32_t s_top[kT];
     const int32_t n = w.n;
-    const int t = threadIdx.x;
-    const int lane16 = t & 15;
-    bool bad = false;
-    int32_t amax = 0;
+    const int t = threadIdx.x, lane16 = t & 15, row0 = t >> 4;
+    auto chunk = [&](int r, int c) -> int4* { return reinterpret_cast<int4*>(s) + r * 16 + (c ^ ((r >> 2) & 15)); };
+    if (kBounds && t < kT) s_top[t] = 0u;
+    int32_t lo = 0, hi = 0;
     for (int32_t tile = bid; tile < tiles_total; tile += nblk) {
         const int32_t I0 = (tile / tiles_x) * kT;
         const int32_t J0 = (tile % tiles_x) * kT;
-        if (a_src != nullptr) {
-            // rows of n int32 from any 4-byte boundary: a warp per row, two
-            // loads of 32 consecutive columns; the pitched copy (padding
-            // columns 0) is written from shared memory below
+        if (a_src == nullptr) {
+            int4 x[4];
+#pragma unroll
+            for (int p = 0; p < 4; ++p) {
+                const int32_t i = I0 + row0 + 16 * p, j = J0 + lane16 * 4;
+                x[p] = i < n && j < w.lda ? *reinterpret_cast<const int4*>(w.a + (size_t)i * w.lda + j)
+                                          : make_int4(0, 0, 0, 0);
+            }
+#pragma unroll
+            for (int p = 0; p < 4; ++p) *chunk(row0 + 16 * p, lane16) = x[p];
+        } else {
             const int lane = t & 31;
             int32_t x[8][2];
 #pragma unroll
@@ -66,114 +90,71 @@ __device__ __forceinline__ void greedy_pass1_body(const Workspace& w, int32_t ti
                 }
             }
 #pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                const int r = (t >> 5) + 8 * q;
-                uint32_t top = 0;
+            for (int q = 0; q < 8; ++q)
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
-                    s[r][lane + 32 * h] = x[q][h];
-                    if (J0 + lane + 32 * h < n) {
-                        bad |= (x[q][h] >= kBenefitLimit) || (x[q][h] <= -kBenefitLimit);
-                        amax = max(amax, x[q][h] == INT32_MIN ? INT32_MAX : abs(x[q][h]));
-                        top = max(top, (uint32_t)(x[q][h] + kBenefitLimit));
-                    }
+                    const int r = (t >> 5) + 8 * q, c = lane + 32 * h;
+                    reinterpret_cast<int32_t*>(chunk(r, c >> 2))[c & 3] = x[q][h];
                 }
-                top = __reduce_max_sync(0xffffffffu, top);
-                if (kMode == kPass1Bounds && lane == 0 && I0 + r < n) put_bound(w, I0 + r, J0, top);
-            }
-        }
-        // load 64 rows x 64 cols with int4, 16 threads per row, 4 passes
-#pragma unroll
-        for (int p = 0; p < 4 && a_src == nullptr; ++p) {
-            const int r = (t >> 4) + 16 * p;
-            const int c = lane16 * 4;
-            const int32_t i = I0 + r, j = J0 + c;
-            int4 v = make_int4(0, 0, 0, 0);
-            if (i < n && j < w.lda) v = *reinterpret_cast<const int4*>(w.a + (size_t)i * w.lda + j);
-            s[r][c + 0] = v.x; s[r][c + 1] = v.y; s[r][c + 2] = v.z; s[r][c + 3] = v.w;
-            // row best over this tile's 4 columns of this thread
-            unsigned long long best = 0;
-            uint32_t top = 0;
-            const int32_t vals[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                if (i < n && j + e < n) {
-                    const int32_t x = vals[e];
-                    bad |= (x >= kBenefitLimit) || (x <= -kBenefitLimit);
-                    amax = max(amax, x == INT32_MIN ? INT32_MAX : abs(x));
-                    if (kMode == kPass1Rounds) best = umax64(best, pack_benefit(x, (uint32_t)(j + e)));
-                    if (kMode == kPass1Bounds) top = max(top, (uint32_t)(x + kBenefitLimit));
-                }
-            }
-            if (kMode == kPass1Rounds) {
-#pragma unroll
-                for (int off = 8; off > 0; off >>= 1) best = umax64(best, __shfl_xor_sync(0xffffffffu, best, off));
-                if (lane16 == 0 && i < n && best != 0) atomicMax(&w.g_row[i], best);
-            } else if (kMode == kPass1Bounds) {
-#pragma unroll
-                for (int off = 8; off > 0; off >>= 1) top = max(top, __shfl_xor_sync(0xffffffffu, top, off));
-                if (lane16 == 0 && i < n) put_bound(w, i, J0, top);
-            }
         }
         __syncthreads();
-        // column best: thread (group g = t/64, column c = t%64) scans 16 rows
-        if (kMode == kPass1Rounds) {
-            const int c = t & 63, g = t >> 6;
-            const int32_t j = J0 + c;
-            unsigned long long best = 0;
-            if (j < n) {
-#pragma unroll
-                for (int r = 0; r < 16; ++r) {
-                    const int32_t i = I0 + g * 16 + r;
-                    if (i < n) best = umax64(best, pack_benefit(s[g * 16 + r][c], (uint32_t)i));
-                }
-            }
-            colpart[g][c] = best;
-        }
         if (a_src != nullptr) {
 #pragma unroll
             for (int p = 0; p < 4; ++p) {
-                const int r = (t >> 4) + 16 * p, c = lane16 * 4;
-                if (I0 + r < n && J0 + c < w.lda)
-                    *reinterpret_cast<int4*>(const_cast<int32_t*>(w.a) + (size_t)(I0 + r) * w.lda + J0 + c) =
-                        make_int4(s[r][c], s[r][c + 1], s[r][c + 2], s[r][c + 3]);
+                const int32_t r = row0 + 16 * p, i = I0 + r, j = J0 + lane16 * 4;
+                if (i < n && j < w.lda)
+                    *reinterpret_cast<int4*>(const_cast<int32_t*>(w.a) + (size_t)i * w.lda + j) = *chunk(r, lane16);
             }
         }
-        // transposed store: at row j = J0 + jr, 4 agents per thread
+        // rows 4 lane16 .., columns 4 row0 ..
+        int4 b[4];
 #pragma unroll
-        for (int p = 0; p < 4; ++p) {
-            const int jr = (t >> 4) + 16 * p;
-            const int i4 = lane16 * 4;
-            const int32_t j = J0 + jr;
-            if (j < n) {
-                int4 v;
-                v.x = s[i4 + 0][jr]; v.y = s[i4 + 1][jr]; v.z = s[i4 + 2][jr]; v.w = s[i4 + 3][jr];
-                *reinterpret_cast<int4*>(w.at + (size_t)j * w.ldt + I0 + i4) = v;
+        for (int e = 0; e < 4; ++e) b[e] = *chunk(lane16 * 4 + e, row0);
+        const int32_t j = J0 + row0 * 4;
+        int32_t* at = w.at + (size_t)j * w.ldt + I0 + lane16 * 4;
+        if (j < n) *reinterpret_cast<int4*>(at) = make_int4(b[0].x, b[1].x, b[2].x, b[3].x);
+        if (j + 1 < n) *reinterpret_cast<int4*>(at + w.ldt) = make_int4(b[0].y, b[1].y, b[2].y, b[3].y);
+        if (j + 2 < n) *reinterpret_cast<int4*>(at + 2 * (size_t)w.ldt) = make_int4(b[0].z, b[1].z, b[2].z, b[3].z);
+        if (j + 3 < n) *reinterpret_cast<int4*>(at + 3 * (size_t)w.ldt) = make_int4(b[0].w, b[1].w, b[2].w, b[3].w);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const int32_t top = max(max(b[e].x, b[e].y), max(b[e].z, b[e].w));
+            lo = min(lo, min(min(b[e].x, b[e].y), min(b[e].z, b[e].w)));
+            hi = max(hi, top);
+            if (kBounds) atomicMax(&s_top[lane16 * 4 + e], (uint32_t)(top + kBenefitLimit));
+        }
+        __syncthreads();
+        if (kBounds && t < kT) {  // (the next tile's maxima come after its first barrier)
+            if (I0 + t < n) {
+                uint32_t* bound = w.g_bound + (size_t)(I0 + t) * w.bound_tiles + (J0 >> w.bound_shift);
+                if (w.bound_shift == kBoundShift) *bound = s_top[t];
+                else atomicMax(bound, s_top[t]);
             }
+            s_top[t] = 0u;
         }
-        __syncthreads();
-        if (kMode != kPass1Rounds) continue;
-        if (t < kT) {
-            const int32_t j = J0 + t;
-            unsigned long long best = umax64(umax64(colpart[0][t], colpart[1][t]), umax64(colpart[2][t], colpart[3][t]));
-            if (j < n && best != 0) atomicMax(&w.g_col[j], best);
-        }
-        __syncthreads();
     }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) amax = max(amax, __shfl_xor_sync(0xffffffffu, amax, off));
-    if ((t & 31) == 0 && amax) atomicMax(&w.st->max_abs, amax);
-    if (bad) {
-        atomicExch(&w.st->error, kErrRange);
-        atomicExch(&w.st->status, kError);
-    }
+    report_range(w, lo, hi);
 }
 
 // tiles tile0 .. tiles_total - 1 (row-major: a band of whole tile rows)
-template <int kMode>
+template <bool kBounds>
 __global__ void __launch_bounds__(256) greedy_pass1_kernel(Workspace w, int32_t tiles_x, int32_t tiles_total,
                                                            int32_t tile0, const int32_t* a_src) {
-    greedy_pass1_body<kMode>(w, tiles_x, tiles_total, tile0 + blockIdx.x, gridDim.x, a_src);
+    greedy_pass1_body<kBounds>(w, tiles_x, tiles_total, tile0 + blockIdx.x, gridDim.x, a_src);
+}
+
+// Rounds: every owner's best partner in its row of mat (a for agents, at for
+// jobs), a warp per row.
+__global__ void __launch_bounds__(256) greedy_best_kernel(Workspace w, const int32_t* mat, int32_t ld,
+                                                          unsigned long long* keys) {
+    const int lane = threadIdx.x & 31;
+    for (int32_t o = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5); o < w.n; o += gridDim.x * (blockDim.x / 32)) {
+        unsigned long long best = 0;
+        for (int32_t c = lane; c < w.n; c += 32) best = umax64(best, pack_benefit(mat[(size_t)o * ld + c], (uint32_t)c));
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) best = umax64(best, __shfl_xor_sync(0xffffffffu, best, off));
+        if (lane == 0) keys[o] = best;
+    }
 }
 
 // Match every mutually-best (agent, job) pair.
@@ -741,19 +722,6 @@ __global__ void __launch_bounds__(256) greedy_da_start_kernel(Workspace w) {
 // rows are read as one array (padding columns are 0, which changes nothing),
 // four 16-byte loads in flight per thread: HBM-bound (n = 10000, 400 MB: 115
 // us with one load in flight and a column test per element, now 62).
-__device__ __forceinline__ void report_range(const Workspace& w, int32_t lo, int32_t hi) {
-    // the largest |x| of lo <= x <= hi, without the overflow of -INT32_MIN
-    int32_t amax = max(hi, lo == INT32_MIN ? INT32_MAX : -lo);
-    amax = (int32_t)__reduce_max_sync(0xffffffffu, (uint32_t)max(amax, 0));
-    if ((threadIdx.x & 31) == 0 && amax) {
-        atomicMax(&w.st->max_abs, amax);
-        if (amax >= kBenefitLimit) {
-            atomicExch(&w.st->error, kErrRange);
-            atomicExch(&w.st->status, kError);
-        }
-    }
-}
-
 __global__ void __launch_bounds__(256) range_check_kernel(Workspace w) {
     const int4* a = reinterpret_cast<const int4*>(w.a);
     const size_t total = (size_t)w.n * (size_t)(w.lda / 4), stride = (size_t)gridDim.x * blockDim.x;
@@ -799,7 +767,7 @@ __global__ void __launch_bounds__(256) greedy_pass1_batched_kernel(BatchQueues q
     for_each_item(q.inst, q.q0, q.cap, [&](const Instance& in, int32_t bid, int32_t nblk) {
         const Workspace w = in.w;
         const int32_t tx = (w.n + kT - 1) / kT;
-        greedy_pass1_body<kPass1Bounds>(w, tx, tx * tx, bid, nblk, in.a_src);
+        greedy_pass1_body<true>(w, tx, tx * tx, bid, nblk, in.a_src);
     });
 }
 
@@ -891,32 +859,35 @@ cudaError_t launch_range_check(const Workspace& w, const int32_t* a_src, cudaStr
 
 // Pass 1 over the rows of tile rows [row_tile0, row_tile1) (64 rows each):
 // the bands of a matrix that arrives in pieces can be processed as they land.
-cudaError_t launch_greedy_pass1_rows(const Workspace& w, int32_t mode, int32_t row_tile0, int32_t row_tile1,
+cudaError_t launch_greedy_pass1_rows(const Workspace& w, bool bounds, int32_t row_tile0, int32_t row_tile1,
                                      const int32_t* a_src, cudaStream_t s) {
     const int32_t tx = (w.n + kT - 1) / kT;
     const int32_t t0 = row_tile0 * tx, t1 = (row_tile1 < tx ? row_tile1 : tx) * tx;
     const int32_t count = t1 - t0;
     if (count <= 0) return cudaSuccess;
     const int32_t grid = count < dgs::device_sms() * 8 ? count : dgs::device_sms() * 8;
-    if (mode == kPass1Bounds) greedy_pass1_kernel<kPass1Bounds><<<grid, 256, 0, s>>>(w, tx, t1, t0, a_src);
-    else if (mode == kPass1Rounds) greedy_pass1_kernel<kPass1Rounds><<<grid, 256, 0, s>>>(w, tx, t1, t0, a_src);
-    else greedy_pass1_kernel<kPass1Plain><<<grid, 256, 0, s>>>(w, tx, t1, t0, a_src);
+    if (bounds) greedy_pass1_kernel<true><<<grid, 256, 0, s>>>(w, tx, t1, t0, a_src);
+    else greedy_pass1_kernel<false><<<grid, 256, 0, s>>>(w, tx, t1, t0, a_src);
     return cudaGetLastError();
 }
 
 cudaError_t launch_greedy_pass1_bounds(const Workspace& w, int32_t row_tile0, int32_t row_tile1, const int32_t* a_src,
                                        cudaStream_t s) {
-    return launch_greedy_pass1_rows(w, kPass1Bounds, row_tile0, row_tile1, a_src, s);
-}
-cudaError_t launch_greedy_pass1_rounds(const Workspace& w, cudaStream_t s) {
-    return launch_greedy_pass1_rows(w, kPass1Rounds, 0, (w.n + kT - 1) / kT, nullptr, s);
+    return launch_greedy_pass1_rows(w, true, row_tile0, row_tile1, a_src, s);
 }
 cudaError_t launch_greedy_pass1(const Workspace& w, const int32_t* a_src, cudaStream_t s) {
-    return launch_greedy_pass1_rows(w, kPass1Plain, 0, (w.n + kT - 1) / kT, a_src, s);
+    return launch_greedy_pass1_rows(w, false, 0, (w.n + kT - 1) / kT, a_src, s);
 }
 
 cudaError_t launch_greedy_loop_cond(const Workspace& w, unsigned long long handle, cudaStream_t s) {
     greedy_loop_cond_kernel<<<1, 1, 0, s>>>(w, handle);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_greedy_best(const Workspace& w, cudaStream_t s) {
+    const int32_t grid = dgs::device_sms() * 8;
+    greedy_best_kernel<<<grid, 256, 0, s>>>(w, w.a, w.lda, w.g_row);
+    greedy_best_kernel<<<grid, 256, 0, s>>>(w, w.at, w.ldt, w.g_col);
     return cudaGetLastError();
 }
 
