@@ -591,44 +591,38 @@ __device__ __forceinline__ void controller_body(const Workspace& w, int32_t smem
         };
         for (int32_t cb = c_lo; cb < c_hi; cb += 32) {
             const int32_t mine = cb + lane < c_hi ? w.sl_chunk[cb + lane] : 0;
-            const int32_t most = (int32_t)__reduce_max_sync(0xffffffffu, (uint32_t)mine);
-            // a lane per chunk where one trip to memory takes them all (kAhead
-            // words in flight), else a lane per edge
-            constexpr int kAhead = 8;
-            if (most <= kAhead) {
-                int32_t incl = mine;
+            int32_t incl = mine;
 #pragma unroll
-                for (int off = 1; off < 32; off <<= 1) {
-                    const int32_t o = __shfl_up_sync(0xffffffffu, incl, off);
-                    if (lane >= off) incl += o;
+            for (int off = 1; off < 32; off <<= 1) {
+                const int32_t o = __shfl_up_sync(0xffffffffu, incl, off);
+                if (lane >= off) incl += o;
+            }
+            const int32_t excl = incl - mine, edges = __shfl_sync(0xffffffffu, incl, 31);
+            // the edges of these 32 chunks, one per lane and step wherever they
+            // are (a search in the prefix sums finds the chunk), kAhead steps'
+            // loads in flight
+            constexpr int kAhead = 4;
+            for (int32_t q0 = 0; q0 < edges; q0 += 32 * kAhead) {
+                int32_t c[kAhead];
+                unsigned long long e[kAhead];
+#pragma unroll
+                for (int k = 0; k < kAhead; ++k) {
+                    const int32_t q = q0 + 32 * k + lane;
+                    c[k] = 0;
+#pragma unroll
+                    for (int step = 16; step > 0; step >>= 1)
+                        if (__shfl_sync(0xffffffffu, excl, c[k] + step) <= q) c[k] += step;
+                    const int32_t at = q - __shfl_sync(0xffffffffu, excl, c[k]);
+                    c[k] += cb;
+                    e[k] = q < edges ? w.sl_edge[(size_t)c[k] * 32 + at] : 0ull;
                 }
-                const int32_t pos = pos0 + incl - mine;
-                const unsigned long long* src = w.sl_edge + (size_t)(cb + lane) * 32;
-                for (int32_t k0 = 0; k0 < most; k0 += kAhead) {
-                    unsigned long long e[kAhead];
 #pragma unroll
-                    for (int k = 0; k < kAhead; ++k) e[k] = k0 + k < mine ? src[k0 + k] : 0ull;
-#pragma unroll
-                    for (int k = 0; k < kAhead; ++k)
-                        if (k0 + k < mine) list_edge(pos + k0 + k, cb + lane, e[k]);
-                }
-                pos0 += __shfl_sync(0xffffffffu, incl, 31);
-            } else {
-                for (int32_t k0 = 0; k0 < min(32, c_hi - cb); k0 += 4) {
-                    int32_t m[4];
-                    unsigned long long e[4];
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        m[k] = __shfl_sync(0xffffffffu, mine, k0 + k);
-                        e[k] = lane < m[k] ? w.sl_edge[(size_t)(cb + k0 + k) * 32 + lane] : 0ull;
-                    }
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        if (lane < m[k]) list_edge(pos0 + lane, cb + k0 + k, e[k]);
-                        pos0 += m[k];
-                    }
+                for (int k = 0; k < kAhead; ++k) {
+                    const int32_t q = q0 + 32 * k + lane;
+                    if (q < edges) list_edge(pos0 + q, c[k], e[k]);
                 }
             }
+            pos0 += edges;
         }
         if (tid == 0) s_L = s_live = total;
         __syncthreads();
