@@ -28,9 +28,10 @@
  *     call waits for a sweep.  The outputs -- sigma_out, *objective_out,
  *     dgs_stats and dgs_options.status_out -- are valid once the stream has
  *     reached the end of the solve (for example after
- *     cudaStreamSynchronize); outputs in host memory are written then by a
- *     host callback on the stream, so host memory passed for them must stay
- *     valid until the stream has reached that point.  The return value reports only what is
+ *     cudaStreamSynchronize); outputs in pageable host memory are written
+ *     then by a host callback on the stream (which costs 70 to 90 us),
+ *     outputs in pinned host memory by the device; either must stay valid
+ *     until the stream has reached that point.  The return value reports only what is
  *     known when the work is enqueued (invalid arguments, allocation or
  *     launch failures); the outcome of the solve itself (DGS_OK,
  *     DGS_TIMEOUT, DGS_ERR_RANGE, DGS_ERR_INVALID for a USER start that is

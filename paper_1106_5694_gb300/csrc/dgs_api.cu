@@ -682,18 +682,13 @@ dgs_status status_of(const DeviceState& h) {
 // fills the caller's host-side outputs and returns the staging blocks.
 struct Completion {
     DeviceState* staged = nullptr;
-    void* release = nullptr;  // pinned block of the call (the random start), or null
-    size_t release_bytes = 0;
     dgs_stats* stats = nullptr;
     int64_t* objective = nullptr;  // host objective (a device one is written by the finish kernel)
     int32_t* status = nullptr;     // host options.status_out
     dgs_status* status_api = nullptr;
     int64_t launches = 0;          // kernels launched from the host
     int32_t sequential = 0;
-    ~Completion() {
-        pinned_put(staged, sizeof(DeviceState));
-        pinned_put(release, release_bytes);
-    }
+    ~Completion() { pinned_put(staged, sizeof(DeviceState)); }
 };
 
 void fill_stats(const DeviceState& h, const Completion& c, dgs_stats* stats) {
@@ -723,8 +718,7 @@ void CUDART_CB completion_callback(void* p) {
 }
 
 // The random start's permutation, staged in pinned memory for its copy to
-// the device; the block returns to the cache with the call's completion (or
-// after the stream drains, on an error path).
+// the device; the block returns to the cache once the copy has been done.
 struct PinnedStart {
     cudaStream_t s;
     void* p = nullptr;
@@ -732,14 +726,8 @@ struct PinnedStart {
     bool copied = false;
     explicit PinnedStart(cudaStream_t st) : s(st) {}
     ~PinnedStart() {
-        if (p == nullptr) return;
-        if (copied) cudaStreamSynchronize(s);
-        pinned_put(p, bytes);
-    }
-    void* release() {
-        void* q = p;
-        p = nullptr;
-        return q;
+        if (copied) pinned_put_after(p, bytes, s);
+        else pinned_put(p, bytes);
     }
 };
 
@@ -770,6 +758,8 @@ dgs_status solve_impl(const int32_t* benefit, int32_t n, int32_t* sigma_out, int
     const bool obj_on_device = device_writable(objective_out, &obj_dev);
     void* status_dev = nullptr;
     const bool status_on_device = o.status_out != nullptr && device_writable(o.status_out, &status_dev);
+    void* stats_dev = nullptr;
+    const bool stats_on_device = stats != nullptr && device_writable(stats, &stats_dev);
 
     EventPair whole;
     if (o.profile) DGS_TRY(whole.begin(stream));
@@ -840,13 +830,16 @@ dgs_status solve_impl(const int32_t* benefit, int32_t n, int32_t* sigma_out, int
             DGS_TRY(enqueue_loop(stream, switching_body, &lc));
         }
     }
-    DGS_CUDA(launch_finish_outputs(S.w, sigma_out, obj_on_device ? static_cast<int64_t*>(obj_dev) : nullptr,
-                                   status_on_device ? static_cast<int32_t*>(status_dev) : nullptr, stream),
-             "finish");
     S.launches += 1;
+    const int32_t sequential = o.algorithm == DGS_ALG_SEQUENTIAL ? 1 : 0;
+    DGS_CUDA(launch_finish_outputs(S.w, sigma_out, obj_on_device ? static_cast<int64_t*>(obj_dev) : nullptr,
+                                   status_on_device ? static_cast<int32_t*>(status_dev) : nullptr,
+                                   stats_on_device ? static_cast<dgs_stats*>(stats_dev) : nullptr,
+                                   S.launches + extra_launches, sequential, stream),
+             "finish");
     if (o.profile) DGS_TRY(whole.end(stream));  // the device work of the solve ends here
-    const bool host_outputs = stats != nullptr || !obj_on_device || (o.status_out && !status_on_device) ||
-                              final_status != nullptr || pin.p != nullptr;
+    const bool host_outputs = (stats != nullptr && !stats_on_device) || !obj_on_device ||
+                              (o.status_out && !status_on_device) || final_status != nullptr;
     if (host_outputs) {
         Completion* c = new Completion();
         c->staged = static_cast<DeviceState*>(pinned_get(sizeof(DeviceState)));
@@ -855,12 +848,12 @@ dgs_status solve_impl(const int32_t* benefit, int32_t n, int32_t* sigma_out, int
             snprintf(g_last_error, sizeof(g_last_error), "pinned staging of the loop state");
             return DGS_ERR_OOM;
         }
-        c->stats = stats;
+        c->stats = stats_on_device ? nullptr : stats;
         c->objective = obj_on_device ? nullptr : objective_out;
         c->status = (o.status_out && !status_on_device) ? o.status_out : nullptr;
         c->status_api = final_status;
         c->launches = S.launches + extra_launches;
-        c->sequential = o.algorithm == DGS_ALG_SEQUENTIAL ? 1 : 0;
+        c->sequential = sequential;
         cudaError_t e = cudaMemcpyAsync(c->staged, S.w.st, sizeof(DeviceState), cudaMemcpyDeviceToHost, stream);
         if (e == cudaSuccess) e = cudaLaunchHostFunc(stream, completion_callback, c);
         if (e != cudaSuccess) {
@@ -868,8 +861,6 @@ dgs_status solve_impl(const int32_t* benefit, int32_t n, int32_t* sigma_out, int
             delete c;
             return cuda_fail(e, "completion");
         }
-        c->release_bytes = pin.bytes;
-        c->release = pin.release();  // returned by the callback
     }
     if (S.w.phase_ns) {  // test/diagnostic output only: waits for the solve
         unsigned long long ph[kPtCount];
@@ -940,7 +931,25 @@ dgs_status dgs_solve_host(const int32_t* benefit_host, int32_t n, int32_t* sigma
     if (e != cudaSuccess) return cuda_fail(e, "device allocation");
     int32_t* a_dev = reinterpret_cast<int32_t*>(buf + obytes);
     int32_t* out_dev = reinterpret_cast<int32_t*>(buf);
-    dgs_status st = DGS_OK, outcome = DGS_OK;
+    dgs_status st = DGS_OK;
+    // the outputs beside sigma come through pinned memory that the device writes
+    struct HostOut {
+        int64_t objective;
+        int32_t status;
+        dgs_stats stats;
+    };
+    HostOut* ho = static_cast<HostOut*>(pinned_get(sizeof(HostOut)));
+    if (ho == nullptr) {
+        cudaFreeAsync(buf, s);
+        snprintf(g_last_error, sizeof(g_last_error), "pinned staging of the results");
+        return DGS_ERR_OOM;
+    }
+    memset(ho, 0, sizeof(*ho));
+    dgs_options o;
+    dgs_default_options(&o);
+    if (options) o = *options;
+    int32_t* const user_status = o.status_out;
+    o.status_out = &ho->status;
     // A large matrix from the greedy start is copied in row bands on a copy
     // stream, and greedy pass 1 takes each band as it lands: the copy (bound
     // by the host link) hides pass 1.
@@ -970,7 +979,7 @@ dgs_status dgs_solve_host(const int32_t* benefit_host, int32_t n, int32_t* sigma
         if (e != cudaSuccess) st = cuda_fail(e, "copy benefit to device");
     }
     if (st == DGS_OK)
-        st = solve_impl(a_dev, n, out_dev, objective_out, options, stats, s, &outcome, 0,
+        st = solve_impl(a_dev, n, out_dev, &ho->objective, &o, stats ? &ho->stats : nullptr, s, nullptr, 0,
                         cs != nullptr ? &bands : nullptr);
     if (st == DGS_OK) {
         e = cudaMemcpyAsync(sigma_out_host, out_dev, (size_t)n * sizeof(int32_t), cudaMemcpyDeviceToHost, s);
@@ -987,7 +996,23 @@ dgs_status dgs_solve_host(const int32_t* benefit_host, int32_t n, int32_t* sigma
     cudaStreamSynchronize(s);
     for (cudaEvent_t x : ev)
         if (x != nullptr) cudaEventDestroy(x);
-    return st == DGS_OK ? outcome : st;
+    if (st == DGS_OK) {
+        *objective_out = ho->objective;
+        if (stats) *stats = ho->stats;
+        st = static_cast<dgs_status>(ho->status);
+        if (user_status) {
+            void* dev = nullptr;  // HOST memory, or the caller's device memory
+            if (device_writable(user_status, &dev)) {
+                e = cudaMemcpyAsync(user_status, &ho->status, sizeof(int32_t), cudaMemcpyDefault, s);
+                if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+                if (e != cudaSuccess) st = cuda_fail(e, "copy status");
+            } else {
+                *user_status = ho->status;
+            }
+        }
+    }
+    pinned_put(ho, sizeof(HostOut));
+    return st;
 }
 
 dgs_status dgs_solve_rect(const int32_t* benefit, int32_t n_agents, int32_t m_jobs, int32_t* assign_out,

@@ -452,10 +452,10 @@ cudaError_t launch_row_tasks(const Workspace& w, cudaStream_t s);
 cudaError_t launch_row_owner_evaluation(const Workspace& w, int32_t conditional, cudaStream_t s);
 cudaError_t launch_finish(const Workspace& w, int32_t* sigma_out, cudaStream_t s);
 // The outputs of a solve: sigma_out (every entry -1 after an error), and,
-// where not null, the objective and the final dgs_status code (device-
-// writable pointers).
+// where not null, the objective, the final dgs_status code and the stats
+// (device-writable pointers; launches: kernels launched from the host).
 cudaError_t launch_finish_outputs(const Workspace& w, int32_t* sigma_out, int64_t* objective, int32_t* status,
-                                  cudaStream_t s);
+                                  dgs_stats* stats, int64_t launches, int32_t sequential, cudaStream_t s);
 // Loop conditions of the device-side loops (see enqueue_while): the greedy
 // rounds' loop (while agents are unmatched), and Algorithm 1's switching loop
 // and passes.
@@ -531,6 +531,9 @@ dgs_status capture_while(cudaStream_t capturing, LoopBody body, void* ctx, unsig
 // process runs; pinned_put may be called from a stream callback).
 void* pinned_get(size_t bytes);
 void pinned_put(void* p, size_t bytes);
+// The block returns once the stream has done what it holds now (not from a
+// callback).
+void pinned_put_after(void* p, size_t bytes, cudaStream_t s);
 
 // Where a result pointer lives: device-writable (device, managed or mapped
 // pinned host memory; *alias = the address kernels use) or plain host memory

@@ -62,9 +62,16 @@ dgs_status fail(cudaError_t e, const char* what) {
     return DGS_ERR_CUDA;
 }
 
-// Pinned staging cache: free blocks by size class (powers of two from 4 KB).
+// Pinned staging cache: free blocks by size class (powers of two from 4 KB),
+// and blocks that return once an event has passed.
 std::mutex g_pin_mutex;
 std::map<size_t, std::vector<void*>> g_pin_free;
+struct PinnedLater {
+    cudaEvent_t ev;
+    void* p;
+    size_t bytes;
+};
+std::vector<PinnedLater> g_pin_later;
 
 size_t pin_class(size_t bytes) {
     size_t c = 4096;
@@ -273,6 +280,18 @@ void* pinned_get(size_t bytes) {
     const size_t c = pin_class(bytes);
     {
         std::lock_guard<std::mutex> lock(g_pin_mutex);
+        for (size_t i = 0; i < g_pin_later.size();) {
+            const PinnedLater x = g_pin_later[i];
+            if (cudaEventQuery(x.ev) != cudaSuccess) {
+                cudaGetLastError();
+                ++i;
+                continue;
+            }
+            cudaEventDestroy(x.ev);
+            g_pin_free[pin_class(x.bytes)].push_back(x.p);
+            g_pin_later[i] = g_pin_later.back();
+            g_pin_later.pop_back();
+        }
         auto it = g_pin_free.find(c);
         if (it != g_pin_free.end() && !it->second.empty()) {
             void* p = it->second.back();
@@ -292,6 +311,22 @@ void pinned_put(void* p, size_t bytes) {
     if (p == nullptr) return;
     std::lock_guard<std::mutex> lock(g_pin_mutex);
     g_pin_free[pin_class(bytes)].push_back(p);
+}
+
+void pinned_put_after(void* p, size_t bytes, cudaStream_t s) {
+    if (p == nullptr) return;
+    cudaEvent_t ev = nullptr;
+    cudaError_t e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventRecord(ev, s);
+    if (e != cudaSuccess) {  // wait instead
+        cudaGetLastError();
+        if (ev) cudaEventDestroy(ev);
+        cudaStreamSynchronize(s);
+        pinned_put(p, bytes);
+        return;
+    }
+    std::lock_guard<std::mutex> lock(g_pin_mutex);
+    g_pin_later.push_back(PinnedLater{ev, p, bytes});
 }
 
 bool device_writable(const void* p, void** alias) {
