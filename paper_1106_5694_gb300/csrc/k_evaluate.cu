@@ -678,12 +678,18 @@ __global__ void keys_to_slots_kernel(Workspace w, int32_t* ag, int32_t* aj, int3
 }  // namespace
 
 // Launch shape of the single-instance evaluation: rows per thread (4: 1024
-// threads per CTA; 8: 512) and strip (column tiles per work item; 0: one
-// contiguous balanced range of tiles per CTA), per size
-// class (bucket = bit length of n - 1).  Defaults until an autotune sets a
-// class; DGS_EVAL_ROWS / DGS_EVAL_STRIP override every class (tests).  The
-// shape never changes a result: every key is a maximum over the same pairs.
-constexpr int kStrip = 8;
+// threads per CTA; 8: 512; 16: 256) and strip (column tiles per work item; 0:
+// one contiguous balanced range of tiles per CTA), per size class (bucket = bit
+// length of n - 1).  Defaults until an autotune sets a class; DGS_EVAL_ROWS /
+// DGS_EVAL_STRIP override every class (tests).  The shape never changes a
+// result: every key is a maximum over the same pairs.
+//
+// The default, 8 rows and contiguous ranges, is the fastest of the autotuner's
+// 16 candidates from n = 128 to 20000 but for 3% at n = 1500 and at 30000: every
+// CTA fills its pipeline once and gets the same number of tiles.  Against
+// strips of 8 tiles (us): n = 256 7.9 / 12.7, 1021 8.3 / 15.0, 4096 26.5 / 38.9,
+// 10000 100 / 120, 20000 383 / 498.
+constexpr EvalShape kDefaultShape{8, 0, 0};
 constexpr int32_t kBuckets = 18;
 std::atomic<int32_t> g_shape[kBuckets];  // 0: default, else tma << 16 | rows << 8 | strip
 
@@ -698,7 +704,7 @@ EvalShape evaluation_shape(int32_t n) {
     static const int32_t env_rows = env_int("DGS_EVAL_ROWS", 0);
     static const int32_t env_strip = env_int("DGS_EVAL_STRIP", -1);
     static const int32_t env_tma = env_int("DGS_EVAL_TMA", -1);
-    EvalShape sh{8, kStrip, 0};
+    EvalShape sh = kDefaultShape;
     const int32_t v = g_shape[size_bucket(n)].load(std::memory_order_relaxed);
     if (v != 0) sh = EvalShape{(v >> 8) & 255, v & 255, v >> 16};
     if (env_rows == 4 || env_rows == 8 || env_rows == 16) sh.rows = env_rows;
