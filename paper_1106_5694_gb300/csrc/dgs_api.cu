@@ -1047,12 +1047,25 @@ dgs_status dgs_evaluate(const int32_t* benefit, int32_t n, const int32_t* sigma_
     Solve S(s);
     DGS_TRY(S.setup(benefit, n, false));
     DGS_TRY(S.init_state(0, nullptr));
-    DGS_CUDA(launch_range_check(S.w, S.a_src, s), "range check");
+    // (rows that have to be re-pitched are checked on the way)
+    const bool checks = S.a_src == nullptr && evaluation_can_check_range(S.w);
+    if (!checks) DGS_CUDA(launch_range_check(S.w, S.a_src, s), "range check");
     DGS_CUDA(launch_start_from_tau(S.w, sigma_in, DGS_INIT_USER, S.seen, s), "start");
-    DGS_CUDA(launch_full_evaluation(S.w, 0, s), "evaluation");
+    DGS_CUDA(checks ? launch_checking_evaluation(S.w, s) : launch_full_evaluation(S.w, 0, s), "evaluation");
     DGS_CUDA(launch_keys_to_slots(S.w, agent_gain, agent_job, job_gain, job_agent, s), "keys to slots");
     DeviceState h;
     DGS_TRY(S.read_state(&h));
+    if (checks && h.status == kError && h.error != kErrRange) {
+        // no evaluation after a bad start; a value out of range is the error to report
+        DGS_CUDA(launch_range_check(S.w, nullptr, s), "range check");
+        DGS_TRY(S.read_state(&h));
+    } else if (checks && h.status != kError && !evaluation_stands(S.w, h.max_abs, h.sample_abs)) {
+        DGS_CUDA(cudaMemsetAsync(S.w.key_a, 0, sizeof(unsigned long long) * (size_t)n, s), "clear keys");
+        DGS_CUDA(cudaMemsetAsync(S.w.key_j, 0, sizeof(unsigned long long) * (size_t)n, s), "clear keys");
+        DGS_CUDA(launch_full_evaluation(S.w, 0, s), "evaluation");
+        DGS_CUDA(launch_keys_to_slots(S.w, agent_gain, agent_job, job_gain, job_agent, s), "keys to slots");
+        DGS_TRY(S.read_state(&h));
+    }
     return map_device_status(h);
 }
 

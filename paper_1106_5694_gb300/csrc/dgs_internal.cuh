@@ -57,7 +57,7 @@ struct DeviceState {
     uint32_t bar_count;      // grid barrier of cooperative launches: arrivals
     uint32_t bar_gen;        //   and generation
     int32_t reeval_all;      // 1: every slot is re-evaluated after a switch (DGS_REEVAL_ALL)
-    int32_t pad_state;
+    int32_t sample_abs;      // max |a| of a sample (an evaluation that checks the range itself)
     int32_t stage;           // kStage* (batched and served solves only)
     int32_t init_mode;       // batched: DGS_INIT_* of the instance (from Instance::init_mode)
     int64_t f;               // current objective
@@ -295,6 +295,21 @@ __device__ __forceinline__ unsigned long long umax64(unsigned long long x, unsig
     return x > y ? x : y;
 }
 
+// |x| of lo <= x <= hi: raises the largest one seen and reports values out of
+// range (whole warps call it).
+__device__ __forceinline__ void report_range(const Workspace& w, int32_t lo, int32_t hi) {
+    // without the overflow of -INT32_MIN
+    int32_t amax = max(hi, lo == INT32_MIN ? INT32_MAX : -lo);
+    amax = (int32_t)__reduce_max_sync(0xffffffffu, (uint32_t)max(amax, 0));
+    if ((threadIdx.x & 31) == 0 && amax) {
+        atomicMax(&w.st->max_abs, amax);
+        if (amax >= kBenefitLimit) {
+            atomicExch(&w.st->error, kErrRange);
+            atomicExch(&w.st->status, kError);
+        }
+    }
+}
+
 // f += the sum of every thread's x over the CTA, by one atomic (the whole CTA
 // calls it, at most 1024 threads).
 __device__ __forceinline__ void add_objective(DeviceState* st, long long x) {
@@ -409,9 +424,8 @@ cudaError_t launch_greedy_best(const Workspace& w, cudaStream_t s);
 cudaError_t launch_greedy_round(const Workspace& w, cudaStream_t s);
 // The greedy start by deferred acceptance (pass 1 with bounds must have run,
 // g_col zero); then the start (sigma, tau, D, f) is read off the jobs' holders.
-// Returns an
-// error (nothing launched) when the launch is refused or DGS_GREEDY_ROUNDS=1;
-// the caller then runs the locally-dominant rounds.
+// Returns an error (nothing launched) when the launch is refused or
+// DGS_GREEDY_ROUNDS=1; the caller then runs the locally-dominant rounds.
 // real_n / real_m: the agents and jobs that are real (below n: the others are
 // the zero rows or columns of a padded instance; at most one of the two).
 // (free_a has to be zero, rescan_list is written.)
@@ -421,6 +435,13 @@ cudaError_t launch_range_check(const Workspace& w, const int32_t* a_src, cudaStr
 cudaError_t launch_start_from_tau(const Workspace& w, const int32_t* user_tau, int32_t mode, uint8_t* seen,
                                   cudaStream_t s);
 cudaError_t launch_full_evaluation(const Workspace& w, int32_t conditional, cudaStream_t s);
+// A full evaluation that checks the range of a as it reads it (see
+// range_sample_kernel); not for every launch shape.  Its keys stand when
+// evaluation_stands(w, max |a|, the sample's max); else they have to be zeroed
+// and evaluated again.
+bool evaluation_can_check_range(const Workspace& w);
+cudaError_t launch_checking_evaluation(const Workspace& w, cudaStream_t s);
+bool evaluation_stands(const Workspace& w, int32_t max_abs, int32_t sample_abs);
 // Launch shape of the full evaluation (rows per thread 4 or 8; strip: column
 // tiles per work item, 0 = one contiguous balanced range of tiles per CTA;
 // tma: X tiles by TMA gathers).

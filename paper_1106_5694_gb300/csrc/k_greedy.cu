@@ -23,21 +23,6 @@ namespace {
 
 constexpr int kT = 64;  // tile edge
 
-// |x| of lo <= x <= hi: raises the largest one seen and reports values out of
-// range (whole warps call it).
-__device__ __forceinline__ void report_range(const Workspace& w, int32_t lo, int32_t hi) {
-    // without the overflow of -INT32_MIN
-    int32_t amax = max(hi, lo == INT32_MIN ? INT32_MAX : -lo);
-    amax = (int32_t)__reduce_max_sync(0xffffffffu, (uint32_t)max(amax, 0));
-    if ((threadIdx.x & 31) == 0 && amax) {
-        atomicMax(&w.st->max_abs, amax);
-        if (amax >= kBenefitLimit) {
-            atomicExch(&w.st->error, kErrRange);
-            atomicExch(&w.st->status, kError);
-        }
-    }
-}
-
 // Pass 1 over 64 x 64 tiles, 256 threads.  A tile's rows go to shared memory in
 // 16-byte chunks, chunk c of row r at place c ^ (r / 4 mod 16): a row's chunks
 // fill all banks, and so do the chunks c of eight rows 4l that the transposing
@@ -718,7 +703,8 @@ __global__ void __launch_bounds__(256) greedy_da_start_kernel(Workspace w) {
     add_objective(st, f);
 }
 
-// |a| < 2^29 check alone (for entry points that do not run pass 1).  The pitched
+// |a| < 2^29 check alone (for calls that neither run pass 1 nor a checking
+// evaluation).  The pitched
 // rows are read as one array (padding columns are 0, which changes nothing),
 // four 16-byte loads in flight per thread: HBM-bound (n = 10000, 400 MB: 115
 // us with one load in flight and a column test per element, now 62).
