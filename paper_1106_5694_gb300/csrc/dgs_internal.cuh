@@ -170,36 +170,9 @@ __device__ __forceinline__ void for_each_entry(const BatchTable& t, int32_t stag
 
 // Work queue of one batched launch: off[k] = first item of slot k, off[cap] =
 // total (exclusive prefix of the per-slot item counts, written by the scan
-// kernel just before the consumer).  CTA b takes the contiguous items
-// [b * per, (b + 1) * per) and calls f(instance, local item, items of that
-// slot) for each, the whole CTA together.
-template <typename F>
-__device__ __forceinline__ void for_each_item(const Instance* inst, const int32_t* off, int32_t cap, F&& f) {
-    const int32_t total = off[cap];
-    if (total <= 0) return;
-    const int32_t per = (total + (int32_t)gridDim.x - 1) / (int32_t)gridDim.x;
-    int32_t item = (int32_t)blockIdx.x * per;
-    const int32_t end = min(total, item + per);
-    if (item >= end) return;
-    int32_t lo = 0, hi = cap;  // off[lo] <= item < off[hi]
-    while (hi - lo > 1) {
-        const int32_t mid = (lo + hi) >> 1;
-        if (off[mid] <= item) lo = mid;
-        else hi = mid;
-    }
-    int32_t k = lo, first = off[k], next = off[k + 1];
-    for (; item < end; ++item) {
-        while (item >= next) {
-            ++k;
-            first = next;
-            next = off[k + 1];
-        }
-        f(inst[k], item - first, next - first);
-    }
-}
-
-// The slot k with off[k] <= g < off[k + 1] (off as above, 0 <= g < off[cap]):
-// 32 probes at a time, by a whole warp, every lane with the same g.
+// kernel just before the consumer).  The slot k with off[k] <= g < off[k + 1]
+// (0 <= g < off[cap]): 32 probes at a time, by a whole warp, every lane with
+// the same g.
 __device__ __forceinline__ int32_t find_slot(const int32_t* off, int32_t cap, int32_t g) {
     const int lane = threadIdx.x & 31;
     int32_t lo = 0, hi = cap;
