@@ -636,7 +636,9 @@ template <int kRows, bool kTma = false, bool kRange = false>
 __device__ __forceinline__ void full_evaluation_body(const Workspace& w, int32_t conditional, const Schedule& sc,
                                                      const CUtensorMap* tm = nullptr) {
     DeviceState* st = w.st;
-    if (st->status != kRunning) return;
+    // (kRange: another CTA may report a value out of range meanwhile, so the
+    // CTA decides as one)
+    if (kRange ? __syncthreads_or(st->status != kRunning) : (int)(st->status != kRunning)) return;
     if (conditional && !(st->need_update && use_full_update(st->rescan_count, w.n, st->update_policy))) return;
     if (conditional && blockIdx.x == 0 && threadIdx.x == 0) st->full_evals += 1;
     const Packing pk = packing_for(w.n, kRange ? st->sample_abs : st->max_abs);
