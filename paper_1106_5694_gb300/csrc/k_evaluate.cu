@@ -274,14 +274,14 @@ __device__ __forceinline__ unsigned long long unpack_key(int32_t key, const Pack
 // block J).  Packed path (when |gain| * 2^s fits in int32, s = index bits):
 // two int32 keys per row, (gain << s) + (mask - column) in g and (gain << s) +
 // (mask - partner agent) in s, whose max picks the larger gain, then the lower
-// index; ca / cj: mask - row and mask - sigma(row), the column-side tie
-// offsets.  Exact path: best gain g, its lowest column c, lowest partner
+// index; ca / cj: mask - the first row and mask - sigma(row), the column-side
+// tie offsets.  Exact path: best gain g, its lowest column c, lowest partner
 // agent s among the columns reaching it; sj = sigma of the rows.
 template <int kRows, bool kPacked>
 struct Rows {
     int32_t g[kRows], s[kRows], d[kRows];
     int32_t c[kPacked ? 1 : kRows];
-    int32_t ca[kPacked ? kRows : 1], cj[kPacked ? kRows : 1];
+    int32_t ca, cj[kPacked ? kRows : 1];
     int32_t sj[kPacked ? 1 : kRows];
 };
 
@@ -295,7 +295,7 @@ __device__ __forceinline__ void rows_start(Rows<kRows, kPacked>& rs, const Stage
         if (kPacked) {
             rs.g[r] = pk.mask;
             rs.s[r] = pk.mask;
-            rs.ca[r] = pk.mask - (J0 + ty * kRows + r);
+            if (r == 0) rs.ca = pk.mask - (J0 + ty * kRows);
             rs.cj[r] = pk.mask - stage->sj[ty * kRows + r];
         } else {
             rs.g[r] = 0;
@@ -358,7 +358,7 @@ __device__ __forceinline__ void compute_tile(const Stage* stage, Rows<kRows, kPa
                     const uint32_t hs = (uint32_t)(x + yv[e] - rs.d[r]) * pw;
                     rs.g[r] = max(rs.g[r], (int32_t)(hs + cka));  // row jr, lowest column
                     rs.s[r] = max(rs.s[r], (int32_t)(hs + ckj));  // row jr, lowest partner agent
-                    ta[r] = (int32_t)(hs + (uint32_t)rs.ca[r]);   // row k, lowest column (+ D[k] 2^s)
+                    ta[r] = (int32_t)(hs - (uint32_t)r);          // row k, lowest column (+ D[k] 2^s - ca)
                     tj[r] = (int32_t)(hs + (uint32_t)rs.cj[r]);   // row k, lowest partner agent (+ D[k] 2^s)
                 }
             }
@@ -371,7 +371,7 @@ __device__ __forceinline__ void compute_tile(const Stage* stage, Rows<kRows, kPa
                 }
             }
             if (!kRagged || ta[0] != INT32_MIN) {
-                ca = max(ca, (int32_t)((uint32_t)ta[0] - dks));
+                ca = max(ca, (int32_t)((uint32_t)ta[0] + (uint32_t)rs.ca - dks));
                 cj = max(cj, (int32_t)((uint32_t)tj[0] - dks));
             }
         } else {
@@ -692,21 +692,63 @@ __global__ void __launch_bounds__(256) range_sample_kernel(Workspace w) {
 }
 
 // Batched: the tiles of every instance that needs an evaluation (queued by the
-// scan kernel) in one order, an equal contiguous range of them per CTA, so
-// that the pipeline is filled once per instance and CTA.  (Items of two strips
-// of eight tiles, equal numbers of items per CTA: 1024 peer-shaped instances,
-// n in [64, 4096], 5.6 ms, now 3.5.)
+// scan kernel) in one order, cut into equal contiguous runs of about kBatchRun
+// tiles that the CTAs take in turn (the pipeline is filled once per run and
+// instance, which costs about 8 us).  The walk over the runs is warp 0's, and
+// its state and the instance's pointers are in shared memory: the tile loop
+// needs every register, and next to 226 KB of shared memory there is hardly any
+// L1 for spilled ones (1024 peer-shaped instances, n in [64, 4096]: 3.5 ms with
+// 96 bytes spilled and one range per CTA, 8.9 ms with 216 bytes, 2.5 now; runs
+// of 64 tiles 5% slower, of 640 the same).
+constexpr int32_t kBatchRun = 256;
+struct BatchWalk {
+    Workspace w;
+    int32_t part, at, end;  // the run, its next tile and one past its last
+    int32_t k;              // the slot of tile at
+    int32_t lo, hi;         // tiles of the current instance; lo == hi: done
+};
+__device__ __forceinline__ void next_run(const BatchQueues& q, BatchWalk& s) {
+    const int32_t grid = (int32_t)gridDim.x, *off = q.q0, cap = q.cap;
+    const int64_t total = off[cap];
+    const int32_t parts = max(1, (int32_t)(total / ((int64_t)grid * kBatchRun))) * grid;
+    int32_t part = s.part, at = s.at, end = s.end, k = s.k;
+    __syncwarp();
+    if (at >= end) {
+        do {
+            part += grid;
+            at = (int32_t)(total * part / parts);
+            end = (int32_t)(total * (part + 1) / parts);
+        } while (part < parts && at >= end);
+        if (part < parts) k = find_slot(off, cap, at);
+    }
+    const bool more = part < parts;
+    if (more)
+        while (off[k + 1] <= at) ++k;
+    const int32_t first = more ? off[k] : 0, next = more ? min(end, off[k + 1]) : 0;
+    if ((threadIdx.x & 31) == 0) {
+        if (more) s.w = q.inst[k].w;
+        s.part = part;
+        s.end = end;
+        s.k = k;
+        s.lo = more ? at - first : 0;
+        s.hi = more ? next - first : 0;
+        s.at = next;
+    }
+}
 template <int kRows>
 __global__ void __launch_bounds__(Geo<kRows>::kThreads, 1) full_evaluation_batched_kernel(BatchQueues q) {
-    // (a copy: pointers read from global memory would be read again after
-    // every key update, which might have changed them)
-    __shared__ Workspace w;
-    for_each_range(q.inst, q.q0, q.cap, blockIdx.x, gridDim.x, [&](const Instance& in, int32_t lo, int32_t hi) {
-        __syncthreads();  // the copy is no longer read
-        if (threadIdx.x == 0) w = in.w;
+    __shared__ BatchWalk s;
+    if (threadIdx.x == 0) {
+        s.part = (int32_t)blockIdx.x - (int32_t)gridDim.x;
+        s.at = s.end = s.k = 0;
+    }
+    for (;;) {
+        __syncthreads();  // the last run's copy is no longer read
+        if (threadIdx.x < 32) next_run(q, s);
         __syncthreads();
-        full_evaluation_body<kRows>(w, 0, Schedule{0, 0, 1, lo, hi});
-    });
+        if (s.lo >= s.hi) break;
+        full_evaluation_body<kRows>(s.w, 0, Schedule{0, 0, 1, s.lo, s.hi});
+    }
 }
 
 // agent slot i <- key_a[tau(i)], job slot j <- key_j[j]  (public evaluation
