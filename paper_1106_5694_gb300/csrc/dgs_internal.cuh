@@ -54,8 +54,6 @@ struct DeviceState {
     int32_t update_policy;   // 0: by cost, 1: always full evaluation, 2: always row tasks
     int32_t max_abs;         // max |a| (set by the passes that check the range)
     long long greedy_rescans;  // greedy start: tiles of an agent's row looked at (rounds: rows rescanned)
-    uint32_t bar_count;      // grid barrier of cooperative launches: arrivals
-    uint32_t bar_gen;        //   and generation
     int32_t reeval_all;      // 1: every slot is re-evaluated after a switch (DGS_REEVAL_ALL)
     int32_t sample_abs;      // max |a| of a sample (an evaluation that checks the range itself)
     int32_t stage;           // kStage* (batched and served solves only)
@@ -348,37 +346,6 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
 // 1-D bulk prefetch into L2; src 16-byte aligned, bytes a multiple of 16.
 __device__ __forceinline__ void bulk_prefetch_l2(const void* src, uint32_t bytes) {
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
-}
-
-// Grid-wide barrier for cooperative launches (every CTA co-resident).  The
-// wait is bounded in time; returns false (block-uniform) on timeout.
-constexpr uint64_t kBarrierTimeoutNs = 4000000000ull;
-__device__ __forceinline__ bool grid_barrier(DeviceState* st) {
-    __shared__ int32_t s_bar_ok;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        uint32_t g;
-        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(g) : "l"(&st->bar_gen) : "memory");
-        uint32_t prev;
-        asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(prev) : "l"(&st->bar_count) : "memory");
-        int32_t ok = 1;
-        if (prev == gridDim.x - 1) {
-            asm volatile("st.relaxed.gpu.global.u32 [%0], 0;" ::"l"(&st->bar_count) : "memory");
-            asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&st->bar_gen) : "memory");
-        } else {
-            const uint64_t t0 = globaltimer_ns();
-            for (;;) {
-                uint32_t cur;
-                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(cur) : "l"(&st->bar_gen) : "memory");
-                if (cur != g) break;
-                if (globaltimer_ns() - t0 > kBarrierTimeoutNs) { ok = 0; break; }
-                __nanosleep(20);
-            }
-        }
-        s_bar_ok = ok;
-    }
-    __syncthreads();
-    return s_bar_ok != 0;
 }
 
 // ------------------------------------------------------ host-side launchers
