@@ -2,15 +2,17 @@
 // and the host loop that enqueues the kernels of one solve.
 //
 // Solve flow (Algorithm 3, Section 5, plus the greedy start of Section 3.1):
-//   pass 1        transpose a -> at, |a| < 2^29 check, first greedy round keys
-//   greedy rounds match mutually-best pairs, rescan rows/columns (device loop,
-//                 checked from the host every few rounds)
-//   start         sigma, D, f from the starting tau
+//   pass 1        transpose a -> at, |a| < 2^29 check, bounds on every
+//                 agent's best benefit in each tile of jobs
+//   greedy start  deferred acceptance; sigma, D, f read off the jobs' holders
+//                 (another start: one kernel from the given tau)
 //   evaluation    full difference evaluation (every slot)
-//   switching     controller (quiet sweeps on one CTA) ->
-//                 [mark rescan rows -> full evaluation | row tasks] -> controller ...
-// The host reads the 100-byte loop state every few launches to learn when the
-// loop has ended; everything else stays on the device.
+//   switching     a conditional graph node whose body is [mark -> full
+//                 evaluation | row tasks -> prepare -> controller], the
+//                 controller running quiet sweeps on one CTA
+//   finish        sigma, objective, status and statistics to the caller
+// The host only enqueues; it waits for the loop state where a call returns
+// its result by value (evaluation, greedy start, host matrices, profiling).
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>

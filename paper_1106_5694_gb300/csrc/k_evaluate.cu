@@ -19,7 +19,7 @@
 // pipeline (one barrier per tile).  Every element of a is read exactly once
 // per evaluation.  (One-dimensional TMA bulk copies of the same 256-byte
 // segments were measured request-rate bound at about 1.5 TB/s on GB300, which
-// is why the copies are issued by the threads.)  A CTA walks a strip of tiles
+// is why the copies are issued by the threads.)  A CTA walks a run of tiles
 // with the same J, keeping the row-side maxima of its 64 rows in registers;
 // column-side maxima of each tile are combined across the CTA in shared
 // memory at the next barrier and committed with 64-bit atomicMax, which is

@@ -823,7 +823,7 @@ __global__ void __launch_bounds__(kDaThreads, kDaPerSm) greedy_da_batched_kernel
 }
 
 // The assignment of every instance in kStageGreedy from its jobs' holders
-// (greedy_da_finish_kernel per instance).
+// (D and f follow in the start kernel).
 __global__ void greedy_da_finish_batched_kernel(BatchTable t) {
     for_each_entry(t, kStageGreedy, [&](const Instance& in, int32_t bid, int32_t nblk) {
         const Workspace& w = in.w;
