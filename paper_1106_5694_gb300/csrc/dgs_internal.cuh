@@ -505,19 +505,20 @@ bool device_writable(const void* p, void** alias);
 // grids of the persistent and grid-stride kernels are multiples of it).
 int32_t device_sms();
 
-constexpr int kSmemSlots = 24;
-
-// Raise a kernel's dynamic shared memory limit once per device (slot = one
-// small integer per kernel).
-inline cudaError_t ensure_smem_limit(const void* func, int slot, size_t bytes) {
-    static int done[kSmemSlots][64] = {};
+// Raise the dynamic shared memory limit of kernel kKernel on the current
+// device to at least `bytes` (each kernel has a record of its own: a limit
+// raised for one says nothing about another's).
+template <auto kKernel>
+inline cudaError_t ensure_smem_limit(size_t bytes) {
+    static int done[64] = {};
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= 64 || slot < 0 || slot >= kSmemSlots) return cudaErrorInvalidValue;
-    if (done[slot][dev] >= (int)bytes) return cudaSuccess;
-    e = cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    if (e == cudaSuccess) done[slot][dev] = (int)bytes;
+    if (dev < 0 || dev >= 64) return cudaErrorInvalidValue;
+    if (done[dev] >= (int)bytes) return cudaSuccess;
+    e = cudaFuncSetAttribute(reinterpret_cast<const void*>(kKernel), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)bytes);
+    if (e == cudaSuccess) done[dev] = (int)bytes;
     return e;
 }
 

@@ -1660,13 +1660,12 @@ bool use_small_loop(const Workspace& w) {
 }
 
 template <int kT>
-static cudaError_t launch_small_loop_t(const Workspace& w, const CtlGlobal& gs, cudaStream_t s, int slot) {
+static cudaError_t launch_small_loop_t(const Workspace& w, const CtlGlobal& gs, cudaStream_t s) {
     const int32_t mode = controller_smem_mode(w.n);
     const size_t smem = controller_smem_bytes(w.n);
     CtlScratch c{gs.res, gs.claimed, gs.estate, gs.edges, gs.acc};
-    const void* fn = reinterpret_cast<const void*>(small_loop_kernel<uint32_t, kT>);
     if (smem + kCtlStaticSmem > 48 * 1024) {
-        cudaError_t e = ensure_smem_limit(fn, slot, smem);
+        cudaError_t e = ensure_smem_limit<small_loop_kernel<uint32_t, kT>>(smem);
         if (e != cudaSuccess) return e;
     }
     const bool short_wrap = env_short_wraps() != 0;
@@ -1687,9 +1686,9 @@ int32_t small_loop_threads() {
 
 cudaError_t launch_small_loop(const Workspace& w, const CtlGlobal& gs, cudaStream_t s) {
     switch (small_loop_threads()) {
-        case 1024: return launch_small_loop_t<1024>(w, gs, s, 14);
-        case 512: return launch_small_loop_t<512>(w, gs, s, 15);
-        default: return launch_small_loop_t<256>(w, gs, s, 8);
+        case 1024: return launch_small_loop_t<1024>(w, gs, s);
+        case 512: return launch_small_loop_t<512>(w, gs, s);
+        default: return launch_small_loop_t<256>(w, gs, s);
     }
 }
 
@@ -1699,10 +1698,9 @@ cudaError_t launch_controller_impl(const Workspace& w, const CtlGlobal& gs, cuda
     const size_t smem = controller_smem_bytes(w.n);
     CtlScratch c{gs.res, gs.claimed, gs.estate, gs.edges, gs.acc};
     const bool narrow = w.n <= 65535;
-    const void* fn = narrow ? reinterpret_cast<const void*>(controller_kernel<uint32_t>)
-                            : reinterpret_cast<const void*>(controller_kernel<unsigned long long>);
     if (smem + kCtlStaticSmem > 48 * 1024) {
-        cudaError_t e = ensure_smem_limit(fn, narrow ? 1 : 3, smem);
+        cudaError_t e = narrow ? ensure_smem_limit<controller_kernel<uint32_t>>(smem)
+                               : ensure_smem_limit<controller_kernel<unsigned long long>>(smem);
         if (e != cudaSuccess) return e;
     }
     const bool short_wrap = env_short_wraps() != 0;
@@ -1743,7 +1741,7 @@ cudaError_t launch_row_tasks(const Workspace& w, cudaStream_t s) {
         const int fit = (int)((227 * 1024) / (smem + 2048));
         grid = dgs::device_sms() * (fit > 4 ? 4 : fit < 1 ? 1 : fit);
         if (smem > 48 * 1024) {
-            cudaError_t e = ensure_smem_limit(reinterpret_cast<const void*>(row_tasks_kernel<true>), 2, smem);
+            cudaError_t e = ensure_smem_limit<row_tasks_kernel<true>>(smem);
             if (e != cudaSuccess) return e;
         }
         row_tasks_kernel<true><<<grid, 512, smem, s>>>(w);
@@ -1760,8 +1758,7 @@ cudaError_t launch_row_owner_evaluation(const Workspace& w, int32_t conditional,
     if (w.n <= kRowOwnerStageMaxN) {
         const size_t smem = 2 * 4 * (size_t)w.ldt;
         if (smem > 48 * 1024) {
-            cudaError_t e =
-                ensure_smem_limit(reinterpret_cast<const void*>(row_owner_evaluation_kernel<true>), 12, smem);
+            cudaError_t e = ensure_smem_limit<row_owner_evaluation_kernel<true>>(smem);
             if (e != cudaSuccess) return e;
         }
         const int per_sm = smem <= 110 * 1024 ? 2 : 1;
@@ -1802,9 +1799,8 @@ cudaError_t launch_b_mark_rescan(const BatchTable& rows, cudaStream_t s) {
 // max_n: no queued instance is larger.  128 threads per row up to n = 4096 (a
 // row is then at most 16 KB, 13 CTAs per SM), else 512.
 template <int kT>
-static cudaError_t launch_b_row_tasks_t(const BatchQueues& q, size_t smem, int slot, cudaStream_t s) {
-    const void* fn = reinterpret_cast<const void*>(row_tasks_batched_kernel<kT>);
-    cudaError_t e = ensure_smem_limit(fn, slot, smem);
+static cudaError_t launch_b_row_tasks_t(const BatchQueues& q, size_t smem, cudaStream_t s) {
+    cudaError_t e = ensure_smem_limit<row_tasks_batched_kernel<kT>>(smem);
     if (e != cudaSuccess) return e;
     const int by_smem = (int)((227 * 1024) / (smem + 2048)), by_threads = 2048 / kT;
     const int per_sm = std::max(1, std::min({by_smem, by_threads, 13}));
@@ -1814,7 +1810,7 @@ static cudaError_t launch_b_row_tasks_t(const BatchQueues& q, size_t smem, int s
 
 cudaError_t launch_b_row_tasks(const BatchQueues& q, int32_t max_n, cudaStream_t s) {
     const size_t smem = 4 * (size_t)((max_n + 63) / 64 * 64);
-    return max_n <= 4096 ? launch_b_row_tasks_t<128>(q, smem, 6, s) : launch_b_row_tasks_t<512>(q, smem, 17, s);
+    return max_n <= 4096 ? launch_b_row_tasks_t<128>(q, smem, s) : launch_b_row_tasks_t<512>(q, smem, s);
 }
 
 cudaError_t launch_b_scan(const BatchQueues& q, int32_t phase, cudaStream_t s) {
@@ -1831,7 +1827,7 @@ cudaError_t launch_b_prepare_edges(const BatchTable& rows, cudaStream_t s) {
 // 32-bit edge words); each CTA lays out its shared memory for its own n.
 cudaError_t launch_b_controller(const BatchTable& one, cudaStream_t s) {
     const size_t smem = kCtlSmemLimit;
-    cudaError_t e = ensure_smem_limit(reinterpret_cast<const void*>(controller_batched_kernel), 5, smem);
+    cudaError_t e = ensure_smem_limit<controller_batched_kernel>(smem);
     if (e != cudaSuccess) return e;
     const bool short_wrap = env_short_wraps() != 0;
     controller_batched_kernel<<<dgs::device_sms(), kCtlThreads, smem, s>>>(one, short_wrap ? 4u : kRoundSpanMax,

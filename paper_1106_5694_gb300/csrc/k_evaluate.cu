@@ -855,10 +855,7 @@ template <int kRows, bool kTma, bool kRange = false>
 static cudaError_t launch_eval(const Workspace& w, int32_t conditional, int32_t strip, const CUtensorMap& tm,
                                cudaStream_t s) {
     constexpr size_t smem = eval_smem_bytes<kRows>();
-    // attribute cache slots
-    const int slot = kRange ? 17 : kRows == 16 ? 13 : kRows == 8 ? (kTma ? 11 : 0) : (kTma ? 10 : 7);
-    cudaError_t e =
-        ensure_smem_limit(reinterpret_cast<const void*>(full_evaluation_kernel<kRows, kTma, kRange>), slot, smem);
+    cudaError_t e = ensure_smem_limit<full_evaluation_kernel<kRows, kTma, kRange>>(smem);
     if (e != cudaSuccess) return e;
     full_evaluation_kernel<kRows, kTma, kRange><<<dgs::device_sms(), Geo<kRows>::kThreads, smem, s>>>(w, conditional, strip, tm);
     return cudaGetLastError();
@@ -899,7 +896,7 @@ bool evaluation_stands(const Workspace& w, int32_t max_abs, int32_t sample_abs) 
 // workspace pointers it reads from global memory).
 cudaError_t launch_b_evaluation(const BatchQueues& q, cudaStream_t s) {
     constexpr size_t smem = eval_smem_bytes<8>();
-    cudaError_t e = ensure_smem_limit(reinterpret_cast<const void*>(full_evaluation_batched_kernel<8>), 4, smem);
+    cudaError_t e = ensure_smem_limit<full_evaluation_batched_kernel<8>>(smem);
     if (e != cudaSuccess) return e;
     full_evaluation_batched_kernel<8><<<dgs::device_sms(), Geo<8>::kThreads, smem, s>>>(q);
     return cudaGetLastError();

@@ -938,7 +938,7 @@ cudaError_t launch_greedy_da(const Workspace& w, int32_t real_n, int32_t real_m,
     if (greedy_rounds_env() || w.g_bound == nullptr) return cudaErrorNotSupported;
     constexpr int kGroups = kDaWarps / kDaGroup;
     const size_t smem = sizeof(uint32_t) * kGroups * (size_t)w.bound_tiles;
-    cudaError_t e = ensure_smem_limit(reinterpret_cast<const void*>(greedy_da_kernel<kDaGroup>), 16, smem);
+    cudaError_t e = ensure_smem_limit<greedy_da_kernel<kDaGroup>>(smem);
     if (e != cudaSuccess) return e;
     const int32_t most = (w.n + kGroups - 1) / kGroups;
     const int32_t grid = most < da_grid(smem) ? most : da_grid(smem);

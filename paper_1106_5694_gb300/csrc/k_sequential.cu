@@ -251,7 +251,7 @@ cudaError_t launch_sequential(const Workspace& w, cudaStream_t s) {
     const int32_t in_smem = w.n <= kSeqSmemMaxN ? 1 : 0;
     const size_t smem = in_smem ? 8 * (size_t)w.n : 0;
     if (smem > 48 * 1024) {
-        cudaError_t e = ensure_smem_limit(reinterpret_cast<const void*>(sequential_kernel), 9, smem);
+        cudaError_t e = ensure_smem_limit<sequential_kernel>(smem);
         if (e != cudaSuccess) return e;
     }
     sequential_kernel<<<1, kSeqThreads, smem, s>>>(w, in_smem);
