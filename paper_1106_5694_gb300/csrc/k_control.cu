@@ -1740,10 +1740,9 @@ cudaError_t launch_row_tasks(const Workspace& w, cudaStream_t s) {
         // rows of an update then go in one wave
         const int fit = (int)((227 * 1024) / (smem + 2048));
         grid = dgs::device_sms() * (fit > 4 ? 4 : fit < 1 ? 1 : fit);
-        if (smem > 48 * 1024) {
-            cudaError_t e = ensure_smem_limit<row_tasks_kernel<true>>(smem);
-            if (e != cudaSuccess) return e;
-        }
+        // (at every size: what a kernel has without, 48 KB, includes its static part)
+        cudaError_t e = ensure_smem_limit<row_tasks_kernel<true>>(smem);
+        if (e != cudaSuccess) return e;
         row_tasks_kernel<true><<<grid, 512, smem, s>>>(w);
     } else {
         row_tasks_kernel<false><<<grid, 512, 0, s>>>(w);
@@ -1757,10 +1756,8 @@ constexpr int32_t kRowOwnerStageMaxN = 27 * 1024;
 cudaError_t launch_row_owner_evaluation(const Workspace& w, int32_t conditional, cudaStream_t s) {
     if (w.n <= kRowOwnerStageMaxN) {
         const size_t smem = 2 * 4 * (size_t)w.ldt;
-        if (smem > 48 * 1024) {
-            cudaError_t e = ensure_smem_limit<row_owner_evaluation_kernel<true>>(smem);
-            if (e != cudaSuccess) return e;
-        }
+        cudaError_t e = ensure_smem_limit<row_owner_evaluation_kernel<true>>(smem);
+        if (e != cudaSuccess) return e;
         const int per_sm = smem <= 110 * 1024 ? 2 : 1;
         row_owner_evaluation_kernel<true><<<dgs::device_sms() * per_sm, 512, smem, s>>>(w, conditional);
     } else {

@@ -250,10 +250,8 @@ cudaError_t launch_slots_from_keys(const Workspace& w, cudaStream_t s) {
 cudaError_t launch_sequential(const Workspace& w, cudaStream_t s) {
     const int32_t in_smem = w.n <= kSeqSmemMaxN ? 1 : 0;
     const size_t smem = in_smem ? 8 * (size_t)w.n : 0;
-    if (smem > 48 * 1024) {
-        cudaError_t e = ensure_smem_limit<sequential_kernel>(smem);
-        if (e != cudaSuccess) return e;
-    }
+    cudaError_t e = ensure_smem_limit<sequential_kernel>(smem);
+    if (e != cudaSuccess) return e;
     sequential_kernel<<<1, kSeqThreads, smem, s>>>(w, in_smem);
     return cudaGetLastError();
 }

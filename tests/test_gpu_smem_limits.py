@@ -70,3 +70,36 @@ ref_st, ref, ref_obj, _ = B.dgs_solve_ex(a)
 assert res[0] == B.DGS_OK == ref_st, (res[0], B.dgs_last_cuda_error())
 assert res[2] == ref_obj and torch.equal(torch.as_tensor(res[1]).cpu(), ref.cpu())
 """, DGS_SERVER_SOLO_N="0")
+
+
+# 48 KB of a kernel's shared memory need no raised limit, static and dynamic
+# taken together: rows of exactly 48 KB beside the static part do.
+@pytest.mark.parametrize("n,evaluation,other", [(12225, "TILE_PAIRS", "ROW_OWNER"), (12288, "TILE_PAIRS", "ROW_OWNER"),
+                                                (6144, "ROW_OWNER", "TILE_PAIRS"), (6081, "ROW_OWNER", "TILE_PAIRS")])
+def test_rows_of_48_kb_in_a_fresh_process(n, evaluation, other):
+    _run(f"""
+a = matrix({n}, 1)
+st, sig, f, _ = B.dgs_solve_ex(a, max_sweeps=40, evaluation=B.DGS_EVAL_{evaluation})
+assert st in (B.DGS_OK, B.DGS_TIMEOUT), (st, B.dgs_last_cuda_error())
+big = matrix(12800, 2)  # raises every limit
+assert B.dgs_solve_ex(big, max_sweeps=1, evaluation=B.DGS_EVAL_{evaluation})[0] in (B.DGS_OK, B.DGS_TIMEOUT)
+st, ref, ref_f, _ = B.dgs_solve_ex(a, max_sweeps=40, evaluation=B.DGS_EVAL_{other})
+assert st in (B.DGS_OK, B.DGS_TIMEOUT), (st, B.dgs_last_cuda_error())
+assert f == ref_f and torch.equal(sig, ref)
+""")
+
+
+@pytest.mark.parametrize("n", [6144, 6110])
+def test_sequential_algorithm_of_48_kb_in_a_fresh_process(n):
+    _run(f"""
+def seq(a):
+    st, sig, f, _ = B.dgs_solve_ex(a, max_sweeps=5, algorithm=B.DGS_ALG_SEQUENTIAL)
+    assert st in (B.DGS_OK, B.DGS_TIMEOUT), (st, B.dgs_last_cuda_error())
+    return sig, f
+
+a = matrix({n}, 1)
+sig, f = seq(a)
+seq(matrix(6400, 2))  # raises the limit
+ref, ref_f = seq(a)
+assert f == ref_f and torch.equal(sig, ref)
+""")
