@@ -8,6 +8,7 @@
 // to them); here the loop's continuation is decided by the last kernel of
 // each iteration on the device, and a call returns once its work is queued.
 #include <cstdio>
+#include <cstdlib>
 #include <cstring>
 #include <map>
 #include <mutex>
@@ -94,6 +95,21 @@ dgs_status create_loop_handle(cudaStream_t capturing, unsigned long long* handle
     return DGS_OK;
 }
 
+namespace {
+// DGS_FAKE_LOOP_REFUSAL=1 (tests; read at every capture): the loop body's
+// launch is one that the runtime refuses (no block has 2048 threads).
+bool fake_refusal() {
+    const char* e = std::getenv("DGS_FAKE_LOOP_REFUSAL");
+    return e && std::atoi(e) == 1;
+}
+__global__ void refused_kernel() {}
+dgs_status refused_body(cudaStream_t s) {
+    refused_kernel<<<1, 2048, 0, s>>>();
+    const cudaError_t e = cudaGetLastError();
+    return e == cudaSuccess ? DGS_OK : fail(e, "loop body");
+}
+}  // namespace
+
 dgs_status capture_while(cudaStream_t capturing, LoopBody body, void* ctx, unsigned long long handle) {
     cudaStreamCaptureStatus cst = cudaStreamCaptureStatusNone;
     cudaGraph_t g = nullptr;
@@ -127,10 +143,13 @@ dgs_status capture_while(cudaStream_t capturing, LoopBody body, void* ctx, unsig
     cudaGraph_t bg = p.conditional.phGraph_out[0];
     e = cudaStreamBeginCaptureToGraph(cs.s, bg, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed);
     if (e != cudaSuccess) return fail(e, "loop body capture");
-    const dgs_status st = body(ctx, cs.s, (unsigned long long)h);
+    const dgs_status st = fake_refusal() ? refused_body(cs.s) : body(ctx, cs.s, (unsigned long long)h);
     cudaGraph_t out = nullptr;
     e = cudaStreamEndCapture(cs.s, &out);
-    if (st != DGS_OK) return st;
+    if (st != DGS_OK) {
+        cudaGetLastError();  // (the end of an invalidated capture fails too; the next call must not find that)
+        return st;
+    }
     if (e != cudaSuccess) return fail(e, "loop body capture");
     return DGS_OK;
 }
@@ -201,8 +220,14 @@ dgs_status build_loop(LoopBody body, void* ctx, GraphHolder* hd) {
     const dgs_status st = capture_while(cs.s, body, ctx);
     cudaGraph_t out = nullptr;
     e = cudaStreamEndCapture(cs.s, &out);
-    if (st != DGS_OK) return st;
-    if (e != cudaSuccess) return fail(e, "loop capture");
+    if (st != DGS_OK || e != cudaSuccess) {
+        // the end of a capture that a refused launch has invalidated frees the
+        // graph captured into, here a loop node's body, which destroying the
+        // node's graph would free again (a crash): the graph is left behind
+        hd->g = nullptr;
+        cudaGetLastError();
+        return st != DGS_OK ? st : fail(e, "loop capture");
+    }
     e = cudaGraphInstantiate(&hd->x, hd->g, 0);
     if (e != cudaSuccess) return fail(e, "loop graph instantiation");
     return DGS_OK;
