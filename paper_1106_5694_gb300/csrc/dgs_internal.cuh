@@ -4,6 +4,7 @@
 #pragma once
 
 #include <cstdint>
+#include <mutex>
 #include <cuda_runtime.h>
 
 #include "../../include/dgs.h"
@@ -507,10 +508,14 @@ int32_t device_sms();
 
 // Raise the dynamic shared memory limit of kernel kKernel on the current
 // device to at least `bytes` (each kernel has a record of its own: a limit
-// raised for one says nothing about another's).
+// raised for one says nothing about another's).  Threads may call it at the
+// same time with other sizes: the limit only grows, so the look, the call and
+// the record are one step.
 template <auto kKernel>
 inline cudaError_t ensure_smem_limit(size_t bytes) {
+    static std::mutex mu;
     static int done[64] = {};
+    std::lock_guard<std::mutex> lock(mu);
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
