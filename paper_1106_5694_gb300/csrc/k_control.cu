@@ -98,7 +98,7 @@ __device__ __forceinline__ int32_t block_scan(int32_t x, int32_t* warp_sums, int
 // in global memory; mode 0: everything in global memory.  (The slot of each
 // edge position is read only at a commit and when an edge comes back, and is
 // in global memory.)
-constexpr size_t kCtlStaticSmem = 2048;  // bound on the controller's static shared memory
+constexpr size_t kCtlStaticSmem = 2048;  // bound on the controller's static shared memory (checked at ControllerShared)
 constexpr size_t kCtlSmemLimit = 227 * 1024 - kCtlStaticSmem;
 constexpr int32_t kListCap = 2048;  // accepted (or coloured) positions listed in shared memory
 constexpr int32_t kCand = 128;      // candidates listed at a time by a colouring window
@@ -266,6 +266,22 @@ struct WindowShared {
     uint32_t conf[kCand], word[kCand];  // the listed edges: agents in 15 bits each, applicable (15), comes back (31)
     uint16_t pos[kCand];
 };
+
+// Everything that the controller keeps in static shared memory.
+struct ControllerShared {
+    WindowShared win;
+    unsigned long long pt[kPtCount];  // diagnostics
+    unsigned long long gain, deadline;
+    long long swaps, f;
+    int32_t warp_sums[33];
+    int32_t L, live, stop, acc, app, y, sweeps, event, max_sweeps, trace_cap, events;
+    int32_t window;  // the next sweeps may run as a colouring window
+    uint32_t round, stamp;
+};
+constexpr size_t kSmallLoopShared = 2 * sizeof(int32_t);  // small_loop_kernel's own
+// (the dynamic part begins at the next multiple of 128)
+static_assert((sizeof(ControllerShared) + kSmallLoopShared + 127) / 128 * 128 <= kCtlStaticSmem,
+              "the launches ask for all shared memory but kCtlStaticSmem");
 
 template <int kT>
 __device__ __forceinline__ int32_t colour_window(const Workspace& w, const CtlLayout& lay, uint32_t* Eg, int32_t L,
@@ -489,17 +505,15 @@ __device__ __forceinline__ void controller_body(const Workspace& w, int32_t smem
     DeviceState* st = w.st;
     if (st->status != kRunning) return;
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    __shared__ int32_t warp_sums[33];
-    __shared__ int32_t s_L, s_live, s_stop, s_acc, s_app, s_y, s_sweeps, s_event;
-    __shared__ int32_t s_max_sweeps, s_trace_cap;
-    __shared__ int32_t s_events;
-    __shared__ long long s_swaps;
-    __shared__ int32_t s_window;  // the next sweeps may run as a colouring window
-    __shared__ WindowShared s_win;
-    __shared__ uint32_t s_round;
-    __shared__ uint32_t s_stamp;
-    __shared__ unsigned long long s_gain, s_deadline;
-    __shared__ long long s_f;
+    __shared__ ControllerShared sh;
+    int32_t(&warp_sums)[33] = sh.warp_sums;
+    int32_t &s_L = sh.L, &s_live = sh.live, &s_stop = sh.stop, &s_acc = sh.acc, &s_app = sh.app, &s_y = sh.y;
+    int32_t &s_sweeps = sh.sweeps, &s_event = sh.event, &s_max_sweeps = sh.max_sweeps, &s_trace_cap = sh.trace_cap;
+    int32_t &s_events = sh.events, &s_window = sh.window;
+    WindowShared& s_win = sh.win;
+    uint32_t &s_round = sh.round, &s_stamp = sh.stamp;
+    unsigned long long &s_gain = sh.gain, &s_deadline = sh.deadline;
+    long long &s_swaps = sh.swaps, &s_f = sh.f;
 
     const int32_t n = w.n;
     const int tid = threadIdx.x;
@@ -529,7 +543,7 @@ __device__ __forceinline__ void controller_body(const Workspace& w, int32_t smem
     // diagnostics (DGS_PHASE_TIMERS=1): thread 0 sums into shared memory and
     // adds the sums to global memory once per launch, so that the counters
     // add no global round trips to the loops they time
-    __shared__ unsigned long long s_pt[kPtCount];
+    unsigned long long(&s_pt)[kPtCount] = sh.pt;
     if (pt)
         for (int k = 0; k < kPtCount; ++k) s_pt[k] = 0ull;
 #define DGS_PT(slot, v) \
@@ -1258,6 +1272,7 @@ __global__ void __launch_bounds__(kT, 1) small_loop_kernel(Workspace w, int32_t 
                                                                    uint32_t span, uint32_t stamp_wrap,
                                                                    int32_t compact_min, int32_t colour_pass) {
     __shared__ int32_t s_go, s_count;
+    static_assert(sizeof(s_go) + sizeof(s_count) == kSmallLoopShared, "");
     DeviceState* st = w.st;
     const int32_t n = w.n;
     const int tid = threadIdx.x, warp = tid >> 5;
