@@ -1045,19 +1045,21 @@ __device__ __forceinline__ void prepare_edges_body(const Workspace& w, int32_t b
             gain = in_c ? w.jb_gain[j] : (key ? key_gain(key) : 0);
             target = in_c ? w.jb_agent[j] : (key ? key_index(key) : -1);
         }
-        const uint32_t am = __activemask();
         unsigned long long e = 0ull;
         if (gain > 0) {
             const int32_t u = (t < n) ? t : w.sigma[t - n];
             const int32_t v = (t < n) ? w.sigma[target] : target;
             e = edge_word(u, v) | (exchange_gain(w, u, v) > 0 ? kApplies : 0ull) | (key ? kRevives : 0ull);
         }
-        // the warp's 32 consecutive slots form one chunk
-        const uint32_t bm = __ballot_sync(am, gain > 0);
+        // the warp's 32 consecutive slots form one chunk; in the last one only
+        // those below 2n are here (the branches above split a chunk around n,
+        // so the mask is taken from the slots, not from who happens to be here)
         const int32_t lane = (int32_t)(threadIdx.x & 31u);
+        const int32_t here = 2 * n - (t - lane);
+        const uint32_t bm = __ballot_sync(here >= 32 ? 0xffffffffu : (1u << here) - 1u, gain > 0);
         if (gain > 0)
             w.sl_edge[(t & ~31) + __popc(bm & ((1u << lane) - 1u))] = e | ((unsigned long long)(t & 31) << kPlaceShift);
-        if (lane == __ffs(am) - 1) w.sl_chunk[t >> 5] = __popc(bm);
+        if (lane == 0) w.sl_chunk[t >> 5] = __popc(bm);
     }
 }
 
