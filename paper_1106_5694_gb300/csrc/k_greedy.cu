@@ -683,7 +683,9 @@ __global__ void __launch_bounds__(1024) greedy_rect_fill_kernel(Workspace w, int
 // benefit) and f.
 __global__ void __launch_bounds__(256) greedy_da_start_kernel(Workspace w) {
     DeviceState* st = w.st;
-    if (st->status != kRunning) return;
+    // (uniform for the CTA, whose sum comes at the end: another CTA may report a
+    // job without a holder meanwhile)
+    if (__syncthreads_or(st->status != kRunning)) return;
     if (blockIdx.x == 0 && threadIdx.x == 0) st->greedy_remaining = 0;
     long long f = 0;
     for (int32_t j = blockIdx.x * blockDim.x + threadIdx.x; j < w.n; j += gridDim.x * blockDim.x) {
