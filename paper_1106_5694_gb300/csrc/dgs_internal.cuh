@@ -215,12 +215,18 @@ __host__ __device__ __forceinline__ int32_t batch_blocks_pass1(int32_t n) {
     return b < 1 ? 1 : (b > kBatchPass1MaxBlocks ? kBatchPass1MaxBlocks : b);
 }
 // Units of the evaluation (64 x 64 tile pairs) and of one row task (n / 32
-// columns, and the latency that any row costs).
+// columns, and the latency that any row costs; in batches of more slots units
+// 16 times as large, so that the sum over the instances stays an int32: at most
+// n / 2 rows of each are tasks, and the transposed copies, 4 n^2 bytes each,
+// share the device's memory).
 __host__ __device__ __forceinline__ int32_t eval_tiles(int32_t n) {
     const int32_t nb = (n + 63) / 64;
     return nb * (nb + 1) / 2;
 }
-__host__ __device__ __forceinline__ int32_t row_weight(int32_t n) { return 16 + (n + 31) / 32; }
+constexpr int32_t kFineWeightSlots = 32768;
+__host__ __device__ __forceinline__ int32_t row_weight(int32_t n, int32_t slots) {
+    return slots <= kFineWeightSlots ? 16 + (n + 31) / 32 : 1 + (n + 511) / 512;
+}
 
 // Phases whose work counts the scan kernel computes.
 enum : int32_t { kScanPass1 = 0, kScanGreedyDA = 1, kScanStart = 2, kScanSwitch = 3 };

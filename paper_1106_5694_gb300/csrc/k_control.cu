@@ -1530,7 +1530,7 @@ __global__ void __launch_bounds__(kT) row_tasks_batched_kernel(BatchQueues q) {
         __syncthreads();  // the copy is no longer read
         if (threadIdx.x == 0) w = in.w;
         __syncthreads();
-        const int32_t weight = row_weight(w.n);  // the rows that begin in [lo, hi)
+        const int32_t weight = row_weight(w.n, q.cap);  // the rows that begin in [lo, hi)
         for (int32_t r = (lo + weight - 1) / weight; r * weight < hi; ++r) {
             if (!row_task_row<true>(w, w.rescan_list[r], atrow_s, &bar, phase, red_a, red_j)) {
                 if (threadIdx.x == 0) { w.st->error = kErrWaitTimeout; w.st->status = kError; }
@@ -1576,7 +1576,7 @@ __global__ void __launch_bounds__(1024) scan_batched_kernel(BatchQueues q, int32
                             x0 = eval_tiles(n);
                             st->full_evals += 1;
                         } else {
-                            x1 = count * row_weight(n);
+                            x1 = count * row_weight(n, q.cap);
                             st->row_updates += 1;
                             st->rows_recomputed += count;
                         }
