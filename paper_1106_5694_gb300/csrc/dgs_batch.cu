@@ -350,7 +350,7 @@ class Engine {
 // device, capacity and size class (their tables, pinned staging and step graph
 // took 1.5 ms to set up and tear down, most of a small batch).  An engine
 // belongs to one call at a time, so calls from several threads run on engines
-// of their own; at most kKeep wait here, none of more than kKeepCapacity
+// of their own; at most kKeep wait here, none of more than kKeptEngineSlots
 // slots (about 3 KB each), and dgs_release_cached_memory gives them back.  (Not
 // destroyed at exit, when the CUDA runtime may be gone.)
 class EngineCache {
@@ -378,7 +378,7 @@ class EngineCache {
     }
     void put(const Key& key, Engine* e) {  // the longest waiting one goes
         e->clear();
-        Engine* drop = key.cap > kKeepCapacity ? e : nullptr;
+        Engine* drop = key.cap > kKeptEngineSlots ? e : nullptr;
         if (drop == nullptr) {
             std::lock_guard<std::mutex> lock(mu_);
             free_.emplace_back(key, e);
@@ -400,7 +400,6 @@ class EngineCache {
 
   private:
     static constexpr size_t kKeep = 4;
-    static constexpr int32_t kKeepCapacity = 4096;
     std::mutex mu_;
     std::vector<std::pair<Key, Engine*>> free_;
 };
@@ -412,16 +411,10 @@ struct EngineLease {
     Engine* e = nullptr;
     bool finished = false;
     dgs_status acquire(int32_t count, int32_t max_n) {
-        // classes: 16 slots, then steps of a half or a third; sizes likewise
-        const auto round = [](int32_t x, int32_t from) {
-            int32_t c = from;
-            for (int i = 0; c < x; ++i) c = (i & 1) ? c / 3 * 4 : c / 2 * 3;
-            return c;
-        };
         cudaError_t err = cudaGetDevice(&key.dev);
         if (err != cudaSuccess) return fail(err, "cudaGetDevice");
-        key.cap = round(count, 16);
-        key.max_n = std::min(round(max_n, 256), (int32_t)DGS_BATCH_MAX_N);
+        key.cap = engine_slots(count);
+        key.max_n = std::min(size_class(max_n, 256), (int32_t)DGS_BATCH_MAX_N);
         key.colour = env_colour_pass();
         e = EngineCache::get().take(key);
         if (e != nullptr) return DGS_OK;

@@ -437,6 +437,16 @@ cudaError_t launch_seq_pass_end(const Workspace& w, unsigned long long outer, cu
 cudaError_t launch_slots_from_keys(const Workspace& w, cudaStream_t s);
 cudaError_t launch_sequential(const Workspace& w, cudaStream_t s);
 
+// Slots of a batched call's engine: classes (16, then steps of a half or a
+// third) up to the largest engine that is kept for later calls; beyond it the
+// count itself, since nothing reuses the rest.
+constexpr int32_t kKeptEngineSlots = 4096;
+inline int32_t size_class(int32_t x, int32_t from) {
+    int32_t c = from;
+    for (int i = 0; c < x; ++i) c = (i & 1) ? c / 3 * 4 : c / 2 * 3;
+    return c;
+}
+inline int32_t engine_slots(int32_t count) { return count > kKeptEngineSlots ? count : size_class(count, 16); }
 // Engines kept by finished batched calls, given back (dgs_release_cached_memory).
 void release_cached_engines();
 size_t carve_instance(char* base, int32_t n, bool need_copy, Instance* in);

@@ -35,3 +35,12 @@ def test_queued_row_weights_fit_their_prefix_sums(tmp_path):
         }}
     }}
     return 0;""")
+
+
+def test_engine_slots_cover_the_count_and_waste_nothing_that_is_not_kept(tmp_path):
+    _run(tmp_path, """
+    for (int64_t c = 1; c <= INT32_MAX; c += 1 + c / 64) {
+        const int64_t s = dgs::engine_slots((int32_t)c);
+        if (s < c || (s > 4096 && s != c) || (s <= 4096 && s > 16 && 2 * s > 3 * c)) { printf("%lld: %lld\\n", (long long)c, (long long)s); return 1; }
+    }
+    return dgs::engine_slots(INT32_MAX) == INT32_MAX ? 0 : 1;""")
