@@ -275,9 +275,9 @@ DGS_API dgs_status dgs_get_tuning(int32_t n, int32_t* rows_per_thread, int32_t* 
  * on `count` independent instances of different sizes together: every
  * instance keeps its own loop state on the device, and one persistent launch
  * per kernel works on all instances that are in that kernel's phase
- * (greedy rounds, first evaluation, switching sweeps).  The host replays a
- * captured CUDA graph of one step (a fixed number of greedy rounds and
- * switching iterations) until every instance has finished.  Each result is
+ * (greedy start, first evaluation, switching sweeps).  The host replays a
+ * captured CUDA graph of one step (the starts of new instances and a fixed
+ * number of switching iterations) until every instance has finished.  Each result is
  * bit-identical to dgs_solve_ex on that instance alone with the same options.
  *
  *   benefits[k]    DEVICE pointer to instance k's ns[k] x ns[k] int32 matrix

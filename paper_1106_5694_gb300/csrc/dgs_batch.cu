@@ -47,7 +47,7 @@ constexpr int32_t kSwitchPerStep = 8;   // switching iterations per step
 // n alone) and the most entries one instance can take in each: rows =
 // ceil(n / 512) blocks of 256 threads over agents, jobs or slots; one = the
 // instance itself.  Work that depends on the device state (pass 1 of new
-// instances, greedy rescans, evaluations, row tasks) goes through the queues
+// instances, greedy starts, evaluations, row tasks) goes through the queues
 // of launch_b_scan instead.
 enum : int32_t { kTabRows = 0, kTabOne, kTabCount };
 constexpr int32_t kMaxPerInstance[kTabCount] = {64, 1};
@@ -163,8 +163,8 @@ class Engine {
     // Place an instance in slot k.  mem: carve_instance(nullptr, n, with_copy)
     // bytes of device memory.  Without a copy region the matrix a is used in
     // place; with one, a (if not null) is the caller's unpitched matrix that
-    // the init kernel re-pitches into the region, and a == null means the
-    // region already holds the pitched matrix.
+    // pass 1 re-pitches into the region, and a == null means the region already
+    // holds the pitched matrix.
     void place(int32_t k, char* mem, int32_t n, bool with_copy, const int32_t* a, int32_t* sigma_out,
                int32_t init_mode, int32_t max_sweeps, int64_t deadline_us, const int32_t* user_tau = nullptr,
                bool reeval_all = false) {

@@ -21,7 +21,7 @@ constexpr uint32_t kSpinLimit = 1u << 26;    // bound on every device-side wait 
 enum : int32_t {
     kStageFree = 0,    // slot unused
     kStageNew = 1,     // workspace initialised, pass 1 (transpose, range check) next
-    kStageGreedy = 2,  // locally-dominant greedy rounds
+    kStageGreedy = 2,  // greedy start (deferred acceptance)
     kStageStart = 3,   // sigma, D, f from the start; first full evaluation
     kStageSwitch = 4,  // switching loop (Algorithm 3)
     kStageDone = 5     // finished; assignment written to the instance's output

@@ -1450,8 +1450,7 @@ __global__ void finish_outputs_kernel(Workspace w, int32_t* sigma_out, int64_t* 
 }
 
 // ------------------------------------------------------- batched launches
-// Initialise the fresh instances of the table: clear their small arrays, mark
-// every agent and job free, re-pitch the caller's matrix where needed, and
+// Initialise the fresh instances of the table: clear their small arrays and
 // write the loop state (stage kStageNew).  Entries walk 16-byte chunks.
 __global__ void init_batched_kernel(BatchTable t, int32_t update_policy) {
     const int32_t count = *t.count;
@@ -1460,19 +1459,12 @@ __global__ void init_batched_kernel(BatchTable t, int32_t update_policy) {
         const Instance& in = t.inst[e.inst];
         if (!in.fresh) continue;
         const Workspace& w = in.w;
-        const size_t nb = ((size_t)w.n + 127) / 128 * 128;
-        const char* fa = reinterpret_cast<const char*>(w.free_a);
-        const char* fj = reinterpret_cast<const char*>(w.free_j);
         const size_t chunks = in.zero_bytes / 16;
         const size_t stride = (size_t)e.nblk * blockDim.x;
-        for (size_t q = (size_t)e.bid * blockDim.x + threadIdx.x; q < chunks; q += stride) {
-            char* p = in.zero_begin + 16 * q;
-            const bool ones = (p >= fa && p < fa + nb) || (p >= fj && p < fj + nb);
-            const uint32_t v = ones ? 0x01010101u : 0u;
-            *reinterpret_cast<uint4*>(p) = make_uint4(v, v, v, v);
-        }
-        // a caller's matrix that needs re-pitching (n % 4 != 0 or misaligned) is
-        // copied into the workspace by pass 1, which reads it anyway
+        for (size_t q = (size_t)e.bid * blockDim.x + threadIdx.x; q < chunks; q += stride)
+            *reinterpret_cast<uint4*>(in.zero_begin + 16 * q) = make_uint4(0u, 0u, 0u, 0u);
+        // (a caller's matrix that needs re-pitching, n % 4 != 0 or misaligned, is
+        // copied into the workspace by pass 1, which reads it anyway)
         if (e.bid == 0 && threadIdx.x == 0) {
             DeviceState h{};
             h.status = kRunning;
