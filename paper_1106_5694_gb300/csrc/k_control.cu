@@ -1017,9 +1017,12 @@ __device__ __forceinline__ void prepare_edges_body(const Workspace& w, int32_t b
         w.in_y[j] = 0;
         w.moved[w.sigma[j]] = 0;
     }
-    for (int32_t t = bid * blockDim.x + threadIdx.x; t < 2 * n; t += stride) {
-        unsigned long long key;
-        int32_t gain, target;
+    // (whole warps: 32 consecutive slots form one chunk)
+    const int32_t lane = (int32_t)(threadIdx.x & 31u);
+    for (int32_t t0 = bid * blockDim.x + threadIdx.x - lane; t0 < 2 * n; t0 += stride) {
+        const int32_t t = t0 + lane;
+        unsigned long long key = 0ull;
+        int32_t gain = 0, target = -1;
         bool in_c;
         if (t < n) {
             key = w.key_a[w.tau[t]];
@@ -1032,7 +1035,7 @@ __device__ __forceinline__ void prepare_edges_body(const Workspace& w, int32_t b
             }
             gain = in_c ? w.ag_gain[t] : (key ? key_gain(key) : 0);
             target = in_c ? w.ag_job[t] : (key ? key_index(key) : -1);
-        } else {
+        } else if (t < 2 * n) {
             const int32_t j = t - n;
             key = w.key_j[j];
             in_c = w.in_cj[j];
@@ -1045,21 +1048,15 @@ __device__ __forceinline__ void prepare_edges_body(const Workspace& w, int32_t b
             gain = in_c ? w.jb_gain[j] : (key ? key_gain(key) : 0);
             target = in_c ? w.jb_agent[j] : (key ? key_index(key) : -1);
         }
-        unsigned long long e = 0ull;
+        const uint32_t bm = __ballot_sync(0xffffffffu, gain > 0);
         if (gain > 0) {
             const int32_t u = (t < n) ? t : w.sigma[t - n];
             const int32_t v = (t < n) ? w.sigma[target] : target;
-            e = edge_word(u, v) | (exchange_gain(w, u, v) > 0 ? kApplies : 0ull) | (key ? kRevives : 0ull);
+            const unsigned long long e =
+                edge_word(u, v) | (exchange_gain(w, u, v) > 0 ? kApplies : 0ull) | (key ? kRevives : 0ull);
+            w.sl_edge[t0 + __popc(bm & ((1u << lane) - 1u))] = e | ((unsigned long long)lane << kPlaceShift);
         }
-        // the warp's 32 consecutive slots form one chunk; in the last one only
-        // those below 2n are here (the branches above split a chunk around n,
-        // so the mask is taken from the slots, not from who happens to be here)
-        const int32_t lane = (int32_t)(threadIdx.x & 31u);
-        const int32_t here = 2 * n - (t - lane);
-        const uint32_t bm = __ballot_sync(here >= 32 ? 0xffffffffu : (1u << here) - 1u, gain > 0);
-        if (gain > 0)
-            w.sl_edge[(t & ~31) + __popc(bm & ((1u << lane) - 1u))] = e | ((unsigned long long)(t & 31) << kPlaceShift);
-        if (lane == 0) w.sl_chunk[t >> 5] = __popc(bm);
+        if (lane == 0) w.sl_chunk[t0 >> 5] = __popc(bm);
     }
 }
 
