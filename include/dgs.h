@@ -159,10 +159,11 @@ typedef struct {
     int32_t sweeps;           /* iterations of the switching loop (Alg. 3) */
     int32_t events;           /* sweeps that committed at least one exchange */
     int64_t swaps_applied;    /* committed 2-exchanges */
-    int32_t greedy_rounds;    /* greedy start: the most proposals one agent
-                                 made (deferred acceptance; depends on the
-                                 order in which the GPU ran them), or the
-                                 locally-dominant rounds of the fallback */
+    int32_t greedy_rounds;    /* greedy start: the longest chain of proposals
+                                 and displacements (deferred acceptance;
+                                 depends on the order in which the GPU ran
+                                 them, and a walk over tied jobs counts once),
+                                 or the locally-dominant rounds of the fallback */
     int32_t full_evaluations; /* full difference evaluations (all slots) */
     int32_t row_updates;      /* incremental re-evaluations (row tasks) */
     int64_t rows_recomputed;  /* rows re-evaluated by those row tasks */

@@ -14,6 +14,7 @@
 // Pass 1 reads a once in 64x64 tiles and, in the same pass, writes the
 // transposed copy at, checks |a| < 2^29 and computes what the greedy start
 // that follows needs: each agent's best benefit in every tile of jobs.
+#include <algorithm>
 #include <cstdlib>
 
 #include "dgs_internal.cuh"
@@ -274,6 +275,9 @@ constexpr int kDaThreads = 256;
 constexpr int kDaPerSm = 4;
 constexpr int kDaGroup = 4;  // warps that follow one chain
 constexpr int kDaPicks = 4;  // 64-job tiles that one look of a warp reads
+constexpr int32_t kDaTies = 64;       // proposals of one walk over tied jobs (da_walk_ties)
+constexpr int32_t kDaTieWait = 64;    // displacements until the next walk, after one that found nothing;
+constexpr int32_t kDaTieFailed = 4;   // a failed proposal counts as so many
 constexpr int kDaWarps = kDaThreads / 32;
 constexpr uint64_t kDaTimeoutNs = 16000000000ull;  // bound on one warp's work (internal error beyond)
 
@@ -436,15 +440,73 @@ __device__ __forceinline__ unsigned long long da_look_wide(const DaView& d, cons
     return r >= d.floor ? ((unsigned long long)r << 32) | ~rc : 0ull;
 }
 
+// Tied values.  A proposal to job c has just displaced that job's holder
+// (`old`, below the proposer's key `mine`) or failed against it: the turn is the
+// displaced agent's, or the proposer's again.  c was the best job of whose turn
+// it is, at some benefit v, so it has lost every job that it ranks above c, and
+// now c.  Its next job of benefit v after c is therefore its best one, once
+// every job between has been looked at.  The walk does just that: 128 jobs from
+// c's group of 64 on (one load of the row and two of the keys per lane), the
+// proposal, and on with whose turn it then is, until a job was free, none of
+// the 128 will do, or kDaTies proposals are made (so that the caller's bound on
+// time is looked at).
+//
+// It is tried after every displacement and failure for as long as walks find
+// something, and again kDaTieWait displacements after one that did not (earlier
+// when proposals fail).  Without it every turn was a look of the whole group, and
+// where many agents want the same jobs for few different values that is one look
+// per agent and job: constant n = 4096 23 ms, now 11.2, n = 20000 89 -> 35; values
+// in [0, 2) n = 4096 7.3 -> 3.1; in [0, 4) 3.2 -> 1.36, n = 20000 13 -> 4.8.  Without
+// ties it costs at most 1 us (peer-shaped n = 4096 117.6 -> 118.3 us, 10000 263.7
+// -> 264.4): a walk that finds nothing takes as long, and tried after every
+// failure it cost 2 to 3.  It does not help identical agents whose jobs differ in
+// value: there every turn is still a look.
+struct DaWalk {
+    int32_t out;   // as da_propose returns it (-3: agent i's turn)
+    int32_t tied;  // its next `tied`
+};
+__device__ __noinline__ DaWalk da_walk_ties(const int32_t* a, unsigned long long* keys, int32_t n, int32_t lda,
+                                            int32_t i, int32_t c, unsigned long long mine, unsigned long long old) {
+    constexpr uint32_t kAll = 0xffffffffu, kNone = 0x7fffffffu;
+    const int lane = threadIdx.x & 31;
+    int32_t who = i;
+    for (int32_t q = 0; old != 0ull; ++q) {
+        if (old < mine) {  // displaced: its turn
+            who = key_index(old);
+            mine = old;
+        }
+        uint32_t next = kNone;
+        const int32_t c4 = (c & ~(kT - 1)) + lane * 4;
+        if (q < kDaTies && c4 < n && c4 + 3 > c) {
+            const int32_t v = (int32_t)(mine >> 32) - kBenefitLimit;
+            const int4 x = __ldg(reinterpret_cast<const int4*>(a + (size_t)who * lda + c4));
+            const ulonglong2 h0 = __ldcg(reinterpret_cast<const ulonglong2*>(keys + c4));
+            const ulonglong2 h1 = __ldcg(reinterpret_cast<const ulonglong2*>(keys + c4 + 2));
+            if (x.w == v && mine > h1.y && c4 + 3 < n) next = (uint32_t)c4 + 3u;
+            if (x.z == v && mine > h1.x && c4 + 2 < n && c4 + 2 > c) next = (uint32_t)c4 + 2u;
+            if (x.y == v && mine > h0.y && c4 + 1 < n && c4 + 1 > c) next = (uint32_t)c4 + 1u;
+            if (x.x == v && mine > h0.x && c4 > c) next = (uint32_t)c4;
+        }
+        next = __reduce_min_sync(kAll, next);
+        if (next == kNone) return DaWalk{who == i ? -3 : who, q > 0 ? 0 : -kDaTieWait};
+        c = (int32_t)next;
+        if (lane == 0) old = atomic_max_acq_rel(keys + c, mine);
+        old = __shfl_sync(kAll, old, 0);
+    }
+    return DaWalk{-1, 0};
+}
+
 // One proposal of agent i (and its retries after failed ones) by a group of
 // kGroup warps.  Tile t belongs to lane (t / kGroup) % 32 of warp t % kGroup.
 // s_b: the group's copy of the agent's bounds (each thread reads and writes
-// only its own tiles' entries).  Returns the displaced agent, -1 when the job
-// was free, -4 when no job of benefit d.floor takes the agent (that is an
-// error when every job counts, d.floor = 1), -2 on an error.
+// only its own tiles' entries).  tied (the group's first warp's): below 0 the
+// displacements to come until a walk over tied jobs is tried.  Returns the agent
+// whose turn is next (it was displaced), -1 when the job was free, -4 when no job
+// of benefit d.floor takes the agent (that is an error when every job counts,
+// d.floor = 1), -2 on an error.
 template <int kGroup>
 __device__ __forceinline__ int32_t da_propose(const DaView& d, int32_t i, uint32_t* s_b, DaShared<kGroup>& sh, int grp,
-                                              int gw, int32_t& looks) {
+                                              int gw, int32_t& looks, int32_t& tied) {
     constexpr uint32_t kAll = 0xffffffffu;
     constexpr int32_t kNone = 0x7fffffff;
     const int lane = threadIdx.x & 31;
@@ -524,6 +586,11 @@ __device__ __forceinline__ int32_t da_propose(const DaView& d, int32_t i, uint32
             if (lane == 0) old = atomic_max_acq_rel(d.keys + bc, mine);
             old = __shfl_sync(kAll, old, 0);
             out = old < mine ? (old == 0ull ? -1 : key_index(old)) : -3;  // -3: taken meanwhile, look again
+            if (out != -1 && (tied += out == -3 ? kDaTieFailed : 1) >= 0) {
+                const DaWalk r = da_walk_ties(d.a, d.keys, d.n, d.lda, i, bc, mine, old);
+                out = r.out;
+                tied = r.tied;
+            }
         }
         if (kGroup > 1) {
             if (gw == 0 && lane == 0) sh.out = out;
@@ -562,14 +629,14 @@ __global__ void __launch_bounds__(kDaThreads, kDaPerSm) greedy_da_kernel(Workspa
     const bool leader = gw == 0 && lane == 0;
     uint32_t* s_b = s_bounds + (size_t)grp * d.tiles;
     const int32_t groups = (int32_t)gridDim.x * kGroups;
-    int32_t looks = 0, longest = 0;
+    int32_t looks = 0, longest = 0, tied = -kDaTieWait;
     const uint64_t t_start = globaltimer_ns();
     // (neighbouring agents on different SMs)
     int32_t next = grp * (int32_t)gridDim.x + (int32_t)blockIdx.x;
     while (next < count) {
         int32_t a = ph.list ? ph.list[next] : next, r, steps = 1;
         // the chain of displacements that starts with agent a
-        while ((r = da_propose<kGroup>(d, a, s_b, s_sh[grp], grp, gw, looks)) >= 0) {
+        while ((r = da_propose<kGroup>(d, a, s_b, s_sh[grp], grp, gw, looks, tied)) >= 0) {
             a = r;
             ++steps;
             if ((steps & 63) == 0) {  // bounded in time
@@ -600,7 +667,7 @@ __global__ void __launch_bounds__(kDaThreads, kDaPerSm) greedy_da_kernel(Workspa
     }
     if (lane == 0 && looks) {
         atomicAdd((unsigned long long*)&st->greedy_rescans, (unsigned long long)looks);
-        atomicMax(&st->greedy_rounds, longest);  // proposals along the longest chain
+        atomicMax(&st->greedy_rounds, longest);  // turns along the longest chain (a walk over ties is one)
     }
     if (leader && w.phase_ns) {  // diagnostics (DGS_PHASE_TIMERS=1)
         const uint64_t t = globaltimer_ns() - t_start;
@@ -784,7 +851,7 @@ __global__ void __launch_bounds__(kDaThreads, kDaPerSm) greedy_da_batched_kernel
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint32_t* s_b = s_bounds[warp];
     const int32_t warps = (int32_t)gridDim.x * kDaWarps;
-    int32_t looks = 0, longest = 0, k_last = -1, first = 0, end = 0;
+    int32_t looks = 0, longest = 0, tied = -kDaTieWait, k_last = -1, first = 0, end = 0;
     DaView d{};
     auto flush = [&] {  // looks and chains are counted per instance
         if (k_last >= 0 && lane == 0 && looks) {
@@ -807,7 +874,7 @@ __global__ void __launch_bounds__(kDaThreads, kDaPerSm) greedy_da_batched_kernel
                 d = da_view(q.inst[k_last].w, q.inst[k_last].w.n, 1u);
             }
             int32_t a = g - first, r, steps = 1;
-            while ((r = da_propose<1>(d, a, s_b, s_sh[warp], warp, 0, looks)) >= 0) {
+            while ((r = da_propose<1>(d, a, s_b, s_sh[warp], warp, 0, looks, tied)) >= 0) {
                 a = r;
                 ++steps;
             }
@@ -936,14 +1003,23 @@ int32_t greedy_rounds_env() {
     return (e && std::atoi(e) == 1) ? 1 : 0;
 }
 
+// Chains that are followed at the same time: all of them up to n = 512, then
+// at least 512 and half of the agents, at most what fits.  Where agents want the
+// same jobs every chain in flight runs into the others (constant matrices, n =
+// 1021 1.94 ms, 2.45 with a chain per agent; n = 1532 3.9, 4.8; n = 2100 6.4, 7.1;
+// a third of the agents 1.95, 3.1, 5.1); elsewhere more chains gain little
+// (peer-shaped n = 1021 66.2 us, 66.9; n = 1532 76.1, 75.1; n = 2100 92.3, 91.5; a
+// third 66.5, 77.6, 93.6, and uniform values in [0, 1e6), n = 1532, 38.4, 37.6 and
+// 40.5).
+int32_t da_chains(int32_t n) { return std::min(n, std::max(512, (n + 1) / 2)); }
+
 cudaError_t launch_greedy_da(const Workspace& w, int32_t real_n, int32_t real_m, cudaStream_t s) {
     if (greedy_rounds_env() || w.g_bound == nullptr) return cudaErrorNotSupported;
     constexpr int kGroups = kDaWarps / kDaGroup;
     const size_t smem = sizeof(uint32_t) * kGroups * (size_t)w.bound_tiles;
     cudaError_t e = ensure_smem_limit<greedy_da_kernel<kDaGroup>>(smem);
     if (e != cudaSuccess) return e;
-    const int32_t most = (w.n + kGroups - 1) / kGroups;
-    const int32_t grid = most < da_grid(smem) ? most : da_grid(smem);
+    const int32_t grid = std::min(da_grid(smem), (da_chains(w.n) + kGroups - 1) / kGroups);
     if (real_n == w.n && real_m == w.n) {
         greedy_da_kernel<kDaGroup><<<grid, kDaThreads, smem, s>>>(w, DaPhase{nullptr, w.n, w.n, 1u, nullptr});
     } else {
