@@ -424,7 +424,7 @@ cudaError_t launch_finish(const Workspace& w, int32_t* sigma_out, cudaStream_t s
 // (device-writable pointers; launches: kernels launched from the host).
 cudaError_t launch_finish_outputs(const Workspace& w, int32_t* sigma_out, int64_t* objective, int32_t* status,
                                   dgs_stats* stats, int64_t launches, int32_t sequential, cudaStream_t s);
-// Loop conditions of the device-side loops (see enqueue_while): the greedy
+// Loop conditions of the device-side loops (see enqueue_while_cached): the greedy
 // rounds' loop (while agents are unmatched), and Algorithm 1's switching loop
 // and passes.
 cudaError_t launch_greedy_loop_cond(const Workspace& w, unsigned long long handle, cudaStream_t s);
@@ -486,18 +486,16 @@ cudaError_t launch_b_advance(const BatchTable& one, int32_t from_stage, cudaStre
 // loop; `body` enqueues the loop body on the capture stream it is given and
 // passes `handle` to the kernel that decides, at the end of each iteration,
 // whether the loop goes on (cudaGraphSetConditional; the condition is 1 when
-// the body first runs).  The graph is released as soon as it is launched (an
-// executable graph in flight is freed when it completes): the call only
-// enqueues work.  `nested` bodies may themselves call capture_while on their
-// capture stream to add an inner loop; such a loop's condition is set to 1
-// at the start of the graph's launch only, so a body that runs an inner loop
-// re-arms it itself: it creates the inner handle first (create_loop_handle on
-// its capture stream), sets it from a kernel, and passes it to capture_while.
+// the body first runs).  The call only enqueues work.  An executable graph
+// captured earlier on this device with the same body and the same `key` bytes
+// (which must cover every value the body's launches are captured with) is used
+// again; up to 16 are kept (one dropped in flight is freed when it completes).
+// Nested bodies may themselves call capture_while on their capture stream to
+// add an inner loop; such a loop's condition is set to 1 at the start of the
+// graph's launch only, so a body that runs an inner loop re-arms it itself: it
+// creates the inner handle first (create_loop_handle on its capture stream),
+// sets it from a kernel, and passes it to capture_while.
 using LoopBody = dgs_status (*)(void* ctx, cudaStream_t capture, unsigned long long handle);
-dgs_status enqueue_while(cudaStream_t s, LoopBody body, void* ctx);
-// The same, reusing an executable graph captured earlier on this device with
-// the same body and the same `key` bytes (which must cover every value the
-// body's launches are captured with); up to 16 are kept.
 dgs_status enqueue_while_cached(cudaStream_t s, LoopBody body, void* ctx, const void* key, size_t key_bytes);
 dgs_status create_loop_handle(cudaStream_t capturing, unsigned long long* handle);
 // Inside a capture: what a and b enqueue (each on the capture stream) both

@@ -280,27 +280,6 @@ dgs_status enqueue_while_cached(cudaStream_t s, LoopBody body, void* ctx, const 
     return DGS_OK;
 }
 
-dgs_status enqueue_while(cudaStream_t s, LoopBody body, void* ctx) {
-    GraphHolder hd;
-    cudaError_t e = cudaGraphCreate(&hd.g, 0);
-    if (e != cudaSuccess) return fail(e, "graph");
-    CaptureStream cs;
-    e = cs.acquire();
-    if (e != cudaSuccess) return fail(e, "capture stream");
-    e = cudaStreamBeginCaptureToGraph(cs.s, hd.g, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed);
-    if (e != cudaSuccess) return fail(e, "loop capture");
-    const dgs_status st = capture_while(cs.s, body, ctx);
-    cudaGraph_t out = nullptr;
-    e = cudaStreamEndCapture(cs.s, &out);
-    if (st != DGS_OK) return st;
-    if (e != cudaSuccess) return fail(e, "loop capture");
-    e = cudaGraphInstantiate(&hd.x, hd.g, 0);
-    if (e != cudaSuccess) return fail(e, "loop graph instantiation");
-    e = cudaGraphLaunch(hd.x, s);
-    if (e != cudaSuccess) return fail(e, "loop graph launch");
-    return DGS_OK;
-}
-
 void* pinned_get(size_t bytes) {
     const size_t c = pin_class(bytes);
     {

@@ -144,22 +144,21 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-// sigma of the rows this thread copies for tile (J, K): X rows J0 + rq + c *
-// kRowStep and Y rows K0 + rq + c * kRowStep (rq = threadIdx.x / 16).
+// sigma of the rows that this thread copies to Y for column tile K: rows K0 +
+// rq + c * kRowStep (rq = threadIdx.x / 16).
 template <int kRows>
 struct CopyRows {
-    int32_t x[Geo<kRows>::kCopies], y[Geo<kRows>::kCopies];
+    int32_t y[Geo<kRows>::kCopies];
 };
 
-template <int kRows, bool kTma = false>
-__device__ __forceinline__ CopyRows<kRows> copy_rows(const Workspace& w, int32_t J, int32_t K) {
+template <int kRows>
+__device__ __forceinline__ CopyRows<kRows> copy_rows(const Workspace& w, int32_t K) {
     const int32_t rq = threadIdx.x >> 4;
     const int32_t K0 = K * kT, n = w.n;
     CopyRows<kRows> c;
 #pragma unroll
     for (int q = 0; q < Geo<kRows>::kCopies; ++q) {
         const int32_t r = rq + q * Geo<kRows>::kRowStep;
-        c.x[q] = -1;  // X rows come from the producer's per-run sources (or TMA)
         c.y[q] = (K0 + r < n) ? w.sigma[K0 + r] : -1;
     }
     return c;
@@ -169,7 +168,7 @@ template <int kRows>
 __device__ __forceinline__ CopyRows<kRows> no_rows() {
     CopyRows<kRows> c;
 #pragma unroll
-    for (int q = 0; q < Geo<kRows>::kCopies; ++q) c.x[q] = c.y[q] = -1;
+    for (int q = 0; q < Geo<kRows>::kCopies; ++q) c.y[q] = -1;
     return c;
 }
 
@@ -529,7 +528,7 @@ __device__ __forceinline__ void evaluation_loop(const Workspace& w, const Schedu
                 x_sources<kRows>(w, prod.j, xr);
                 xr_j = prod.j;
             }
-            issue_tile<kRows>(w, &stages[s], prod.j, prod.k, copy_rows<kRows, kTma>(w, prod.j, prod.k),
+            issue_tile<kRows>(w, &stages[s], prod.j, prod.k, copy_rows<kRows>(w, prod.k),
                               kTma ? nullptr : &xr);
             if (kTma && threadIdx.x < 32) {
                 if (prod.j != xs_j) {
@@ -544,8 +543,8 @@ __device__ __forceinline__ void evaluation_loop(const Workspace& w, const Schedu
     }
     TileCursor ahead = prod;  // one tile after prod
     bool ahead_ok = prod_ok && cursor_next(ahead, nb, sc);
-    CopyRows<kRows> rows_now = prod_ok ? copy_rows<kRows, kTma>(w, prod.j, prod.k) : no_rows<kRows>();
-    CopyRows<kRows> rows_next = ahead_ok ? copy_rows<kRows, kTma>(w, ahead.j, ahead.k) : no_rows<kRows>();
+    CopyRows<kRows> rows_now = prod_ok ? copy_rows<kRows>(w, prod.k) : no_rows<kRows>();
+    CopyRows<kRows> rows_next = ahead_ok ? copy_rows<kRows>(w, ahead.k) : no_rows<kRows>();
 
     TileCursor cons;
     bool cons_ok = cursor_first(cons, nb, sc);
@@ -600,7 +599,7 @@ __device__ __forceinline__ void evaluation_loop(const Workspace& w, const Schedu
             rows_now = rows_next;
             if (ahead_ok) {
                 ahead_ok = cursor_next(ahead, nb, sc);
-                if (ahead_ok) rows_next = copy_rows<kRows, kTma>(w, ahead.j, ahead.k);
+                if (ahead_ok) rows_next = copy_rows<kRows>(w, ahead.k);
             }
         }
         cp_async_commit();
